@@ -1,8 +1,12 @@
-"""ctypes binding of the C-ABI CUDA library (``libmixdq.so``).
+"""Binding of the C-ABI CUDA library (``libmixdq.so``).
 
 Argument marshalling only: torch tensors supply device memory and the current stream,
 every step of the path runs in the library's kernels.  There is no CPU fallback: if the
 shared library is missing the first call raises.
+
+The layer calls and the tensor helpers that a program runs per step (``NATIVE``) are functions of the extension module
+``_mixdq_native`` (``csrc/bind.cpp``), loaded at the first use of one of them; their signatures stand in their
+docstrings.  Sizes, plans and the parity hooks go through ctypes.
 """
 from __future__ import annotations
 
@@ -80,6 +84,14 @@ _SIGNATURES = {
 
 EXPORTS = tuple(_SIGNATURES)
 
+# Functions of the extension module, defined here at their first use.
+NATIVE = (
+    "weight_minmax_params", "pack_weights", "weight_code_sums", "act_absmax", "act_scale_from_absmax", "act_scale",
+    "act_minmax", "act_asym_params", "linear", "linear_a8_asym", "quantize_acts", "linear_q8", "linear_a8_fused_quant",
+    "linear_a8_static_scratch", "linear_a8_split", "crossattn_kv", "conv3x3", "conv3x3_a8_asym", "conv3x3_q8",
+    "conv3x3_a8_split", "conv1x1",
+)
+
 _lib = None
 
 
@@ -100,6 +112,20 @@ def lib():
             fn.argtypes = args
         _lib = L
     return _lib
+
+
+def __getattr__(name: str):
+    if name not in NATIVE:
+        raise AttributeError(f"module {__name__!r} has no attribute {name!r}")
+    lib()  # the extension links against it: the same copy serves both
+    try:
+        from . import _mixdq_native as native
+    except ImportError as e:
+        raise MixdqError(f"_mixdq_native is missing or does not load ({e}): build it with "
+                         "python -m paper_2405_17873_b200.build") from e
+    native._set_error_class(MixdqError)
+    globals().update((n, getattr(native, n)) for n in NATIVE)
+    return globals()[name]
 
 
 def _chk(rc: int, what: str):
@@ -168,26 +194,6 @@ def new_workspace(nbytes: int, device="cuda") -> Optional[torch.Tensor]:
     return torch.zeros(nbytes, dtype=torch.uint8, device=device)
 
 
-def weight_minmax_params(W: torch.Tensor, bits: int, symmetric: bool, scale_out: Optional[torch.Tensor] = None,
-                         zero_out: Optional[torch.Tensor] = None):
-    N, K = W.shape
-    scale = scale_out if scale_out is not None else torch.empty(N, dtype=torch.float32, device=W.device)
-    zero = zero_out if zero_out is not None else torch.zeros(N, dtype=torch.int32, device=W.device)
-    _chk(lib().mixdq_weight_minmax_params(_ptr(W), N, K, bits, int(symmetric), _ptr(scale), _ptr(zero),
-                                          _stream()), "mixdq_weight_minmax_params")
-    return scale, zero
-
-
-def pack_weights(W: torch.Tensor, bits: int, scale: torch.Tensor, zero: Optional[torch.Tensor] = None,
-                 layout: int = LAYOUT_DEVICE, out: Optional[torch.Tensor] = None) -> torch.Tensor:
-    N, K = W.shape
-    if out is None:
-        out = torch.zeros(packed_bytes(N, K, bits, layout), dtype=torch.uint8, device=W.device)
-    _chk(lib().mixdq_pack_weights(_ptr(W), N, K, bits, _ptr(scale), _ptr(zero), layout, _ptr(out), _stream()),
-         "mixdq_pack_weights")
-    return out
-
-
 def unpack_weights(packed: torch.Tensor, N: int, K: int, bits: int, is_signed: bool,
                    layout: int = LAYOUT_DEVICE) -> torch.Tensor:
     codes = torch.empty((N, K), dtype=torch.int16, device=packed.device)
@@ -196,63 +202,8 @@ def unpack_weights(packed: torch.Tensor, N: int, K: int, bits: int, is_signed: b
     return codes
 
 
-def act_absmax(X: torch.Tensor, skip_rows_mod: int = 0) -> torch.Tensor:
-    X2 = X.reshape(-1, X.shape[-1])
-    out = torch.empty(1, dtype=torch.float32, device=X.device)
-    _chk(lib().mixdq_act_absmax(_ptr(X2), X2.shape[0], X2.shape[1], X2.shape[1], skip_rows_mod, _ptr(out),
-                                _stream()), "mixdq_act_absmax")
-    return out
-
-
-def act_scale_from_absmax(amax: torch.Tensor) -> torch.Tensor:
-    out = torch.empty(1, dtype=torch.float32, device=amax.device)
-    _chk(lib().mixdq_act_scale_from_absmax(_ptr(amax), _ptr(out), _stream()), "mixdq_act_scale_from_absmax")
-    return out
-
-
-def act_scale(X: torch.Tensor, skip_rows_mod: int = 0) -> torch.Tensor:
-    """Dynamic per-tensor int8 scale max|X| / 127, computed on the device."""
-    return act_scale_from_absmax(act_absmax(X, skip_rows_mod))
-
-
-def act_minmax(X: torch.Tensor) -> torch.Tensor:
-    """Device fp32 [2]: min(min x, 0), max(max x, 0)."""
-    X2 = X.reshape(-1, X.shape[-1])
-    out = torch.empty(2, dtype=torch.float32, device=X.device)
-    _chk(lib().mixdq_act_minmax(_ptr(X2), X2.shape[0], X2.shape[1], X2.stride(0), _ptr(out), _stream()),
-         "mixdq_act_minmax")
-    return out
-
-
-def act_asym_params(X: torch.Tensor):
-    """Asymmetric 8-bit activation parameters (device fp32 scale [1], device int32 zero-point [1])."""
-    mm = act_minmax(X)
-    scale = torch.empty(1, dtype=torch.float32, device=X.device)
-    zero = torch.empty(1, dtype=torch.int32, device=X.device)
-    _chk(lib().mixdq_act_asym_params_from_minmax(_ptr(mm), _ptr(scale), _ptr(zero), _stream()),
-         "mixdq_act_asym_params_from_minmax")
-    return scale, zero
-
-
-def weight_code_sums(packed_W: torch.Tensor, N: int, K: int, bits: int) -> torch.Tensor:
-    out = torch.empty(N, dtype=torch.int32, device=packed_W.device)
-    _chk(lib().mixdq_weight_code_sums(_ptr(packed_W), N, K, bits, _ptr(out), _stream()), "mixdq_weight_code_sums")
-    return out
-
-
 def _ws(workspace):
     return (_ptr(workspace), workspace.numel() if workspace is not None else 0)
-
-
-def linear(X, packed_W, N: int, w_bits: int, w_scale, w_zero=None, act_bits: int = 8, act_scale=None,
-           bias=None, workspace=None, status=None, out=None):
-    M, K = X.shape
-    Y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=X.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_linear(_ptr(X), M, K, X.stride(0), _ptr(packed_W), N, w_bits, _ptr(w_scale), _ptr(w_zero),
-                            act_bits, _ptr(act_scale), _ptr(bias), _ptr(Y), wp, wb, _ptr(status), _stream()),
-         "mixdq_linear")
-    return Y
 
 
 def linear_acc_i32(X, packed_W, N: int, w_bits: int, act_scale, workspace=None, status=None):
@@ -262,17 +213,6 @@ def linear_acc_i32(X, packed_W, N: int, w_bits: int, act_scale, workspace=None, 
     _chk(lib().mixdq_linear_acc_i32(_ptr(X), M, K, X.stride(0), _ptr(packed_W), N, w_bits, _ptr(act_scale),
                                     _ptr(acc), wp, wb, _ptr(status), _stream()), "mixdq_linear_acc_i32")
     return acc
-
-
-def linear_a8_asym(X, packed_W, N: int, w_bits: int, w_scale, w_code_sums, act_scale, act_zero, bias=None,
-                   workspace=None, status=None, out=None):
-    M, K = X.shape
-    Y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=X.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_linear_a8_asym(_ptr(X), M, K, X.stride(0), _ptr(packed_W), N, w_bits, _ptr(w_scale),
-                                    _ptr(w_code_sums), _ptr(act_scale), _ptr(act_zero), _ptr(bias), _ptr(Y),
-                                    wp, wb, _ptr(status), _stream()), "mixdq_linear_a8_asym")
-    return Y
 
 
 def linear_a8_asym_acc_i32(X, packed_W, N: int, w_bits: int, w_code_sums, act_scale, act_zero, workspace=None,
@@ -290,30 +230,6 @@ def _out_hw(H, W, stride):
     return (H - 1) // stride + 1, (W - 1) // stride + 1
 
 
-def conv3x3(X, packed_W, Cout: int, w_bits: int, w_scale, w_zero=None, act_bits: int = 8, act_scale=None,
-            bias=None, stride: int = 1, workspace=None, status=None, out=None):
-    B, H, W, Cin = X.shape
-    Ho, Wo = _out_hw(H, W, stride)
-    Y = out if out is not None else torch.empty((B, Ho, Wo, Cout), dtype=torch.float16, device=X.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_conv3x3(_ptr(X), B, H, W, Cin, _ptr(packed_W), Cout, stride, w_bits, _ptr(w_scale),
-                             _ptr(w_zero), act_bits, _ptr(act_scale), _ptr(bias), _ptr(Y), wp, wb,
-                             _ptr(status), _stream()), "mixdq_conv3x3")
-    return Y
-
-
-def conv3x3_a8_asym(X, packed_W, Cout: int, w_bits: int, w_scale, w_code_sums, act_scale, act_zero, bias=None,
-                    stride: int = 1, workspace=None, status=None, out=None):
-    B, H, W, Cin = X.shape
-    Ho, Wo = _out_hw(H, W, stride)
-    Y = out if out is not None else torch.empty((B, Ho, Wo, Cout), dtype=torch.float16, device=X.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_conv3x3_a8_asym(_ptr(X), B, H, W, Cin, _ptr(packed_W), Cout, stride, w_bits, _ptr(w_scale),
-                                     _ptr(w_code_sums), _ptr(act_scale), _ptr(act_zero), _ptr(bias), _ptr(Y),
-                                     wp, wb, _ptr(status), _stream()), "mixdq_conv3x3_a8_asym")
-    return Y
-
-
 def conv3x3_a8_asym_acc_i32(X, packed_W, Cout: int, w_bits: int, w_code_sums, act_scale, act_zero,
                             stride: int = 1, workspace=None, status=None):
     B, H, W, Cin = X.shape
@@ -324,45 +240,6 @@ def conv3x3_a8_asym_acc_i32(X, packed_W, Cout: int, w_bits: int, w_code_sums, ac
                                              _ptr(w_code_sums), _ptr(act_scale), _ptr(act_zero), _ptr(acc), wp,
                                              wb, _ptr(status), _stream()), "mixdq_conv3x3_a8_asym_acc_i32")
     return acc
-
-
-def quantize_acts(X, act_scale, out=None):
-    """int8 codes [rows, K] of X fp16 [rows, K] with the per-tensor scale *act_scale (device)."""
-    rows, K = X.shape
-    Xq = out if out is not None else torch.empty((rows, K), dtype=torch.int8, device=X.device)
-    assert X.stride(1) == 1
-    _chk(lib().mixdq_quantize_acts(C.c_void_p(X.data_ptr()), rows, K, X.stride(0), _ptr(act_scale), _ptr(Xq),
-                                   _stream()), "mixdq_quantize_acts")
-    return Xq
-
-
-def linear_q8(Xq, packed_W, N: int, w_bits: int, w_scale, act_scale, bias=None, status=None, out=None):
-    M, K = Xq.shape
-    Y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=Xq.device)
-    _chk(lib().mixdq_linear_q8(_ptr(Xq), M, K, _ptr(packed_W), N, w_bits, _ptr(w_scale), _ptr(act_scale),
-                               _ptr(bias), _ptr(Y), _ptr(status), _stream()), "mixdq_linear_q8")
-    return Y
-
-
-def linear_a8_fused_quant(X, packed_W, N: int, w_bits: int, w_scale, act_scale, bias=None, tile_cols: int = 128,
-                          status=None, out=None):
-    """mixdq_linear (8-bit activations) as one kernel on 128 x tile_cols tiles, whatever the planner would choose."""
-    M, K = X.shape
-    Y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=X.device)
-    _chk(lib().mixdq_linear_a8_fused_quant(_ptr(X), M, K, X.stride(0), _ptr(packed_W), N, w_bits, _ptr(w_scale),
-                                           _ptr(act_scale), _ptr(bias), _ptr(Y), Y.stride(0), tile_cols, _ptr(status),
-                                           _stream()), "mixdq_linear_a8_fused_quant")
-    return Y
-
-
-def conv3x3_q8(Xq, packed_W, Cout: int, w_bits: int, w_scale, act_scale, bias=None, stride: int = 1, status=None,
-               out=None):
-    B, H, W, Cin = Xq.shape
-    Ho, Wo = (H - 1) // stride + 1, (W - 1) // stride + 1
-    Y = out if out is not None else torch.empty((B, Ho, Wo, Cout), dtype=torch.float16, device=Xq.device)
-    _chk(lib().mixdq_conv3x3_q8(_ptr(Xq), B, H, W, Cin, _ptr(packed_W), Cout, stride, w_bits, _ptr(w_scale),
-                                _ptr(act_scale), _ptr(bias), _ptr(Y), _ptr(status), _stream()), "mixdq_conv3x3_q8")
-    return Y
 
 
 def selftest_abandoned_wait(Xq, packed_W, N: int, w_bits: int, w_scale, act_scale, drop_k_block: int, status):
@@ -390,17 +267,6 @@ def split_workspace_bytes(in_rows: int, row_len: int, split_at: int, out_rows: i
     return out.value
 
 
-def linear_a8_split(X, split_at: int, packed_W_lo, packed_W_hi, N: int, w_bits: int, w_scale, act_scale_lo,
-                    act_scale_hi, bias=None, workspace=None, status=None, out=None):
-    M, K = X.shape
-    Y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=X.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_linear_a8_split(_ptr(X), M, K, X.stride(0), split_at, _ptr(packed_W_lo), _ptr(packed_W_hi), N,
-                                     w_bits, _ptr(w_scale), _ptr(act_scale_lo), _ptr(act_scale_hi), _ptr(bias),
-                                     _ptr(Y), wp, wb, _ptr(status), _stream()), "mixdq_linear_a8_split")
-    return Y
-
-
 def linear_a8_split_acc_i32(X, split_at: int, packed_W_lo, packed_W_hi, N: int, w_bits: int, act_scale_lo,
                             act_scale_hi, workspace=None, status=None):
     M, K = X.shape
@@ -412,19 +278,6 @@ def linear_a8_split_acc_i32(X, split_at: int, packed_W_lo, packed_W_hi, N: int, 
                                              _ptr(lo), _ptr(hi), wp, wb, _ptr(status), _stream()),
          "mixdq_linear_a8_split_acc_i32")
     return lo, hi
-
-
-def conv3x3_a8_split(X, split_at: int, packed_W_lo, packed_W_hi, Cout: int, w_bits: int, w_scale, act_scale_lo,
-                     act_scale_hi, bias=None, stride: int = 1, workspace=None, status=None, out=None):
-    B, H, W, Cin = X.shape
-    Ho, Wo = _out_hw(H, W, stride)
-    Y = out if out is not None else torch.empty((B, Ho, Wo, Cout), dtype=torch.float16, device=X.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_conv3x3_a8_split(_ptr(X), B, H, W, Cin, split_at, _ptr(packed_W_lo), _ptr(packed_W_hi), Cout,
-                                      stride, w_bits, _ptr(w_scale), _ptr(act_scale_lo), _ptr(act_scale_hi),
-                                      _ptr(bias), _ptr(Y), wp, wb, _ptr(status), _stream()),
-         "mixdq_conv3x3_a8_split")
-    return Y
 
 
 def conv3x3_a8_split_acc_i32(X, split_at: int, packed_W_lo, packed_W_hi, Cout: int, w_bits: int, act_scale_lo,
@@ -453,29 +306,6 @@ def conv3x3_acc_i32(X, packed_W, Cout: int, w_bits: int, act_scale, stride: int 
     return acc
 
 
-def conv1x1(X, packed_W, Cout: int, w_bits: int, w_scale, w_zero=None, act_bits: int = 8, act_scale=None,
-            bias=None, workspace=None, status=None):
-    B, H, W, Cin = X.shape
-    Y = torch.empty((B, H, W, Cout), dtype=torch.float16, device=X.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_conv1x1(_ptr(X), B, H, W, Cin, _ptr(packed_W), Cout, w_bits, _ptr(w_scale), _ptr(w_zero),
-                             act_bits, _ptr(act_scale), _ptr(bias), _ptr(Y), wp, wb, _ptr(status), _stream()),
-         "mixdq_conv1x1")
-    return Y
-
-
-def crossattn_kv(text_emb, packed_W, N: int, w_bits: int, w_scale, act_scale, bos_out, workspace=None,
-                 status=None, out=None):
-    B, T, Kt = text_emb.shape
-    assert T == TOKENS_PER_PROMPT
-    Y = out if out is not None else torch.empty((B, T, N), dtype=torch.float16, device=text_emb.device)
-    wp, wb = _ws(workspace)
-    _chk(lib().mixdq_crossattn_kv(_ptr(text_emb), B, Kt, _ptr(packed_W), N, w_bits, _ptr(w_scale),
-                                  _ptr(act_scale), _ptr(bos_out), _ptr(Y), wp, wb, _ptr(status), _stream()),
-         "mixdq_crossattn_kv")
-    return Y
-
-
 def crossattn_kv_acc_i32(text_emb, packed_W, N: int, w_bits: int, act_scale, workspace=None, status=None):
     B, T, Kt = text_emb.shape
     assert T == TOKENS_PER_PROMPT
@@ -489,18 +319,6 @@ def crossattn_kv_acc_i32(text_emb, packed_W, N: int, w_bits: int, act_scale, wor
 
 def static_scratch_bytes() -> int:
     return lib().mixdq_static_scratch_bytes()
-
-
-def linear_a8_static_scratch(X, packed_W, N: int, w_bits: int, w_scale, act_scale, bias=None, status=None,
-                             out=None):
-    """W8A8 / W4A8 linear whose scratch is the library's built-in array: for callers that cannot
-    allocate device memory.  The output tensor is still the caller's (``out``, or a fresh one here)."""
-    M, K = X.shape
-    Y = out if out is not None else torch.empty((M, N), dtype=torch.float16, device=X.device)
-    _chk(lib().mixdq_linear_a8_static_scratch(_ptr(X), M, K, X.stride(0), _ptr(packed_W), N, w_bits,
-                                              _ptr(w_scale), _ptr(act_scale), _ptr(bias), _ptr(Y), _ptr(status),
-                                              _stream()), "mixdq_linear_a8_static_scratch")
-    return Y
 
 
 def probe_mma_loop(kind: int, batches: int, repeats: int = 3) -> float:
