@@ -63,6 +63,12 @@ int encode_tmap_4d_u8(CUtensorMap* map, const void* base, const uint64_t dims[4]
 int encode_tmap_4d_f16(CUtensorMap* map, const void* base, const uint64_t dims[4], const uint64_t strides_bytes[3],
                        const uint32_t box[4], uint32_t hw_step = 1);
 
+// im2col tensor map of a 3x3 window with zero padding 1 over an NHWC image (int8, or fp16): a load takes `pixels`
+// consecutive output pixels -- across image rows and images, whatever the image size -- x `channels` elements at one
+// filter tap (the 128-byte swizzle: channels span 128 bytes).  pad = 1: H and W include a one-pixel border.
+int encode_tmap_im2col3x3(CUtensorMap* map, const void* base, bool f16, int B, int H, int W, int C, int pad, int stride,
+                          int channels, int pixels);
+
 // Once per kernel: ask for the largest shared-memory carve-out.  An SM changes its L1 / shared
 // split only when idle, so kernels with different preferences cannot share an SM and the change
 // itself costs time at every kernel boundary; with one preference everywhere, a small kernel's
@@ -268,6 +274,18 @@ __device__ __forceinline__ void tma_load_4d(uint32_t dst, const CUtensorMap* map
         "cp.async.bulk.tensor.4d.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
         "%3, %4, %5}], [%6];" ::"r"(dst),
         "l"(reinterpret_cast<uint64_t>(map)), "r"(c0), "r"(c1), "r"(c2), "r"(c3), "r"(bar)
+        : "memory");
+}
+
+// im2col form: {channel, w, h, image} of the first pixel's window corner, and the filter tap's offset in the window.
+__device__ __forceinline__ void tma_load_im2col(uint32_t dst, const CUtensorMap* map, int c, int w, int h, int n, int kw, int kh,
+                                                uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%2, "
+        "%3, %4, %5}], [%6], {%7, %8};" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(w), "r"(h), "r"(n), "r"(bar), "h"(static_cast<uint16_t>(kw)),
+        "h"(static_cast<uint16_t>(kh))
         : "memory");
 }
 

@@ -56,6 +56,8 @@ int run(Params p, int amode, const void* packed, int w_bits, void* workspace, si
         cudaStream_t stream);
 // Two-kernel path (quantize once, then a TMA-fed GEMM); see i8_tma.cu.
 bool tma_path_ok(const Params& p, int amode, int w_bits);
+// Whether a 3x3 convolution of another image geometry can take the same path through im2col loads.
+bool im2col_path_ok(const Params& p);
 int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* scratch, cudaStream_t stream);
 // Tile width of the pair form (two-CTA tiles of 256 x width) when the planner prefers it for an int8 GEMM of
 // M x N over k_blocks k-blocks of 128, else 0 (the single-CTA kernels run).  *splits (optional): how many CTA

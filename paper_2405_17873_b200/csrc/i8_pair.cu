@@ -131,6 +131,16 @@ __device__ __forceinline__ void tma_load_4d_pair(uint32_t dst, const CUtensorMap
         : "memory");
 }
 
+__device__ __forceinline__ void tma_load_im2col_pair(uint32_t dst, const CUtensorMap* map, int c, int w, int h, int n, int kw,
+                                                     int kh, uint32_t bar)
+{
+    asm volatile(
+        "cp.async.bulk.tensor.4d.cta_group::2.shared::cluster.global.im2col.mbarrier::complete_tx::bytes [%0], [%1, {%2, %3, %4, %5}], [%6], {%7, %8};" ::"r"(dst),
+        "l"(reinterpret_cast<uint64_t>(map)), "r"(c), "r"(w), "r"(h), "r"(n), "r"(bar), "h"(static_cast<uint16_t>(kw)),
+        "h"(static_cast<uint16_t>(kh))
+        : "memory");
+}
+
 // Arrive on a barrier that may belong to the other CTA of the cluster (address in the cluster's shared
 // window).  Default semantics, as for a local arrive: a release at cluster scope was measured to cost the
 // arriving thread some 2000 cycles per call (it turned a 550-cycle expansion turn into a 2600-cycle one).
@@ -334,8 +344,9 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                 const int m0 = (tile / g.n_tiles) * (2 * BM) + static_cast<int>(rank) * BM;
                 int img_b = 0, ho0 = 0, wo0 = 0, cb = 0, kh = 0, kw = 0, xa = kb_begin * BKE;
                 if (p.conv) {
-                    img_b = m0 / p.HoWo;
-                    const int rem = m0 - img_b * p.HoWo;
+                    const int mc = (p.im2col && m0 >= p.M) ? 0 : m0;  // a tile of no output rows: any pixels will do
+                    img_b = mc / p.HoWo;
+                    const int rem = mc - img_b * p.HoWo;
                     ho0 = rem / p.Wo;
                     wo0 = rem - ho0 * p.Wo;
                     const int tap = kb_begin / p.cblocks;
@@ -359,8 +370,11 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
                     if (leader) mbar_arrive_expect_tx(bar0 + 8 * (L::FULL_A + s), 2 * L::A_BYTES);
                     const uint32_t full = lead_bar0 + 8 * (L::FULL_A + s);
                     if (p.conv) {
-                        tma_load_4d_pair(a0 + s * L::A_BYTES, map, cb * BKE, p.stride * wo0 + kw - 1 + p.pad,
-                                         p.stride * ho0 + kh - 1 + p.pad, img_b, full);
+                        const int wi = p.stride * wo0 - 1 + p.pad, hi = p.stride * ho0 - 1 + p.pad;
+                        if (p.im2col)
+                            tma_load_im2col_pair(a0 + s * L::A_BYTES, map, cb * BKE, wi, hi, img_b, kw, kh, full);
+                        else
+                            tma_load_4d_pair(a0 + s * L::A_BYTES, map, cb * BKE, wi + kw, hi + kh, img_b, full);
                         if (++cb == cblocks) {
                             cb = 0;
                             if (++kw == 3) {

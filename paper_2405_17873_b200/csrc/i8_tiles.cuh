@@ -18,6 +18,7 @@ struct TmaParams {
     int cblocks;  // conv: k-blocks per filter tap = ceil(Cin / 128)
     int Cin, HoWo, Wo;
     int stride;   // conv: input pixels per output pixel along H and W (1 or 2)
+    int im2col;   // conv: the activation map is an im2col one (image sizes that do not tile into 128-pixel boxes)
     int bos;      // output row m maps to row (m / 76) * 77 + m % 76 + 1 of Y
     int batch;
     const float* act_scale;

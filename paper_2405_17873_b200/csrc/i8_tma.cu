@@ -338,6 +338,7 @@ __device__ __forceinline__ bool produce_a_tile(const CUtensorMap* tmap_a, const 
 {
     int img_b = 0, ho0 = 0, wo0 = 0, cb = 0, kh = 0, kw = 0;
     if (p.conv) {
+        if (p.im2col && m0 >= p.M) m0 = 0;  // a tile of no output rows: any pixels will do
         img_b = m0 / p.HoWo;
         const int rem = m0 - img_b * p.HoWo;
         ho0 = rem / p.Wo;
@@ -355,8 +356,11 @@ __device__ __forceinline__ bool produce_a_tile(const CUtensorMap* tmap_a, const 
         const uint32_t full = bar0 + 8 * (L::FULL_A + s);
         mbar_arrive_expect_tx(full, L::A_BYTES);
         if (p.conv) {
-            tma_load_4d(a0 + s * L::A_BYTES, tmap_a, cb * BK, p.stride * wo0 + kw - 1 + p.pad,
-                        p.stride * ho0 + kh - 1 + p.pad, img_b, full);
+            const int wi = p.stride * wo0 - 1 + p.pad, hi = p.stride * ho0 - 1 + p.pad;
+            if (p.im2col)
+                tma_load_im2col(a0 + s * L::A_BYTES, tmap_a, cb * BK, wi, hi, img_b, kw, kh, full);
+            else
+                tma_load_4d(a0 + s * L::A_BYTES, tmap_a, cb * BK, wi + kw, hi + kh, img_b, full);
             if (++cb == p.cblocks) {
                 cb = 0;
                 if (++kw == 3) {
@@ -1252,6 +1256,11 @@ static bool conv_box(int Ho, int Wo, int* Wb, int* Hb, int* Bb)
     return true;
 }
 
+bool im2col_path_ok(const Params& p)
+{
+    return p.Cin % 32 == 0 && (p.stride == 1 || p.stride == 2) && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
+}
+
 bool tma_path_ok(const Params& p, int amode, int w_bits)
 {
     if (amode == A_CONV3) {
@@ -1367,13 +1376,18 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
     tp.tma_store = p.Y && !p.addend && amode != A_BOS && p.ldy % 8 == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 15) == 0;
     if (conv) {
         int Wb, Hb, Bb;
-        if (!conv_box(p.Ho, p.Wo, &Wb, &Hb, &Bb)) return MIXDQ_ERR_UNSUPPORTED;
-        const uint64_t Wi = static_cast<uint64_t>(p.W + 2 * pad), Hi = static_cast<uint64_t>(p.H + 2 * pad);
-        const uint64_t dims[4] = {static_cast<uint64_t>(p.Cin), Wi, Hi, static_cast<uint64_t>(p.batch)};
-        const uint64_t strides[3] = {static_cast<uint64_t>(p.Cin), static_cast<uint64_t>(p.Cin) * Wi,
-                                     static_cast<uint64_t>(p.Cin) * Wi * Hi};
-        const uint32_t box[4] = {BK, static_cast<uint32_t>(Wb), static_cast<uint32_t>(Hb), static_cast<uint32_t>(Bb)};
-        rc = encode_tmap_4d_u8(&ta, aq, dims, strides, box, static_cast<uint32_t>(p.stride));
+        if (tma_path_ok(p, amode, w_bits) && conv_box(p.Ho, p.Wo, &Wb, &Hb, &Bb)) {
+            const uint64_t Wi = static_cast<uint64_t>(p.W + 2 * pad), Hi = static_cast<uint64_t>(p.H + 2 * pad);
+            const uint64_t dims[4] = {static_cast<uint64_t>(p.Cin), Wi, Hi, static_cast<uint64_t>(p.batch)};
+            const uint64_t strides[3] = {static_cast<uint64_t>(p.Cin), static_cast<uint64_t>(p.Cin) * Wi,
+                                         static_cast<uint64_t>(p.Cin) * Wi * Hi};
+            const uint32_t box[4] = {BK, static_cast<uint32_t>(Wb), static_cast<uint32_t>(Hb), static_cast<uint32_t>(Bb)};
+            rc = encode_tmap_4d_u8(&ta, aq, dims, strides, box, static_cast<uint32_t>(p.stride));
+        } else {
+            // any other image size, and stride 2 on odd sides: im2col loads of 128 consecutive output pixels
+            rc = encode_tmap_im2col3x3(&ta, aq, false, p.batch, p.H + 2 * pad, p.W + 2 * pad, p.Cin, pad, p.stride, BK, BM);
+            tp.im2col = 1;
+        }
         tp.conv = 1;
         tp.pad = pad;
         tp.stride = p.stride;

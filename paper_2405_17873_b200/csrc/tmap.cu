@@ -14,20 +14,29 @@ using EncodeTiledFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t
                                    const cuuint64_t*, const cuuint32_t*, const cuuint32_t*,
                                    CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
                                    CUtensorMapFloatOOBfill);
+using EncodeIm2colFn = CUresult (*)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
+                                    const cuuint64_t*, const int*, const int*, cuuint32_t, cuuint32_t, const cuuint32_t*,
+                                    CUtensorMapInterleave, CUtensorMapSwizzle, CUtensorMapL2promotion,
+                                    CUtensorMapFloatOOBfill);
+
+void* driver_entry(const char* name)
+{
+    void* p = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    if (cudaGetDriverEntryPoint(name, &p, cudaEnableDefault, &q) == cudaSuccess && q == cudaDriverEntryPointSuccess) return p;
+    (void)cudaGetLastError();
+    return nullptr;
+}
 
 EncodeTiledFn get_encode_fn()
 {
-    static EncodeTiledFn fn = nullptr;
-    static std::once_flag once;
-    std::call_once(once, [] {
-        void* p = nullptr;
-        cudaDriverEntryPointQueryResult q;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &p, cudaEnableDefault, &q) == cudaSuccess &&
-            q == cudaDriverEntryPointSuccess)
-            fn = reinterpret_cast<EncodeTiledFn>(p);
-        else
-            (void)cudaGetLastError();
-    });
+    static const EncodeTiledFn fn = reinterpret_cast<EncodeTiledFn>(driver_entry("cuTensorMapEncodeTiled"));
+    return fn;
+}
+
+EncodeIm2colFn get_encode_im2col_fn()
+{
+    static const EncodeIm2colFn fn = reinterpret_cast<EncodeIm2colFn>(driver_entry("cuTensorMapEncodeIm2col"));
     return fn;
 }
 
@@ -104,6 +113,26 @@ static int encode_tmap_4d(CUtensorMap* map, CUtensorMapDataType dtype, const voi
     CUresult r = fn(map, dtype, 4, const_cast<void*>(base), d, st, b, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B,
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
+    return r == CUDA_SUCCESS ? MIXDQ_OK : MIXDQ_ERR_CUDA;
+}
+
+int encode_tmap_im2col3x3(CUtensorMap* map, const void* base, bool f16, int B, int H, int W, int C, int pad, int stride,
+                          int channels, int pixels)
+{
+    EncodeIm2colFn fn = get_encode_im2col_fn();
+    if (!fn) return MIXDQ_ERR_CUDA;
+    const cuuint64_t row = static_cast<cuuint64_t>(C) * (f16 ? 2 : 1);
+    if ((reinterpret_cast<uintptr_t>(base) & 15) || (row & 15)) return MIXDQ_ERR_ALIGNMENT;
+    const cuuint64_t d[4] = {static_cast<cuuint64_t>(C), static_cast<cuuint64_t>(W), static_cast<cuuint64_t>(H),
+                             static_cast<cuuint64_t>(B)};
+    const cuuint64_t st[3] = {row, row * W, row * W * H};
+    // the filter's corner pixel runs over [-1, W - 2] (a border that is part of the image moves it by one)
+    const int lower[2] = {pad - 1, pad - 1}, upper[2] = {-1 - pad, -1 - pad};
+    const cuuint32_t step[4] = {1, static_cast<cuuint32_t>(stride), static_cast<cuuint32_t>(stride), 1};
+    CUresult r = fn(map, f16 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_UINT8, 4, const_cast<void*>(base),
+                    d, st, lower, upper, static_cast<cuuint32_t>(channels), static_cast<cuuint32_t>(pixels), step,
+                    CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
+                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? MIXDQ_OK : MIXDQ_ERR_CUDA;
 }
 

@@ -116,10 +116,7 @@ bool pair_path_ok(const Params& p, int amode, int w_bits)
     if (p.M < 2 * BM || p.N < 32) return false;  // below that the fused expansion is the better form
     if (w_bits <= 3 && !p.w_zero) return false;  // bit-plane codes are unsigned
     if (amode == A_CONV3) {
-        int a, b, c;
-        if (p.Cin % 8 != 0) return false;
-        if (p.stride != 1 && !(p.stride == 2 && p.H % 2 == 0 && p.W % 2 == 0)) return false;
-        return conv_box(p.Ho, p.Wo, &a, &b, &c);
+        return p.Cin % 8 == 0 && (p.stride == 1 || p.stride == 2) && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
     }
     return amode == A_LINEAR && p.K % 8 == 0 && p.ldx % 8 == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
 }
@@ -141,13 +138,17 @@ int run_pair(const Params& p, int amode, const void* packed, int w_bits, cudaStr
     CUtensorMap ta, tw, ty{};
     if (amode == A_CONV3) {
         int Wb, Hb, Bb;
-        if (!conv_box(p.Ho, p.Wo, &Wb, &Hb, &Bb)) return MIXDQ_ERR_UNSUPPORTED;
-        const uint64_t dims[4] = {static_cast<uint64_t>(p.Cin), static_cast<uint64_t>(p.W), static_cast<uint64_t>(p.H),
-                                  static_cast<uint64_t>(p.batch)};
-        const uint64_t strides[3] = {static_cast<uint64_t>(p.Cin) * 2, static_cast<uint64_t>(p.Cin) * p.W * 2,
-                                     static_cast<uint64_t>(p.Cin) * p.W * p.H * 2};
-        const uint32_t box[4] = {BKE, static_cast<uint32_t>(Wb), static_cast<uint32_t>(Hb), static_cast<uint32_t>(Bb)};
-        rc = encode_tmap_4d_f16(&ta, p.X, dims, strides, box, static_cast<uint32_t>(p.stride));
+        if ((p.stride == 1 || (p.H % 2 == 0 && p.W % 2 == 0)) && conv_box(p.Ho, p.Wo, &Wb, &Hb, &Bb)) {
+            const uint64_t dims[4] = {static_cast<uint64_t>(p.Cin), static_cast<uint64_t>(p.W), static_cast<uint64_t>(p.H),
+                                      static_cast<uint64_t>(p.batch)};
+            const uint64_t strides[3] = {static_cast<uint64_t>(p.Cin) * 2, static_cast<uint64_t>(p.Cin) * p.W * 2,
+                                         static_cast<uint64_t>(p.Cin) * p.W * p.H * 2};
+            const uint32_t box[4] = {BKE, static_cast<uint32_t>(Wb), static_cast<uint32_t>(Hb), static_cast<uint32_t>(Bb)};
+            rc = encode_tmap_4d_f16(&ta, p.X, dims, strides, box, static_cast<uint32_t>(p.stride));
+        } else {  // any other image size: im2col loads of 128 consecutive output pixels
+            rc = encode_tmap_im2col3x3(&ta, p.X, true, p.batch, p.H, p.W, p.Cin, 0, p.stride, BKE, BM);
+            tp.im2col = 1;
+        }
         tp.conv = 1;
         tp.stride = p.stride;
         tp.cblocks = static_cast<int>(ceil_div(p.Cin, BKE));

@@ -41,6 +41,7 @@ constexpr int kFeedWarps = 8;
 struct TcParams {
     int M, N, K, k_blocks;
     int conv, cblocks, Cin, HoWo, Wo;
+    int im2col, stride;  // conv: the activation map is an im2col one, with this stride
     const float* w_scale;
     const int32_t* w_zero;
     const __half* bias;
@@ -215,7 +216,11 @@ wo_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const TcParams p, int n
                     if (p.conv) {
                         const int tap = kb / p.cblocks, cb = kb - tap * p.cblocks;
                         const int kh = tap / 3, kw = tap - 3 * kh;
-                        tma_load_4d(dst, &tmap_x, cb * BKE, wo0 + kw - 1, ho0 + kh - 1, img_b, bar_full_a + 8 * s);
+                        if (p.im2col)
+                            tma_load_im2col(dst, &tmap_x, cb * BKE, p.stride * wo0 - 1, p.stride * ho0 - 1, img_b, kw, kh,
+                                            bar_full_a + 8 * s);
+                        else
+                            tma_load_4d(dst, &tmap_x, cb * BKE, wo0 + kw - 1, ho0 + kh - 1, img_b, bar_full_a + 8 * s);
                     } else {
                         tma_load_2d(dst, &tmap_x, kb * BKE, m0, bar_full_a + 8 * s);
                     }
@@ -429,10 +434,8 @@ bool tc_path_ok(const Params& p, int amode, int w_bits)
 {
     if (p.M < 64) return false;
     if (amode == A_CONV3) {
-        int a, b, c;
         // whole 32-code runs per k-block: channel count a multiple of 64
-        if (p.stride != 1 || p.Cin % 64 != 0) return false;
-        return conv_box(p.Ho, p.Wo, &a, &b, &c);
+        return p.Cin % 64 == 0 && (p.stride == 1 || p.stride == 2) && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
     }
     (void)w_bits;
     return amode == A_LINEAR && p.K % 8 == 0 && p.ldx % 8 == 0 && (reinterpret_cast<uintptr_t>(p.X) & 15) == 0;
@@ -456,13 +459,18 @@ int run_tc(const Params& p, int amode, const void* packed, int w_bits, int batch
     int rc;
     if (amode == A_CONV3) {
         int Wb, Hb, Bb;
-        if (!conv_box(p.Ho, p.Wo, &Wb, &Hb, &Bb)) return MIXDQ_ERR_UNSUPPORTED;
-        const uint64_t dims[4] = {static_cast<uint64_t>(p.Cin), static_cast<uint64_t>(p.W),
-                                  static_cast<uint64_t>(p.H), static_cast<uint64_t>(batch)};
-        const uint64_t strides[3] = {static_cast<uint64_t>(p.Cin) * 2, static_cast<uint64_t>(p.Cin) * p.W * 2,
-                                     static_cast<uint64_t>(p.Cin) * p.W * p.H * 2};
-        const uint32_t box[4] = {BKE, static_cast<uint32_t>(Wb), static_cast<uint32_t>(Hb), static_cast<uint32_t>(Bb)};
-        rc = encode_tmap_4d_f16(&tx, p.X, dims, strides, box);
+        if (p.stride == 1 && conv_box(p.Ho, p.Wo, &Wb, &Hb, &Bb)) {
+            const uint64_t dims[4] = {static_cast<uint64_t>(p.Cin), static_cast<uint64_t>(p.W),
+                                      static_cast<uint64_t>(p.H), static_cast<uint64_t>(batch)};
+            const uint64_t strides[3] = {static_cast<uint64_t>(p.Cin) * 2, static_cast<uint64_t>(p.Cin) * p.W * 2,
+                                         static_cast<uint64_t>(p.Cin) * p.W * p.H * 2};
+            const uint32_t box[4] = {BKE, static_cast<uint32_t>(Wb), static_cast<uint32_t>(Hb), static_cast<uint32_t>(Bb)};
+            rc = encode_tmap_4d_f16(&tx, p.X, dims, strides, box);
+        } else {  // any other image size, and stride 2: im2col loads of 128 consecutive output pixels
+            rc = encode_tmap_im2col3x3(&tx, p.X, true, batch, p.H, p.W, p.Cin, 0, p.stride, BKE, BM);
+            tp.im2col = 1;
+        }
+        tp.stride = p.stride;
         tp.conv = 1;
         tp.cblocks = p.Cin / BKE;
         tp.Cin = p.Cin;
