@@ -135,6 +135,10 @@ int mixdq_act_absmax(const void* X, int64_t rows, int64_t cols, int64_t row_stri
  * symmetric int8 activation scale of Sec. 4.1 computed on the device. */
 int mixdq_act_scale_from_absmax(const float* amax, float* scale_out, void* stream);
 
+/* Both steps in one call: scale_out[0] = max |x| / 127 (1 when that is 0). */
+int mixdq_act_scale(const void* X, int64_t rows, int64_t cols, int64_t row_stride, int skip_rows_mod,
+                    float* scale_out, void* stream);
+
 /*
  * Range of an fp16 matrix [rows, cols] (row stride `row_stride` elements) with 0 included:
  * minmax_out[0] = min(min x, 0), minmax_out[1] = max(max x, 0) (device fp32 [2]).  The first step of the
@@ -147,6 +151,10 @@ int mixdq_act_minmax(const void* X, int64_t rows, int64_t cols, int64_t row_stri
  * zero_out[0] = clamp(rne(-lo / scale), 0, 255) (int32); scale 1 and zero 0 when hi == lo. */
 int mixdq_act_asym_params_from_minmax(const float* minmax, float* scale_out, int32_t* zero_out,
                                       void* stream);
+
+/* Both steps in one call: the asymmetric parameters of an fp16 matrix. */
+int mixdq_act_asym_params(const void* X, int64_t rows, int64_t cols, int64_t row_stride, float* scale_out,
+                          int32_t* zero_out, void* stream);
 
 /* sums_out[n] = sum_k q[n, k] (device int32 [N]) of the signed codes of a MIXDQ_LAYOUT_DEVICE weight with
  * bits in {4, 8}: computed once per layer, it carries the activation zero-point through the int8 GEMM. */

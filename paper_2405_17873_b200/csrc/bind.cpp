@@ -270,13 +270,10 @@ PyObject* act_scale(const Args& a)
     const at::Tensor& X = a.tensor(0);
     Rows x(X);
     const int skip = static_cast<int>(a.integer(1));
-    Output amax(a, -1, {1}, kF32, X), out(a, -1, {1}, kF32, X);
+    Output out(a, -1, {1}, kF32, X);
     void* st = current_stream();
-    call("mixdq_act_absmax", [&] {
-        return mixdq_act_absmax(x.data, x.rows, x.cols, x.cols, skip, static_cast<float*>(amax.address), st);
-    });
-    call("mixdq_act_scale_from_absmax", [&] {
-        return mixdq_act_scale_from_absmax(static_cast<float*>(amax.address), static_cast<float*>(out.address), st);
+    call("mixdq_act_scale", [&] {
+        return mixdq_act_scale(x.data, x.rows, x.cols, x.cols, skip, static_cast<float*>(out.address), st);
     });
     return out.release();
 }
@@ -296,13 +293,11 @@ PyObject* act_asym_params(const Args& a)
 {
     const at::Tensor& X = a.tensor(0);
     Rows x(X);
-    Output range(a, -1, {2}, kF32, X), scale(a, -1, {1}, kF32, X), zero(a, -1, {1}, kI32, X);
+    Output scale(a, -1, {1}, kF32, X), zero(a, -1, {1}, kI32, X);
     void* st = current_stream();
-    call("mixdq_act_minmax",
-         [&] { return mixdq_act_minmax(x.data, x.rows, x.cols, x.cols, static_cast<float*>(range.address), st); });
-    call("mixdq_act_asym_params_from_minmax", [&] {
-        return mixdq_act_asym_params_from_minmax(static_cast<float*>(range.address), static_cast<float*>(scale.address),
-                                                 static_cast<int32_t*>(zero.address), st);
+    call("mixdq_act_asym_params", [&] {
+        return mixdq_act_asym_params(x.data, x.rows, x.cols, x.cols, static_cast<float*>(scale.address),
+                                     static_cast<int32_t*>(zero.address), st);
     });
     PyObject* pair = PyTuple_Pack(2, scale.object, zero.object);
     if (!pair) throw Failed{};

@@ -75,11 +75,20 @@ int encode_tmap_im2col3x3(CUtensorMap* map, const void* base, bool f16, int B, i
 // tail and the next GEMM's set-up overlap.  Returns MIXDQ_OK or MIXDQ_ERR_CUDA.
 int prefer_max_shared_carveout(const void* kernel);
 
+// Once per (device, kernel): allow clusters of more than 8 CTAs (not portable; 16 on this architecture).
+int allow_large_clusters(const void* kernel);
+
 // Once per (device, kernel): raise the kernel's dynamic shared-memory limit to `bytes`.
 int ensure_dynamic_smem(const void* kernel, int bytes);
 
 // Streaming multiprocessors of the current device (looked up once per device; 0 on error).
 int sm_count();
+
+// A call on `stream` has written constants of a layer: the library's next kernel there must not start before they are
+// complete.  False: no room for another stream's note (the caller orders the two by other means).
+bool note_constants_written(cudaStream_t stream);
+// Whether there is such a note for `stream`; takes it.
+bool take_constants_note(cudaStream_t stream);
 
 #ifdef __CUDACC__
 
@@ -98,11 +107,24 @@ inline int launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sm
     return launch_pdl_cluster(kernel, grid, block, smem, stream, 1u, cluster_z, static_cast<Args&&>(args)...);
 }
 
+template <typename... KArgs, typename... Args>
+inline int launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, unsigned cluster_x,
+                     unsigned cluster_z, Args&&... args);
+
 // The same with a cluster of cluster_x x 1 x cluster_z CTAs (kernels whose CTA pairs share tensor-core
 // instructions need their pairs adjacent along x).
 template <typename... KArgs, typename... Args>
 inline int launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream,
                               unsigned cluster_x, unsigned cluster_z, Args&&... args)
+{
+    g_layer_kernel_launches.fetch_add(1, std::memory_order_relaxed);
+    return launch_ex(kernel, grid, block, smem, stream, cluster_x, cluster_z, static_cast<Args&&>(args)...);
+}
+
+// The launch itself, for kernels that are not a layer call's.
+template <typename... KArgs, typename... Args>
+inline int launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t stream, unsigned cluster_x,
+                     unsigned cluster_z, Args&&... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = grid;
@@ -111,7 +133,7 @@ inline int launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.stream = stream;
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    attr[0].val.programmaticStreamSerializationAllowed = take_constants_note(stream) ? 0 : 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = cluster_x;
     attr[1].val.clusterDim.y = 1;
@@ -119,7 +141,6 @@ inline int launch_pdl_cluster(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
     cfg.attrs = attr;
     cfg.numAttrs = (cluster_z > 1 || cluster_x > 1) ? 2 : 1;
     if (prefer_max_shared_carveout(reinterpret_cast<const void*>(kernel)) != MIXDQ_OK) return MIXDQ_ERR_CUDA;
-    g_layer_kernel_launches.fetch_add(1, std::memory_order_relaxed);
     cudaError_t err = cudaLaunchKernelEx(&cfg, kernel, static_cast<KArgs>(args)...);
     if (err != cudaSuccess) {
         (void)cudaGetLastError();
@@ -143,6 +164,32 @@ __device__ __forceinline__ void pdl_wait()
     asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
+
+// ---- thread-block clusters
+
+__device__ __forceinline__ uint32_t cluster_ctarank()
+{
+    uint32_t r;
+    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
+    return r;
+}
+
+// Address of this CTA's shared-memory location `addr` as seen in CTA `rank` of the cluster.
+__device__ __forceinline__ uint32_t map_to_cta(uint32_t addr, uint32_t rank)
+{
+    uint32_t out;
+    asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(out) : "r"(addr), "r"(rank));
+    return out;
+}
+
+// Barrier over all threads of all CTAs of the cluster (hardware barrier, not a spin), whole or in two steps.
+__device__ __forceinline__ void cluster_arrive() { asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_wait() { asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory"); }
+__device__ __forceinline__ void cluster_sync()
+{
+    cluster_arrive();
+    cluster_wait();
+}
 
 // Spin budget of every bounded wait, in SM clock cycles (a few hundred ms).
 constexpr long long kWaitBudgetCycles = 400000000LL;

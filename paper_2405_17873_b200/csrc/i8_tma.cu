@@ -142,13 +142,6 @@ __global__ void quant_split_kernel(const __half* __restrict__ X, long long ldx, 
     *reinterpret_cast<uint4*>(dst) = q;
 }
 
-// Barrier over all threads of all CTAs of the cluster (hardware barrier, not a spin).
-__device__ __forceinline__ void cluster_sync_all()
-{
-    asm volatile("barrier.cluster.arrive.release.aligned;" ::: "memory");
-    asm volatile("barrier.cluster.wait.acquire.aligned;" ::: "memory");
-}
-
 // 16 bytes from the shared memory of CTA `cta_rank` of this cluster, at this CTA's offset `addr`.
 __device__ __forceinline__ int4 ld_cluster_v4(uint32_t addr, int cta_rank)
 {
@@ -736,7 +729,7 @@ tma_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     // `rank` adds up rows [rank * 128 / splits, ...) over all of them (integer adds: exact,
     // order-free), dequantizes and stores; threads run along a row so stores coalesce.
     __syncthreads();
-    if (splits > 1) cluster_sync_all();
+    if (splits > 1) cluster_sync();
     if (!*s_abort && !direct) {
         // a thread keeps one group of four columns (its factors stay in registers) and walks
         // down the rows; consecutive threads take consecutive column groups
@@ -837,7 +830,7 @@ tma_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
     }
     tc_fence_before_sync();
     __syncthreads();
-    if (splits > 1) cluster_sync_all();  // peers may still be reading this CTA's shared memory
+    if (splits > 1) cluster_sync();  // peers may still be reading this CTA's shared memory
     if (warp == 1) tmem_dealloc(tmem_base, L::TMEM_COLS);
 }
 

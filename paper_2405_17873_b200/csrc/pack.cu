@@ -1,7 +1,5 @@
 // Offline side of the path: per-channel min-max parameters, weight quantization and
-// packing (3 / 4 / 8 bits, canonical and device layouts), the unpack parity hook, and the
-// per-tensor activation range helpers.  None of this is on the per-step hot path, so the
-// kernels favour exactness (products in double, one IEEE divide per scale) over speed.
+// packing (2 / 3 / 4 / 8 bits, canonical and device layouts) and the unpack parity hook.
 #include "common.cuh"
 #include "codes.cuh"
 
@@ -22,34 +20,63 @@ __device__ __forceinline__ int clampi(long long v, int lo, int hi)
     return v < lo ? lo : (v > hi ? hi : static_cast<int>(v));
 }
 
-// One block per output channel: min / max of the row, then scale and zero-point.
-__global__ void weight_minmax_kernel(const __half* __restrict__ W, int64_t K, int bits, int symmetric,
-                                     float* __restrict__ scale_out, int32_t* __restrict__ zero_out)
+// Min / max of every output channel's row, then its scale and zero-point.  T threads per row: a warp for rows of up to
+// 4096 weights (all its 16-byte loads in flight at once, no barrier), a CTA of 256 for longer ones.  Bound by reading W:
+// 10240 x 1280 took 17 us with one CTA and two-byte loads per row.
+constexpr int kRowWarp = 4096;
+
+template <int T>
+__global__ void __launch_bounds__(256)
+weight_minmax_kernel(const __half* __restrict__ W, int64_t N, int64_t K, int bits, int symmetric,
+                     float* __restrict__ scale_out, int32_t* __restrict__ zero_out)
 {
-    const int64_t n = blockIdx.x;
-    const __half* row = W + n * K;
+    const int64_t n = blockIdx.x * static_cast<int64_t>(256 / T) + threadIdx.x / T;
+    const int t = threadIdx.x % T;
     float lo = 0.f, hi = 0.f;
-    for (int64_t k = threadIdx.x; k < K; k += blockDim.x) {
-        float w = __half2float(row[k]);
-        lo = fminf(lo, w);
-        hi = fmaxf(hi, w);
+    if (n < N) {
+        const __half* row = W + n * K;
+        __half2 l2 = __half2half2(__ushort_as_half(0)), h2 = l2;
+        int64_t done = 0;
+        if ((reinterpret_cast<uintptr_t>(row) & 15) == 0) {
+            const uint4* v4 = reinterpret_cast<const uint4*>(row);
+            const int chunks = static_cast<int>(K >> 3);
+#pragma unroll 8
+            for (int c = t; c < chunks; c += T) {
+                const uint4 v = __ldg(v4 + c);
+                const __half2* h = reinterpret_cast<const __half2*>(&v);
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    l2 = __hmin2(l2, h[j]);
+                    h2 = __hmax2(h2, h[j]);
+                }
+            }
+            done = static_cast<int64_t>(chunks) << 3;
+        }
+        lo = fminf(__low2float(l2), __high2float(l2));
+        hi = fmaxf(__low2float(h2), __high2float(h2));
+        for (int64_t k = done + t; k < K; k += T) {
+            const float w = __half2float(row[k]);
+            lo = fminf(lo, w);
+            hi = fmaxf(hi, w);
+        }
     }
-    __shared__ float s_lo[32], s_hi[32];
     for (int o = 16; o > 0; o >>= 1) {
         lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
         hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
     }
-    if ((threadIdx.x & 31) == 0) {
-        s_lo[threadIdx.x >> 5] = lo;
-        s_hi[threadIdx.x >> 5] = hi;
-    }
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        for (int i = 1; i < nw; ++i) {
+    if (T > 32) {
+        __shared__ float s_lo[8], s_hi[8];
+        if ((threadIdx.x & 31) == 0) {
+            s_lo[threadIdx.x >> 5] = lo;
+            s_hi[threadIdx.x >> 5] = hi;
+        }
+        __syncthreads();
+        for (int i = 0; i < 8; ++i) {
             lo = fminf(lo, s_lo[i]);
             hi = fmaxf(hi, s_hi[i]);
         }
+    }
+    if (t == 0 && n < N) {
         if (symmetric) {
             const float amax = fmaxf(-lo, hi);
             const float qmax = static_cast<float>((1 << (bits - 1)) - 1);
@@ -65,75 +92,129 @@ __global__ void weight_minmax_kernel(const __half* __restrict__ W, int64_t K, in
     }
 }
 
-// Code of element (n, k); positions beyond K hold the pad code (0 signed, zero-point unsigned).
-__device__ __forceinline__ int code_at(const __half* __restrict__ W, int64_t n, int64_t k, int64_t K,
-                                       int bits, float inv, bool has_zero, int z)
+// Quantize and pack: one thread per 32 consecutive codes of a row, read once (four 16-byte loads where rows are
+// aligned) and written as the group's BITS words.  A code is clamp(rne(w * inv) [+ zero]): one fma against 1.5 * 2^23
+// rounds the exact product to nearest even, the clamp acts on that float (it is monotonic, so a product too large
+// for the trick clamps to the right end too), the code is the low bits of the result.  The form before this one made
+// one thread per output WORD, so that a bit-plane layout computed every code once per plane, with products in double:
+// 10240 x 1280 to 3 bits took 74 us.
+template <int BITS>
+__global__ void __launch_bounds__(256)
+pack_kernel(const __half* __restrict__ W, int64_t N, int64_t K, int groups, const float* __restrict__ scale,
+            const int32_t* __restrict__ zero, int layout, int64_t pitch, uint8_t* __restrict__ out)
 {
-    if (k >= K) return has_zero ? z : 0;
-    const long long r = rne_product(__half2float(W[n * K + k]), inv);
-    if (has_zero) return clampi(r + z, 0, (1 << bits) - 1);
-    const int qmax = (1 << (bits - 1)) - 1;
-    return clampi(r, -qmax, qmax);
-}
-
-// One thread per 32-bit output word of a packed row.
-__global__ void pack_kernel(const __half* __restrict__ W, int64_t N, int64_t K, int bits,
-                            const float* __restrict__ scale, const int32_t* __restrict__ zero,
-                            int layout, int64_t pitch, uint8_t* __restrict__ out)
-{
-    const int64_t words_per_row = (pitch + 3) / 4;
-    const int64_t idx = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x;
-    if (idx >= N * words_per_row) return;
-    const int64_t n = idx / words_per_row;
-    const int64_t w = idx - n * words_per_row;
+    constexpr float kMagic = 12582912.f;
+    const int64_t idx = blockIdx.x * static_cast<int64_t>(256) + threadIdx.x;
+    if (idx >= N * groups) return;
+    const int64_t n = idx / groups;
+    const int g = static_cast<int>(idx - n * groups);
     const float inv = __fdiv_rn(1.f, scale[n]);
     const bool hz = zero != nullptr;
     const int z = hz ? zero[n] : 0;
-    uint8_t* row = out + n * pitch;
-    uint32_t word = 0;
+    const float lo = kMagic + static_cast<float>(hz ? -z : -((1 << (BITS - 1)) - 1));
+    const float hi = kMagic + static_cast<float>(hz ? (1 << BITS) - 1 - z : (1 << (BITS - 1)) - 1);
+    const uint32_t offset = static_cast<uint32_t>(z) - 0x4B400000u;  // float bits of the clamped sum -> code
+    // positions beyond K: the pad code (0 signed, zero-point unsigned); nothing in a canonical row's last nibble
+    const uint32_t pad = (BITS == 4 && layout == MIXDQ_LAYOUT_CANONICAL) ? 0u : static_cast<uint32_t>(z);
+    const int64_t k0 = 32ll * g;
+    const __half* src = W + n * K + k0;
+    const bool whole = k0 + 32 <= K && (reinterpret_cast<uintptr_t>(src) & 15) == 0;
 
-    if (bits == 8) {
-        for (int j = 0; j < 4; ++j)
-            word |= static_cast<uint32_t>(code_at(W, n, 4 * w + j, K, 8, inv, hz, z) & 0xff) << (8 * j);
-    } else if (bits == 4) {
-        if (layout == MIXDQ_LAYOUT_CANONICAL) {
-            // an odd K leaves the last high nibble empty (0) in the canonical layout
-            for (int j = 0; j < 8; ++j)
-                if (8 * w + j < K)
-                    word |= static_cast<uint32_t>(code_at(W, n, 8 * w + j, K, 4, inv, hz, z) & 0xf)
-                            << (4 * j);
-        } else {
-            // byte j of the word: code j in the low nibble, code j + 4 in the high nibble
+    uint32_t nib[4];         // eight 4-bit fields of codes 8 s .. 8 s + 7, in the order the layout packs them
+    uint32_t words[8];       // the group's packed words
+#pragma unroll
+    for (int s = 0; s < 4; ++s) {
+        float f[8];
+        uint32_t c[8];
+        if (whole) {
+            const uint4 v = __ldg(reinterpret_cast<const uint4*>(src) + s);
+            const __half2* h = reinterpret_cast<const __half2*>(&v);
+#pragma unroll
             for (int j = 0; j < 4; ++j) {
-                const uint32_t lo = code_at(W, n, 8 * w + j, K, 4, inv, hz, z) & 0xf;
-                const uint32_t hi = code_at(W, n, 8 * w + 4 + j, K, 4, inv, hz, z) & 0xf;
-                word |= (lo | (hi << 4)) << (8 * j);
+                const float2 t = __half22float2(h[j]);
+                f[2 * j] = t.x;
+                f[2 * j + 1] = t.y;
             }
-        }
-    } else {  // bit-planes: `bits` (3 or 2) planes per group
-        if (layout == MIXDQ_LAYOUT_CANONICAL) {
-            const int64_t k0 = 32 * (w / bits);  // group g: words bits*g .. are planes 0..bits-1
-            const int plane = static_cast<int>(w % bits);
-            for (int j = 0; j < 32; ++j)
-                word |= static_cast<uint32_t>((code_at(W, n, k0 + j, K, bits, inv, hz, z) >> plane) & 1) << j;
         } else {
-            // block of 128 codes: planes in order, 4 words each; word t of a plane covers codes
-            // 32t .. 32t+31 with bit 4f + s = code 8s + (f even ? f/2 : 4 + f/2), which is the
-            // field order of the 4-bit device layout spread over four shifts of the word
-            const int64_t blk = w / (4 * bits);
-            const int r = static_cast<int>(w % (4 * bits));
-            const int plane = r / 4;
-            const int64_t k0 = 128 * blk + 32 * (r % 4);
-            for (int pos = 0; pos < 32; ++pos) {
-                const int f = pos >> 2, sft = pos & 3;
-                const int j = 8 * sft + ((f & 1) ? 4 + (f >> 1) : (f >> 1));
-                word |= static_cast<uint32_t>((code_at(W, n, k0 + j, K, bits, inv, hz, z) >> plane) & 1) << pos;
+            for (int j = 0; j < 8; ++j) f[j] = k0 + 8 * s + j < K ? __half2float(src[8 * s + j]) : 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+            c[j] = __float_as_uint(fminf(fmaxf(fmaf(f[j], inv, kMagic), lo), hi)) + offset;
+            if (!whole && k0 + 8 * s + j >= K) c[j] = pad;
+        }
+        if (BITS == 8) {
+            words[2 * s] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
+            words[2 * s + 1] = __byte_perm(__byte_perm(c[4], c[5], 0x0040), __byte_perm(c[6], c[7], 0x0040), 0x5410);
+        } else {
+            // fields in order, or (device layouts) field f = code f / 2 (f even), 4 + f / 2 (f odd)
+            uint32_t w = 0;
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {
+                const int fld = (j < 4) ? 2 * j : 2 * (j - 4) + 1;
+                w |= (c[j] & 0xfu) << (4 * (layout == MIXDQ_LAYOUT_CANONICAL ? j : fld));
             }
+            nib[s] = w;
+            if (BITS == 4) words[s] = w;
         }
     }
-    // the last word of an odd-sized canonical row may be partial
-    const int64_t byte0 = 4 * w;
-    for (int b = 0; b < 4 && byte0 + b < pitch; ++b) row[byte0 + b] = (word >> (8 * b)) & 0xff;
+    int64_t byte0 = 4ll * BITS * g, step = 4;  // where the group's words go in the row
+    if (BITS <= 3) {
+        if (layout == MIXDQ_LAYOUT_CANONICAL) {
+            // plane p: bit j = bit p of code j.  Bit p of the eight fields, gathered into one byte per octet.
+#pragma unroll
+            for (int p = 0; p < BITS; ++p) {
+                uint32_t w = 0;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) {
+                    uint32_t x = (nib[s] >> p) & 0x11111111u;  // bits 0, 4, 8, ... -> 0 .. 7
+                    x = (x | (x >> 3)) & 0x03030303u;
+                    x = (x | (x >> 6)) & 0x000f000fu;
+                    x = (x | (x >> 12)) & 0xffu;
+                    w |= x << (8 * s);
+                }
+                words[p] = w;
+            }
+        } else {
+            // blocks of 128 codes, 16 bytes per plane: bit 4 f + s of the word is field f's bit of octet s
+#pragma unroll
+            for (int p = 0; p < BITS; ++p) {
+                uint32_t w = 0;
+#pragma unroll
+                for (int s = 0; s < 4; ++s) w |= ((nib[s] >> p) & 0x11111111u) << s;
+                words[p] = w;
+            }
+            byte0 = (g >> 2) * 16ll * BITS + (g & 3) * 4;
+            step = 16;
+        }
+    }
+    uint8_t* row = out + n * pitch;
+    if (BITS >= 4 && (pitch & 15) == 0) {
+#pragma unroll
+        for (int i = 0; i < BITS; i += 4)
+            if (byte0 + 4 * i < pitch)
+                *reinterpret_cast<uint4*>(row + byte0 + 4 * i) = make_uint4(words[i], words[i + 1], words[i + 2], words[i + 3]);
+    } else if ((pitch & 3) == 0) {
+#pragma unroll
+        for (int i = 0; i < BITS; ++i)
+            if (byte0 + i * step < pitch) *reinterpret_cast<uint32_t*>(row + byte0 + i * step) = words[i];
+    } else {
+        // odd-sized canonical rows: byte by byte, the last word may be partial
+#pragma unroll
+        for (int i = 0; i < BITS; ++i)
+            for (int b = 0; b < 4; ++b)
+                if (byte0 + i * step + b < pitch) row[byte0 + i * step + b] = static_cast<uint8_t>(words[i] >> (8 * b));
+    }
+}
+
+template <int BITS>
+void launch_pack(const __half* W, int64_t N, int64_t K, const float* scale, const int32_t* zero, int layout, int64_t pitch,
+                 uint8_t* out, cudaStream_t st)
+{
+    // groups of 32 codes that cover the row's packed bytes (blocks of 128 codes in the device's bit-plane layouts)
+    const int64_t groups = ceil_div(pitch, 4 * BITS);
+    pack_kernel<BITS><<<static_cast<unsigned>(ceil_div(N * groups, 256)), 256, 0, st>>>(
+        W, N, K, static_cast<int>(groups), scale, zero, layout, pitch, out);
 }
 
 // One thread per code.
@@ -161,127 +242,6 @@ __global__ void code_sums_kernel(const uint8_t* __restrict__ packed, int64_t K, 
     if (threadIdx.x == 0) sums[blockIdx.x] = part[0] + part[1] + part[2] + part[3];
 }
 
-// Range of a tensor with 0 included: floats ordered through a monotone map to unsigned integers.
-__device__ __forceinline__ unsigned int ordered_bits(float f)
-{
-    const unsigned int u = __float_as_uint(f);
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
-// range_bits[0]: ordered bits of the running minimum, [1]: of the running maximum.
-__global__ void minmax_kernel(const __half* __restrict__ X, int64_t rows, int64_t cols, int64_t row_stride,
-                              unsigned int* __restrict__ range_bits)
-{
-    float lo = 0.f, hi = 0.f;
-    const int64_t chunks_per_row = (cols + 7) / 8;
-    const int64_t total = rows * chunks_per_row;
-    const bool vec_ok = (cols % 8 == 0) && (row_stride % 8 == 0) &&
-                        ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t r = i / chunks_per_row;
-        const int64_t c = (i - r * chunks_per_row) * 8;
-        const __half* p = X + r * row_stride + c;
-        if (vec_ok) {
-            const uint4 v = *reinterpret_cast<const uint4*>(p);
-            const __half2* h = reinterpret_cast<const __half2*>(&v);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = __half22float2(h[j]);
-                lo = fminf(lo, fminf(f.x, f.y));
-                hi = fmaxf(hi, fmaxf(f.x, f.y));
-            }
-        } else {
-            for (int j = 0; j < 8 && c + j < cols; ++j) {
-                const float f = __half2float(p[j]);
-                lo = fminf(lo, f);
-                hi = fmaxf(hi, f);
-            }
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) {
-        lo = fminf(lo, __shfl_xor_sync(0xffffffffu, lo, o));
-        hi = fmaxf(hi, __shfl_xor_sync(0xffffffffu, hi, o));
-    }
-    if ((threadIdx.x & 31) == 0) {
-        if (lo < 0.f) atomicMin(range_bits, ordered_bits(lo));
-        if (hi > 0.f) atomicMax(range_bits + 1, ordered_bits(hi));
-    }
-}
-
-// Both accumulators start at the ordered bits of +0.
-__global__ void minmax_init_kernel(unsigned int* __restrict__ range_bits)
-{
-    range_bits[0] = 0x80000000u;
-    range_bits[1] = 0x80000000u;
-}
-
-// Ordered bits back to the bit patterns of {lo, hi}.
-__global__ void minmax_finish_kernel(unsigned int* __restrict__ range_bits)
-{
-    for (int i = 0; i < 2; ++i) {
-        const unsigned int o = range_bits[i];
-        range_bits[i] = (o & 0x80000000u) ? (o & 0x7fffffffu) : ~o;
-    }
-}
-
-// scale = (hi - lo) / 255, zero = clamp(rne(-lo / scale), 0, 255); an all-zero tensor: scale 1, zero 0.
-__global__ void act_asym_params_kernel(const float* __restrict__ minmax, float* __restrict__ scale_out,
-                                       int32_t* __restrict__ zero_out)
-{
-    const float lo = minmax[0], hi = minmax[1];
-    if (hi == lo) {
-        scale_out[0] = 1.f;
-        zero_out[0] = 0;
-        return;
-    }
-    const float s = __fdiv_rn(__fsub_rn(hi, lo), 255.f);
-    const float inv = __fdiv_rn(1.f, s);
-    // -lo * inv <= 255 * (1 + 2^-22): the magic-number addition rounds the exact product to nearest even
-    const float t = __fmaf_rn(-lo, inv, 12582912.f);
-    int z = static_cast<int>(__float_as_uint(t)) - 0x4B400000;
-    z = z < 0 ? 0 : (z > 255 ? 255 : z);
-    scale_out[0] = s;
-    zero_out[0] = z;
-}
-
-// max |x| as an atomic max on the bit pattern (non-negative floats order like integers).
-__global__ void absmax_kernel(const __half* __restrict__ X, int64_t rows, int64_t cols,
-                              int64_t row_stride, int skip_mod, unsigned int* __restrict__ amax_bits)
-{
-    float m = 0.f;
-    const int64_t chunks_per_row = (cols + 7) / 8;
-    const int64_t total = rows * chunks_per_row;
-    const bool vec_ok = (cols % 8 == 0) && (row_stride % 8 == 0) &&
-                        ((reinterpret_cast<uintptr_t>(X) & 15) == 0);
-    for (int64_t i = blockIdx.x * static_cast<int64_t>(blockDim.x) + threadIdx.x; i < total;
-         i += static_cast<int64_t>(gridDim.x) * blockDim.x) {
-        const int64_t r = i / chunks_per_row;
-        const int64_t c = (i - r * chunks_per_row) * 8;
-        if (skip_mod > 0 && r % skip_mod == 0) continue;
-        const __half* p = X + r * row_stride + c;
-        if (vec_ok) {
-            const uint4 v = *reinterpret_cast<const uint4*>(p);
-            const __half2* h = reinterpret_cast<const __half2*>(&v);
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const float2 f = __half22float2(h[j]);
-                m = fmaxf(m, fmaxf(fabsf(f.x), fabsf(f.y)));
-            }
-        } else {
-            for (int j = 0; j < 8 && c + j < cols; ++j) m = fmaxf(m, fabsf(__half2float(p[j])));
-        }
-    }
-    for (int o = 16; o > 0; o >>= 1) m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0 && m > 0.f) atomicMax(amax_bits, __float_as_uint(m));
-}
-
-__global__ void act_scale_kernel(const float* __restrict__ amax, float* __restrict__ scale_out)
-{
-    const float a = amax[0];
-    scale_out[0] = (a == 0.f) ? 1.f : __fdiv_rn(a, 127.f);
-}
-
 bool width_ok(int bits) { return bits == 2 || bits == 3 || bits == 4 || bits == 8; }
 
 }  // namespace
@@ -292,14 +252,16 @@ using namespace mixdq;
 
 // The layer kernels load a layer's constants (packed weights, scales, zero-points, code sums) before they
 // wait for earlier kernels of the stream, so a kernel that WRITES such constants must be complete, not merely
-// finishing, when the next layer call is enqueued behind it.  The entry points below that produce constants
-// therefore end with this empty kernel: launched plainly, it starts only after everything before it on the
-// stream has completed and its writes are visible, and whatever follows it overlaps nothing but it.
+// finishing, when a layer kernel behind it starts.  The entry points below that produce constants therefore leave a
+// note for the stream, and the library's next kernel on it is launched plainly, without the programmatic overlap
+// (launch_ex).  Where no note can be left, this empty kernel, launched plainly, stands between the two.  (It used to
+// end every one of these calls: two launches and some 3 us of a 10240 x 1280 layer's preparation.)
 __global__ void constants_complete_kernel() {}
 
 static int finish_constants(cudaStream_t st)
 {
     if (cudaGetLastError() != cudaSuccess) return MIXDQ_ERR_CUDA;
+    if (note_constants_written(st)) return MIXDQ_OK;
     constants_complete_kernel<<<1, 32, 0, st>>>();
     return check_launch();
 }
@@ -324,8 +286,12 @@ extern "C" int mixdq_weight_minmax_params(const void* W, int64_t N, int64_t K, i
     if (!W || !scale_out || N <= 0 || K <= 0) return MIXDQ_ERR_INVALID_ARG;
     if (bits < 2 || bits > 8) return MIXDQ_ERR_UNSUPPORTED;
     if (!symmetric && !zero_out) return MIXDQ_ERR_INVALID_ARG;
-    weight_minmax_kernel<<<static_cast<unsigned>(N), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __half*>(W), K, bits, symmetric, scale_out, zero_out);
+    if (K <= kRowWarp)
+        weight_minmax_kernel<32><<<static_cast<unsigned>(ceil_div(N, 8)), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __half*>(W), N, K, bits, symmetric, scale_out, zero_out);
+    else
+        weight_minmax_kernel<256><<<static_cast<unsigned>(N), 256, 0, static_cast<cudaStream_t>(stream)>>>(
+            static_cast<const __half*>(W), N, K, bits, symmetric, scale_out, zero_out);
     return finish_constants(static_cast<cudaStream_t>(stream));
 }
 
@@ -338,10 +304,15 @@ extern "C" int mixdq_pack_weights(const void* W, int64_t N, int64_t K, int bits,
     if (bits <= 3 && !zero) return MIXDQ_ERR_UNSUPPORTED;  // bit-plane codes are unsigned only
     if (reinterpret_cast<uintptr_t>(packed_out) & 15) return MIXDQ_ERR_ALIGNMENT;
     const int64_t pitch = row_pitch_bytes(K, bits, layout);
-    const int64_t words = N * ((pitch + 3) / 4);
-    pack_kernel<<<static_cast<unsigned>(ceil_div(words, 256)), 256, 0, static_cast<cudaStream_t>(stream)>>>(
-        static_cast<const __half*>(W), N, K, bits, scale, zero, layout, pitch,
-        static_cast<uint8_t*>(packed_out));
+    const __half* w = static_cast<const __half*>(W);
+    uint8_t* out = static_cast<uint8_t*>(packed_out);
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    switch (bits) {
+        case 2: launch_pack<2>(w, N, K, scale, zero, layout, pitch, out, st); break;
+        case 3: launch_pack<3>(w, N, K, scale, zero, layout, pitch, out, st); break;
+        case 4: launch_pack<4>(w, N, K, scale, zero, layout, pitch, out, st); break;
+        default: launch_pack<8>(w, N, K, scale, zero, layout, pitch, out, st);
+    }
     return finish_constants(static_cast<cudaStream_t>(stream));
 }
 
@@ -355,53 +326,6 @@ extern "C" int mixdq_unpack_weights(const void* packed, int64_t N, int64_t K, in
     const int64_t pitch = row_pitch_bytes(K, bits, layout);
     unpack_kernel<<<static_cast<unsigned>(ceil_div(N * K, 256)), 256, 0, static_cast<cudaStream_t>(stream)>>>(
         static_cast<const uint8_t*>(packed), N, K, bits, is_signed, layout, pitch, codes_out);
-    return check_launch();
-}
-
-extern "C" int mixdq_act_absmax(const void* X, int64_t rows, int64_t cols, int64_t row_stride,
-                                int skip_rows_mod, float* amax_out, void* stream)
-{
-    if (!X || !amax_out || rows <= 0 || cols <= 0 || row_stride < cols || skip_rows_mod < 0)
-        return MIXDQ_ERR_INVALID_ARG;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    MIXDQ_CUDA_TRY(cudaMemsetAsync(amax_out, 0, sizeof(float), st));
-    const int64_t chunks = rows * ((cols + 7) / 8);
-    const unsigned grid = static_cast<unsigned>(chunks < 256 * 1184 ? ceil_div(chunks, 256) : 1184);
-    absmax_kernel<<<grid, 256, 0, st>>>(static_cast<const __half*>(X), rows, cols, row_stride,
-                                        skip_rows_mod, reinterpret_cast<unsigned int*>(amax_out));
-    return check_launch();
-}
-
-extern "C" int mixdq_act_scale_from_absmax(const float* amax, float* scale_out, void* stream)
-{
-    if (!amax || !scale_out) return MIXDQ_ERR_INVALID_ARG;
-    act_scale_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(amax, scale_out);
-    return check_launch();
-}
-
-extern "C" int mixdq_act_minmax(const void* X, int64_t rows, int64_t cols, int64_t row_stride,
-                                float* minmax_out, void* stream)
-{
-    if (!X || !minmax_out || rows <= 0 || cols <= 0 || row_stride < cols) return MIXDQ_ERR_INVALID_ARG;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
-    unsigned int* bits = reinterpret_cast<unsigned int*>(minmax_out);
-    minmax_init_kernel<<<1, 1, 0, st>>>(bits);
-    int rc = check_launch();
-    if (rc != MIXDQ_OK) return rc;
-    const int64_t chunks = rows * ((cols + 7) / 8);
-    const unsigned grid = static_cast<unsigned>(chunks < 256 * 1184 ? ceil_div(chunks, 256) : 1184);
-    minmax_kernel<<<grid, 256, 0, st>>>(static_cast<const __half*>(X), rows, cols, row_stride, bits);
-    rc = check_launch();
-    if (rc != MIXDQ_OK) return rc;
-    minmax_finish_kernel<<<1, 1, 0, st>>>(bits);
-    return check_launch();
-}
-
-extern "C" int mixdq_act_asym_params_from_minmax(const float* minmax, float* scale_out, int32_t* zero_out,
-                                                 void* stream)
-{
-    if (!minmax || !scale_out || !zero_out) return MIXDQ_ERR_INVALID_ARG;
-    act_asym_params_kernel<<<1, 1, 0, static_cast<cudaStream_t>(stream)>>>(minmax, scale_out, zero_out);
     return check_launch();
 }
 

@@ -1,6 +1,7 @@
 // Tensor-map (TMA descriptor) encoding.  The driver entry point is looked up through the
 // runtime so that the library has no link-time dependency on libcuda and still loads on
 // a machine without a GPU driver.
+#include <atomic>
 #include <mutex>
 #include <unordered_set>
 
@@ -153,37 +154,76 @@ int current_device()
 
 }  // namespace
 
-int prefer_max_shared_carveout(const void* kernel)
+namespace {
+
+// Sets a function attribute once per (device, kernel).
+int set_once(const void* kernel, cudaFuncAttribute attribute, int value, std::mutex& mu, std::unordered_set<const void*> (&done)[kMaxDevices])
 {
-    static std::mutex mu;
-    static std::unordered_set<const void*> done[kMaxDevices];
     const int dev = current_device();
     if (dev < 0) return MIXDQ_ERR_CUDA;
     std::lock_guard<std::mutex> lock(mu);
     if (done[dev].count(kernel)) return MIXDQ_OK;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared) !=
-        cudaSuccess) {
-        (void)cudaGetLastError();
-        return MIXDQ_ERR_CUDA;
-    }
+    MIXDQ_CUDA_TRY(cudaFuncSetAttribute(kernel, attribute, value));
     done[dev].insert(kernel);
     return MIXDQ_OK;
+}
+
+}  // namespace
+
+int prefer_max_shared_carveout(const void* kernel)
+{
+    static std::mutex mu;
+    static std::unordered_set<const void*> done[kMaxDevices];
+    return set_once(kernel, cudaFuncAttributePreferredSharedMemoryCarveout, cudaSharedmemCarveoutMaxShared, mu, done);
 }
 
 int ensure_dynamic_smem(const void* kernel, int bytes)
 {
     static std::mutex mu;
     static std::unordered_set<const void*> done[kMaxDevices];
-    const int dev = current_device();
-    if (dev < 0) return MIXDQ_ERR_CUDA;
-    std::lock_guard<std::mutex> lock(mu);
-    if (done[dev].count(kernel)) return MIXDQ_OK;
-    if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes) != cudaSuccess) {
-        (void)cudaGetLastError();
-        return MIXDQ_ERR_CUDA;
-    }
-    done[dev].insert(kernel);
-    return MIXDQ_OK;
+    return set_once(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes, mu, done);
+}
+
+int allow_large_clusters(const void* kernel)
+{
+    static std::mutex mu;
+    static std::unordered_set<const void*> done[kMaxDevices];
+    return set_once(kernel, cudaFuncAttributeNonPortableClusterSizeAllowed, 1, mu, done);
+}
+
+namespace {
+
+constexpr size_t kMaxNotes = 64;
+std::mutex g_notes_mutex;
+cudaStream_t g_notes[kMaxNotes];
+std::atomic<size_t> g_note_count{0};  // read without the lock by every launch
+
+}  // namespace
+
+bool note_constants_written(cudaStream_t stream)
+{
+    std::lock_guard<std::mutex> lock(g_notes_mutex);
+    const size_t n = g_note_count.load(std::memory_order_relaxed);
+    for (size_t i = 0; i < n; ++i)
+        if (g_notes[i] == stream) return true;
+    if (n == kMaxNotes) return false;
+    g_notes[n] = stream;
+    g_note_count.store(n + 1, std::memory_order_release);
+    return true;
+}
+
+bool take_constants_note(cudaStream_t stream)
+{
+    if (g_note_count.load(std::memory_order_acquire) == 0) return false;
+    std::lock_guard<std::mutex> lock(g_notes_mutex);
+    const size_t n = g_note_count.load(std::memory_order_relaxed);
+    for (size_t i = 0; i < n; ++i)
+        if (g_notes[i] == stream) {
+            g_notes[i] = g_notes[n - 1];
+            g_note_count.store(n - 1, std::memory_order_release);
+            return true;
+        }
+    return false;
 }
 
 int sm_count()

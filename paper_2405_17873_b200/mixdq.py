@@ -37,6 +37,8 @@ _SIGNATURES = {
     "mixdq_unpack_weights": (_int, [_vp, _i64, _i64, _int, _int, _int, _vp, _vp]),
     "mixdq_act_absmax": (_int, [_vp, _i64, _i64, _i64, _int, _vp, _vp]),
     "mixdq_act_scale_from_absmax": (_int, [_vp, _vp, _vp]),
+    "mixdq_act_scale": (_int, [_vp, _i64, _i64, _i64, _int, _vp, _vp]),
+    "mixdq_act_asym_params": (_int, [_vp, _i64, _i64, _i64, _vp, _vp, _vp]),
     "mixdq_act_minmax": (_int, [_vp, _i64, _i64, _i64, _vp, _vp]),
     "mixdq_act_asym_params_from_minmax": (_int, [_vp, _vp, _vp, _vp]),
     "mixdq_weight_code_sums": (_int, [_vp, _i64, _i64, _int, _vp, _vp]),
