@@ -359,6 +359,15 @@ def _fracs(rate, measured, nominal, probe=None):
     return d
 
 
+def _tile_name(M, N, k_blocks, bits):
+    from paper_2405_17873_b200 import mixdq
+    channels, tokens = mixdq.int8_chan_tile(M, N, k_blocks, bits)
+    if tokens:
+        return f"{channels} channels x {tokens} tokens"
+    rows, cols, sp = mixdq.int8_tile_plan(M, N, k_blocks, bits, with_splits=True)
+    return f"{rows}x{cols}" + (f", reduction over {sp} CTA pairs" if sp > 1 else "")
+
+
 def config_records(torch, mixdq, synth, stream, peaks, probe_int8):
     """One record per stated configuration besides the layer sweep: the single W8A8 linear layer, the weight-only
     trio at 4096 and 16 tokens, the FFN pair in W4A8 / W8A8 at image batch 1 and 4, the BOS-aware K / V
@@ -381,10 +390,10 @@ def config_records(torch, mixdq, synth, stream, peaks, probe_int8):
         bd = None if b is None else dev(b)
         us = _time_graph(torch, stream, lambda: mixdq.linear(Xd, pk, N, bits, s, None, 8, sx, bd, ws, status, out=Y))
         tops = 2.0 * M * N * K / us / 1e6
-        rows, cols, sp = mixdq.int8_tile_plan(M, N, (K + 127) // 128, bits, with_splits=True)
+        tile = _tile_name(M, N, (K + 127) // 128, bits)
         out.append({"config": tag, "M": M, "N": N, "K": K, "w_bits": bits, "a_bits": 8, "us": round(us, 2),
                     "tops": round(tops, 1), "bound": "tensor", "l2": "warm",
-                    "tile": f"{rows}x{cols}" + (f", reduction over {sp} CTA pairs" if sp > 1 else ""),
+                    "tile": tile,
                     "frac": _fracs(tops, int8_peak, NOMINAL["int8_tops"], probe_int8)})
 
     # 1. single linear layer, W8A8
@@ -739,10 +748,9 @@ def run_ours(args):
             us = t0.elapsed_time(t1) * 1e3 / (reps * rounds)
             tops = pl.spec.ops(args.batch) / us / 1e6
             kb = 9 * ((pl.spec.Cin + 127) // 128) if pl.spec.kind == "conv3x3" else (pl.spec.K + 127) // 128
-            rows, cols, sp = mixdq.int8_tile_plan(pl.spec.rows(args.batch), pl.spec.N, kb, pl.spec.w_bits, with_splits=True)
             per_layer.append({"layer": name, "kind": pl.spec.kind, "M": pl.spec.rows(args.batch), "N": pl.spec.N,
                               "K": pl.spec.K, "w_bits": pl.spec.w_bits,
-                              "tile": f"{rows}x{cols}" + (f", reduction over {sp} CTA pairs" if sp > 1 else ""),
+                              "tile": _tile_name(pl.spec.rows(args.batch), pl.spec.N, kb, pl.spec.w_bits),
                               "us": round(us, 2),
                               "tops": round(tops, 1), "frac_of_burst_peak": round(tops / burst, 3),
                               "frac_of_sustained_peak": round(tops / (peaks["bf16_tflops_sustained"] * INT8_TO_BF16_NOMINAL), 3),

@@ -66,16 +66,24 @@ unsigned long long mixdq_kernel_launches(void);
  * a long reduction, partial sums added through distributed shared memory); 0 for 128-row tiles.  A linear layer for
  * which mixdq_linear_fused_quant_tile is positive runs as one kernel on 128-row tiles of that width instead, and a
  * shortcut-split layer (mixdq_linear_a8_split, mixdq_conv3x3_a8_split) takes the 256-row tiles reported for the sum of
- * its branches' reduction blocks, without a split reduction, or else 128-row tiles.  For tests and benchmarks: nothing
- * is launched. */
+ * its branches' reduction blocks, without a split reduction, or else 128-row tiles.  Other than those two, a layer for
+ * which mixdq_int8_chan_tile reports a tile takes that one instead.  For tests and benchmarks: nothing is launched. */
 int mixdq_int8_tile_plan(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int* tile_rows, int* tile_cols,
                          int* reduction_splits);
+
+/* Diagnostic (the paper has no counterpart): the tile of the channel-major form (output channels on the rows of the
+ * tensor-core tile), which runs layers whose tiles fit the SMs at once: *tile_channels is 128, or 256 when two CTAs
+ * share a tile, *tile_tokens a multiple of 16 per CTA; both 0 where the tiles of mixdq_int8_tile_plan are faster.
+ * Arguments as there.  Taken with a workspace by every int8 layer but the second branch of a shortcut-split layer.
+ * Nothing is launched. */
+int mixdq_int8_chan_tile(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int* tile_channels, int* tile_tokens);
 
 /* Diagnostic (the paper has no counterpart; its implementation runs the activation quantization as a kernel of
  * its own, Sec. 4.1 "Hardware Profiling"): width of the 128-row output tiles when mixdq_linear, called with a
  * workspace, 8-bit symmetric activations and a row-major X, runs a layer of M rows, N channels and K inputs as ONE
  * kernel that quantizes its activation tiles itself; 0 when the layer runs as quantization pass + GEMM (the
- * one-kernel form pays only for short reductions, K <= 640, on one wave of tiles).  Negative: an error code.
+ * one-kernel form pays only for short reductions, K <= 640, on one wave of tiles).  Below 2048 rows a layer for which
+ * mixdq_int8_chan_tile reports a tile runs as two kernels all the same.  Negative: an error code.
  * For tests and benchmarks: nothing is launched. */
 int mixdq_linear_fused_quant_tile(int64_t M, int64_t N, int64_t K, int w_bits);
 

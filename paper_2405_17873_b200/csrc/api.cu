@@ -204,6 +204,20 @@ extern "C" int mixdq_int8_tile_plan(int64_t M, int64_t N, int64_t k_blocks, int 
     return MIXDQ_OK;
 }
 
+extern "C" int mixdq_int8_chan_tile(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int* tile_channels, int* tile_tokens)
+{
+    if (!tile_channels || !tile_tokens || M <= 0 || N <= 0 || k_blocks <= 0 || M > 0x7fffffff || N > 0x7fffffff ||
+        k_blocks > 0x7fffffff)
+        return MIXDQ_ERR_INVALID_ARG;
+    if (w_bits != 4 && w_bits != 8) return MIXDQ_ERR_UNSUPPORTED;
+    const int sms = sm_count();
+    if (sms <= 0) return MIXDQ_ERR_CUDA;
+    int cg = 1;
+    *tile_tokens = i8::plan_chan_tile(static_cast<int>(M), static_cast<int>(N), static_cast<int>(k_blocks), w_bits == 4, sms, &cg);
+    *tile_channels = *tile_tokens > 0 ? 128 * cg : 0;
+    return MIXDQ_OK;
+}
+
 extern "C" int mixdq_linear_fused_quant_tile(int64_t M, int64_t N, int64_t K, int w_bits)
 {
     if (M <= 0 || N <= 0 || K <= 0 || M > 0x7fffffff || N > 0x7fffffff || K > 0x7fffffff) return MIXDQ_ERR_INVALID_ARG;

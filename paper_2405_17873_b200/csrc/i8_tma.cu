@@ -1135,63 +1135,119 @@ int pick_splits(int64_t tiles, int k_blocks, int num_sms)
 
 }  // namespace
 
-// Which kernel form runs an int8 GEMM of M x N over k_blocks k-blocks: 0 = the single-CTA kernels of this file,
-// otherwise the tile width of the pair form.  Both are estimated in SM cycles from a model whose constants were
-// fitted to timings of every layer shape of the SDXL-turbo-shaped UNet at image batch 1 and 4 on a B200 (each
-// form at each width): rounds of tiles over the SMs (or SM pairs) times the cost of a tile -- the larger of its
-// main loop, a per-k-block cost that grows with the tile width, and its epilogue -- plus fixed costs.
-int plan_pair_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* splits)
+// The kernel forms with the tokens on the rows, estimated in SM cycles from a model whose constants were fitted to
+// timings of every layer shape of the SDXL-turbo-shaped UNet at image batch 1 and 4 on a B200 (each form at each
+// width): rounds of tiles over the SMs (or SM pairs) times the cost of a tile -- the larger of its main loop, a
+// per-k-block cost that grows with the tile width, and its epilogue -- plus fixed costs.
+namespace {
+
+struct TokenPlan {
+    double pair_cost = 0;      // best pair form (i8_pair.cu); no such form for fewer than 256 rows: pair_bn = 0
+    int pair_bn = 0, pair_splits = 1;
+    double single_cost = 0;    // single-CTA kernels of this file
+    int single_splits = 1;
+};
+
+TokenPlan token_plan(int M, int N, int k_blocks, bool w4, int num_sms, bool allow_splits)
 {
-    if (splits) *splits = 1;
-    if (M < 2 * BM || num_sms < 2) return 0;
+    TokenPlan r;
     const double nkb = k_blocks;
-    const int pairs = num_sms / 2;
-    // pair form: 256 x bn tiles, widths below 160 never paid off
-    double best = 0;
-    int best_bn = 0, best_splits = 1;
-    for (int bn = 160; bn <= 256; bn += 32) {
-        const int64_t tiles = ceil_div(M, 2 * BM) * ceil_div(N, bn);
-        const double per_kb = w4 ? 350.0 + 1.4 * bn : 250.0 + 1.2 * bn;
-        const double rounds = std::ceil(static_cast<double>(tiles) / pairs);
-        const double t = rounds * (std::max(nkb * per_kb, 30.0 * bn) + 800.0) + 16.0 * bn + 5000.0;
-        if (best_bn == 0 || t < best) {
-            best = t;
-            best_bn = bn;
-            best_splits = 1;
-        }
-        // few tiles, long reduction: one tile per cluster, the reduction split over up to four pairs; the
-        // partial tiles meet through distributed shared memory at a fixed cost of some 14 000 cycles
-        // (a cluster sits inside one GPC: the device holds fewer clusters of 4, 6 or 8 CTAs than SMs / size)
-        for (int sp = 2; sp <= 4 && splits && tiles * sp <= pairs && k_blocks / sp >= 8; ++sp) {
-            if (tiles > pair_cluster_capacity(w4, 2 * sp)) continue;
-            const double ts = std::ceil(nkb / sp) * per_kb + 16.0 * bn + 14000.0 + 5000.0;
-            if (ts < best) {
-                best = ts;
-                best_bn = bn;
-                best_splits = sp;
+    if (M >= 2 * BM && num_sms >= 2) {
+        const int pairs = num_sms / 2;
+        // pair form: 256 x bn tiles, widths below 160 never paid off
+        for (int bn = 160; bn <= 256; bn += 32) {
+            const int64_t tiles = ceil_div(M, 2 * BM) * ceil_div(N, bn);
+            const double per_kb = w4 ? 350.0 + 1.4 * bn : 250.0 + 1.2 * bn;
+            const double rounds = std::ceil(static_cast<double>(tiles) / pairs);
+            const double t = rounds * (std::max(nkb * per_kb, 30.0 * bn) + 800.0) + 16.0 * bn + 5000.0;
+            if (r.pair_bn == 0 || t < r.pair_cost) {
+                r.pair_cost = t;
+                r.pair_bn = bn;
+                r.pair_splits = 1;
+            }
+            // few tiles, long reduction: one tile per cluster, the reduction split over up to four pairs; the
+            // partial tiles meet through distributed shared memory at a fixed cost of some 14 000 cycles
+            // (a cluster sits inside one GPC: the device holds fewer clusters of 4, 6 or 8 CTAs than SMs / size)
+            for (int sp = 2; sp <= 4 && allow_splits && tiles * sp <= pairs && k_blocks / sp >= 8; ++sp) {
+                if (tiles > pair_cluster_capacity(w4, 2 * sp)) continue;
+                const double ts = std::ceil(nkb / sp) * per_kb + 16.0 * bn + 14000.0 + 5000.0;
+                if (ts < r.pair_cost) {
+                    r.pair_cost = ts;
+                    r.pair_bn = bn;
+                    r.pair_splits = sp;
+                }
             }
         }
     }
     // single-CTA kernels: 128 x 128 tiles (128 x 256 for wide int8 layers), persistent once the tiles cover the
     // SMs, else one tile per CTA with the reduction split over a cluster
-    double old;
     const double c = w4 ? 580.0 : 420.0;
     const bool wide = !w4 && (N >= 1024 || N % 256 == 0) && ceil_div(M, BM) * ceil_div(N, 256) >= 100;
     if (wide) {
         const double tiles = static_cast<double>(ceil_div(M, BM) * ceil_div(N, 256));
-        old = std::ceil(tiles / num_sms) * std::max(nkb * 620.0, 10000.0) + 3000.0;
+        r.single_cost = std::ceil(tiles / num_sms) * std::max(nkb * 620.0, 10000.0) + 3000.0;
     } else {
         const int64_t tiles = ceil_div(M, BM) * ceil_div(N, 128);
         if (tiles >= num_sms) {
-            old = std::ceil(static_cast<double>(tiles) / num_sms) * std::max(nkb * c, 5000.0) + 3000.0;
+            r.single_cost = std::ceil(static_cast<double>(tiles) / num_sms) * std::max(nkb * c, 5000.0) + 3000.0;
         } else {
-            const int s = pick_splits(tiles, k_blocks, num_sms);
-            old = std::ceil(nkb / s) * c + 3000.0 + 3000.0 + (s > 1 ? 2500.0 : 0.0);
+            r.single_splits = pick_splits(tiles, k_blocks, num_sms);
+            r.single_cost = std::ceil(nkb / r.single_splits) * c + 3000.0 + 3000.0 + (r.single_splits > 1 ? 2500.0 : 0.0);
         }
     }
-    if (best >= 1.05 * old) return 0;
-    if (splits) *splits = best_splits;
-    return best_bn;
+    return r;
+}
+
+}  // namespace
+
+// Tile width of the pair form, or 0 for the single-CTA kernels.
+int plan_pair_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* splits)
+{
+    const TokenPlan t = token_plan(M, N, k_blocks, w4, num_sms, splits != nullptr);
+    if (splits) *splits = 1;
+    if (t.pair_bn == 0 || t.pair_cost >= 1.05 * t.single_cost) return 0;
+    if (splits) *splits = t.pair_splits;
+    return t.pair_bn;
+}
+
+// Channel-major form (i8_chan.cu): its tile's tokens, or 0 where the forms with the tokens on the rows are faster.  The
+// kernel runs one tile per CTA or CTA pair, so the tiles have to fit the SMs at once; a second wave costs more than the
+// form gains (4096 x 1280 x 640 int4: 11.3 us against 10.1).  Cycles of a tile of t tokens, from a fit to 104 layers (16 to
+// 16384 rows, 320 to 2560 channels, 3 to 180 k-blocks, linear and convolution; every tile that fits one wave; mean error
+// 6 per cent): fixed part + k-blocks x (issue + t) + epilogue of the tokens, where the share of the SMs in use slows each
+// k-block (they compete for the L2) and the start.  Chosen by it, the 104 layers ran within 2.2 per cent of each one's best
+// form and tile.
+//   * One CTA below 48 tokens or pairs below 64 never were the best (but for layers of so few rows).
+//   * int8 weights on pairs of more than 192 tokens leave room for four activation slots only: half the speed.
+//   * The single-CTA kernels' split reductions measured 5000 cycles over their estimate, the pair form's ten per cent under.
+int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg)
+{
+    const double nkb = k_blocks;
+    double best = 0;
+    int best_tokens = 0;
+    for (int c = 1; c <= 2; ++c) {
+        const int64_t c_tiles = ceil_div(N, 128 * c);
+        for (int t = 16 * c; t <= (c == 2 && !w4 ? 192 : 128 * c); t += 16 * c) {
+            if (t < 32 * c && M > 64) continue;
+            if (t >= M + 16 * c) break;  // (nothing but padding more than the tile before)
+            const int64_t ctas = c * c_tiles * ceil_div(M, t);
+            if (ctas > num_sms) continue;
+            const double busy = static_cast<double>(ctas) / num_sms;
+            const double cost = (w4 ? 3400.0 : 3700.0) + nkb * ((c == 1 ? (w4 ? 207.0 : 182.0) : (w4 ? 145.0 : 160.0)) + 1.1 * t + 92.0 * busy) +
+                                16.0 * t + (c == 1 ? 1270.0 : 3100.0) * busy;
+            if (best_tokens == 0 || cost < best) {
+                best = cost;
+                best_tokens = t;
+                *cg = c;
+            }
+        }
+    }
+    if (best_tokens == 0) return 0;
+    const TokenPlan o = token_plan(M, N, k_blocks, w4, num_sms, true);
+    const double single = o.single_cost + (o.single_splits > 1 ? 5000.0 : 0.0);
+    const bool pair = o.pair_bn > 0 && o.pair_cost < 1.05 * single;
+    const double other = pair ? o.pair_cost * (o.pair_splits > 1 ? 0.9 : 1.0) : single;
+    return best < other ? best_tokens : 0;
 }
 
 // Fused-quantization kernel (i8_fq.cu) or the two-kernel forms.  The fused kernel's k-block costs three to four
@@ -1311,8 +1367,14 @@ int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* sc
     int8_t* aq = static_cast<int8_t*>(scratch);
     if (amode == A_LINEAR && !p.act_zero && !p.addend && !p.test_drop_b_kblock) {
         const int num_sms = sm_count();
-        const int fq_bn = num_sms > 0 ? plan_fq_tile(p.M, p.N, static_cast<int>(ceil_div(p.K, BK)), w_bits == 4, num_sms) : 0;
-        if (fq_bn > 0) return run_fq(p, packed, w_bits, fq_bn, stream);
+        const int kb = static_cast<int>(ceil_div(p.K, BK));
+        const int fq_bn = num_sms > 0 ? plan_fq_tile(p.M, p.N, kb, w_bits == 4, num_sms) : 0;
+        // Below 2048 rows the quantization pass is short (1.7 us for 1024 x 640) and the channel-major GEMM after it makes
+        // up for it: 1024 x 640 x 640 W4 5.2 us against 8.2, W8 5.4 against 6.6.  From there on they come out equal (4096 x
+        // 640 x 640 W4: 9.2 and 9.3 us) or the fused kernel ahead (W8 9.2 and 7.5, K = 320 8.0 and 7.1).
+        int cg;
+        if (fq_bn > 0 && (p.M >= 2048 || plan_chan_tile(p.M, p.N, kb, w_bits == 4, num_sms, &cg) == 0))
+            return run_fq(p, packed, w_bits, fq_bn, stream);
     }
 
     // 1. quantize the activations once
@@ -1340,6 +1402,14 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
     const bool conv = amode == A_CONV3;
     const int pad = (conv && p.act_zero) ? 1 : 0;
     int rc;
+    const int num_sms = sm_count();
+    if (num_sms <= 0) return MIXDQ_ERR_CUDA;
+    if (!p.addend && !p.test_drop_b_kblock) {
+        int cg = 1;
+        const int kb = static_cast<int>(conv ? 9 * ceil_div(p.Cin, BK) : ceil_div(p.K, BK));
+        const int tokens = plan_chan_tile(p.M, p.N, kb, w4, num_sms, &cg);
+        if (tokens > 0) return run_chan(p, amode, packed, w_bits, aq, cg, tokens, stream);
+    }
 
     // 2. tensor maps
     CUtensorMap ta, tw, ty{};
@@ -1395,8 +1465,6 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
         tp.k_blocks = static_cast<int>(ceil_div(p.K, BK));
     }
     if (rc != MIXDQ_OK) return rc;
-    const int num_sms = sm_count();
-    if (num_sms <= 0) return MIXDQ_ERR_CUDA;
     // the pair form (two-CTA tiles of 256 x bn, i8_pair.cu) where its estimate beats the single-CTA kernels
     int pair_splits = 1;
     const int pair_bn = (!p.addend && amode != A_BOS && !p.test_drop_b_kblock)

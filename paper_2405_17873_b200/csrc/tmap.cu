@@ -44,7 +44,7 @@ EncodeIm2colFn get_encode_im2col_fn()
 }  // namespace
 
 int encode_tmap_2d_u8(CUtensorMap* map, const void* base, uint64_t row_bytes, uint64_t rows,
-                      uint64_t pitch_bytes, uint32_t box_bytes, uint32_t box_rows, bool swizzle128)
+                      uint64_t pitch_bytes, uint32_t box_bytes, uint32_t box_rows, int swizzle)
 {
     EncodeTiledFn fn = get_encode_fn();
     if (!fn) return MIXDQ_ERR_CUDA;
@@ -55,7 +55,8 @@ int encode_tmap_2d_u8(CUtensorMap* map, const void* base, uint64_t row_bytes, ui
     cuuint32_t estr[2] = {1, 1};
     CUresult r = fn(map, CU_TENSOR_MAP_DATA_TYPE_UINT8, 2, const_cast<void*>(base), dims, strides, box, estr,
                     CU_TENSOR_MAP_INTERLEAVE_NONE,
-                    swizzle128 ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE,
+                    swizzle == SWIZZLE_128 ? CU_TENSOR_MAP_SWIZZLE_128B
+                                           : (swizzle == SWIZZLE_64 ? CU_TENSOR_MAP_SWIZZLE_64B : CU_TENSOR_MAP_SWIZZLE_NONE),
                     CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
     return r == CUDA_SUCCESS ? MIXDQ_OK : MIXDQ_ERR_CUDA;
 }

@@ -30,6 +30,7 @@ _SIGNATURES = {
     "mixdq_strerror": (C.c_char_p, [_int]),
     "mixdq_kernel_launches": (C.c_ulonglong, []),
     "mixdq_int8_tile_plan": (_int, [_i64, _i64, _i64, _int, C.POINTER(_int), C.POINTER(_int), C.POINTER(_int)]),
+    "mixdq_int8_chan_tile": (_int, [_i64, _i64, _i64, _int, C.POINTER(_int), C.POINTER(_int)]),
     "mixdq_linear_fused_quant_tile": (_int, [_i64, _i64, _i64, _int]),
     "mixdq_packed_bytes": (_int, [_i64, _i64, _int, _int, C.POINTER(_sz)]),
     "mixdq_weight_minmax_params": (_int, [_vp, _i64, _i64, _int, _int, _vp, _vp, _vp]),
@@ -159,6 +160,13 @@ def int8_tile_plan(M: int, N: int, k_blocks: int, w_bits: int, with_splits: bool
     r, c, sp = _int(0), _int(0), _int(0)
     _chk(lib().mixdq_int8_tile_plan(M, N, k_blocks, w_bits, C.byref(r), C.byref(c), C.byref(sp)), "mixdq_int8_tile_plan")
     return (r.value, c.value, sp.value) if with_splits else (r.value, c.value)
+
+
+def int8_chan_tile(M: int, N: int, k_blocks: int, w_bits: int):
+    """(channels, tokens) of the channel-major tile that runs this shape ahead of int8_tile_plan's, (0, 0) for none."""
+    c, t = _int(0), _int(0)
+    _chk(lib().mixdq_int8_chan_tile(M, N, k_blocks, w_bits, C.byref(c), C.byref(t)), "mixdq_int8_chan_tile")
+    return c.value, t.value
 
 
 def linear_fused_quant_tile(M: int, N: int, K: int, w_bits: int) -> int:
