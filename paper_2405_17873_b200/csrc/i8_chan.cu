@@ -21,9 +21,11 @@
 // filter tap).
 //
 // Measured on B200, GEMM alone in a chain of launches, against the forms with tokens on the rows: W4 1024 x 1280 x 1280 5.0
-// us (6.5), 1024 x 1280 x 5120 9.9 (14.7), 256 x 1280 x 1280 3.5 (7.0), 616 x 1280 x 2048 5.1 (8.8), 4096 x 640 x 640 6.4
-// (7.9), 3x3 convolution 48 x 48 x 640 -> 640 11.9 (16.7), 4 x 16 x 16 x 640 -> 1280 11.6 (16.9); W8 5.1 (5.6), 10.1 (11.9),
-// 3.8 (6.7), 5.4 (8.3), 6.3 (6.5), 11.9 (15.3), 11.6 (15.4).
+// us (6.5), 1024 x 1280 x 5120 9.5 (14.7), 256 x 1280 x 1280 3.5 (7.0), 616 x 1280 x 2048 5.1 (8.8), 4096 x 640 x 640 6.3
+// (7.9), 3x3 convolution 48 x 48 x 640 -> 640 10.6 (16.7), 4 x 16 x 16 x 640 -> 1280 10.3 (16.9); W8 5.2 (5.6), 10.0 (11.9),
+// 3.9 (6.7), 5.5 (8.3), 6.3 (6.5), 11.4 (15.3), 10.8 (15.4).  A long reduction takes 270 cycles per k-block of 128 channels x
+// 80 tokens, of which the tensor pipe is busy 160: two issuers, each some 1000 cycles per pair (wait 150, eight MMAs and a
+// commit 450, the loop), and two activation producers of about the same are the next limits; four of either gained nothing.
 //
 // Epilogue: a thread owns a channel, so scale and bias live in two registers; neighbouring lanes swap halves of a packed
 // token pair and store channel pairs, 64 contiguous bytes of an output row per warp -- no staging tile.
@@ -41,7 +43,9 @@ namespace {
 constexpr int CH = 128;        // channels of one CTA
 constexpr int TOK_MAX = 256;   // tokens of a tile
 constexpr int ROWS_MAX = 128;  // token rows of one CTA
-constexpr int THREADS = 576;
+constexpr int EXP_GROUPS = 3;  // of four warps: expansion (W4), then epilogue
+constexpr int WORKERS = 4 * EXP_GROUPS, WORK0 = 4, HELP0 = WORK0 + WORKERS;
+constexpr int THREADS = (HELP0 + 2) * 32;
 constexpr int SMEM_MAX = 232448;
 
 // Warps: 0 MMA issuer and tensor-memory allocation, 1 and 16 weight producers, 2 and 17 activation producers, 3 barrier
@@ -49,8 +53,7 @@ constexpr int SMEM_MAX = 232448;
 template <int CG, bool W4>
 struct Chan {
     static constexpr int W_BYTES = CH * BK;        // int8 weight rows of a k-block (W8)
-    static constexpr int P_BYTES = CH * BK / 2;    // packed int4 weight rows
-    static constexpr int EXP_GROUPS = 3;
+    static constexpr int P_BYTES = CH * BK;        // packed int4 weight rows of two k-blocks
     static constexpr int ISSUERS = 2;
     // k-blocks go through in pairs: one barrier says that a pair's tiles are in place, one commit that its MMAs have
     // finished, which frees the pair's slots of all rings.  Ring depths in k-blocks; run-time ones: activation slots, and
@@ -58,9 +61,9 @@ struct Chan {
     static constexpr int NE = 6;                   // pairs whose barriers exist at a time: at least the deepest ring
     static constexpr int XS_MAX = 2 * NE;
     static constexpr int WS_MAX = W4 ? 12 : 8;
-    static constexpr int PS = W4 ? 12 : 0;
-    static_assert(NE % EXP_GROUPS == 0 && PS % EXP_GROUPS == 0 && NE % 2 == 0 && PS % 2 == 0,
-                  "a waiter must meet every phase of the barriers it waits on");
+    static constexpr int PS = W4 ? 6 : 0;          // packed rows: slots of a pair each
+    // (a waiter must meet every phase of the barriers it waits on: expansion groups those of every third pair)
+    static_assert(NE % EXP_GROUPS == 0 && PS % EXP_GROUPS == 0 && PS <= NE, "barriers and groups");
     static constexpr int OFF_W = 0;
     static constexpr int RING_W = W4 ? PS * P_BYTES : WS_MAX * W_BYTES;
     static constexpr int READY = 0;                   // leader: the pair's token rows and weights of both CTAs are in place
@@ -73,7 +76,6 @@ struct Chan {
     static constexpr int OFF_BARS = RING_W;
     static constexpr int OFF_MISC = OFF_BARS + NUM_BARS * 8;
     static constexpr int OFF_X = (OFF_MISC + 16 + 1023) & ~1023;
-    static constexpr int WORK0 = 4;
 };
 
 struct ChanArgs {
@@ -81,6 +83,7 @@ struct ChanArgs {
     int c_tiles;   // channel tiles (128 CG channels each)
     int x_slots, w_slots;
     int a_col;     // W4: first tensor-memory column of the expanded weights
+    int wide;      // W4: a pair's packed rows are contiguous in memory and arrive as 128-byte rows
 };
 
 // A load that stays where it is written (the compiler moves plain read-only loads down to their first use, past the
@@ -118,37 +121,56 @@ __device__ __forceinline__ bool wait_mmas(uint32_t bar0, int was, volatile int* 
     return mbar_wait(bar0 + 8 * (L::EMPTY + q % L::NE), (q / L::NE) & 1, abort_flag);
 }
 
-// A TMA producer, one of two warps that take alternate units (pairs of k-blocks, or packed k-blocks); request(slot, barrier,
-// unit) asks for one.  A warp that runs alone takes some five cycles per instruction, so a loop over k-blocks costs 370
-// cycles a turn whatever the size of the request.  Hence the two warps, and the first lap of the ring, which waits for
-// nothing, goes out from all lanes of the first of them at once (65 cycles apart).  free[unit % barriers] says that the
-// slot of the unit `slots` positions later is free; `barriers` is even and at least `slots`: a warp meets every phase.
-template <typename F>
-__device__ __forceinline__ void produce(int which, int lane, int slots, int units, uint32_t free, int barriers, volatile int* abort_flag,
-                                        F&& request)
-{
-    if (which == 0 && lane < slots && lane < units) request(lane, lane, lane);
-    __syncwarp();
-    if (lane == 0) {
-        int s = which, q = which, sb = which + slots;
-        if (s >= slots) s -= slots;
-        if (sb >= barriers) sb -= barriers;
-        uint32_t par = 0;
-        for (int i = slots + which; i < units; i += 2) {
-            if (!mbar_wait(free + 8 * q, par, abort_flag)) break;
-            request(s, sb, i);
-            s += 2;
-            while (s >= slots) s -= slots;
-            sb += 2;
-            if (sb >= barriers) sb -= barriers;
-            q += 2;
-            if (q >= barriers) {
-                q -= barriers;
-                par ^= 1;
-            }
+// Where a k-block lies: reduction elements [c * BK, ...) of filter tap `tap` (a linear layer is one endless tap).
+struct KPos {
+    int tap, c;
+    __device__ __forceinline__ KPos(int i, int cblocks) : tap(0), c(i)
+    {
+        if (i >= cblocks) {  // (not for a linear layer: a division takes 120 cycles of the first request's way)
+            tap = i / cblocks;
+            c = i - tap * cblocks;
         }
     }
+    __device__ __forceinline__ void advance(int n, int cblocks)
+    {
+        for (c += n; c >= cblocks; c -= cblocks) ++tap;
+    }
+};
+
+// A TMA producer, one of two warps that take alternate units, pairs of k-blocks; request(slot, barrier, unit,
+// position) asks for one.  A warp that runs alone takes some five cycles per instruction, so a
+// loop over k-blocks costs 370 cycles a turn whatever the size of the request, and an integer division in it 120 more.
+// Hence the two warps and the running position, and the first lap of the ring, which waits for nothing, goes out from all
+// lanes of the first of them at once (65 cycles apart).  free[unit % barriers] says that the slot of the unit `slots`
+// positions later is free; `barriers` is even and at least `slots`: a warp meets every phase.
+template <typename F>
+__device__ __forceinline__ void produce(int which, int lane, int slots, int units, int cblocks, uint32_t free, int barriers,
+                                        volatile int* abort_flag, F&& request)
+{
+    if (which == 0 && lane < slots && lane < units) request(lane, lane, lane, KPos(2 * lane, cblocks));
     __syncwarp();
+    if (slots + which >= units) return;
+    int s = which, q = which, sb = which + slots;
+    if (s >= slots) s -= slots;
+    if (sb >= barriers) sb -= barriers;
+    uint32_t par = 0;
+    KPos at(2 * (slots + which), cblocks);
+    for (int i = slots + which; i < units; i += 2) {
+        const bool ok = mbar_wait(free + 8 * q, par, abort_flag);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        if (elect_one()) request(s, sb, i, at);
+        __syncwarp();
+        at.advance(4, cblocks);
+        s += 2;
+        while (s >= slots) s -= slots;
+        sb += 2;
+        if (sb >= barriers) sb -= barriers;
+        q += 2;
+        if (q >= barriers) {
+            q -= barriers;
+            par ^= 1;
+        }
+    }
 }
 
 // One warp's share of the epilogue: its 32 lanes' channels x every third group of eight tokens.  Lanes 2 i and 2 i + 1 swap
@@ -159,7 +181,7 @@ __device__ __forceinline__ void store_tokens(uint32_t acc, int c0, int cols, flo
 {
     const uint32_t sel = (lane & 1) ? 0x3276u : 0x5410u;  // odd: token 1 (other's, own); even: token 0 (own, other's)
     const bool all_n = __all_sync(0xffffffffu, in_n);
-    for (; c0 < cols; c0 += 24) {
+    for (; c0 < cols; c0 += 8 * EXP_GROUPS) {
         uint32_t r[8], own[4], out[4];
         tmem_ld_32x8(acc + c0, r);
         tmem_ld_wait();
@@ -215,7 +237,7 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     pdl_launch_dependents();
     if (warp == 3 && lane == 0) {
         for (int s = 0; s < L::NE; ++s) {
-            mbar_init(bar0 + 8 * (L::READY + s), 1 + (W4 ? CG * 8 : 1));  // activation bytes; weight bytes or expansion warps
+            mbar_init(bar0 + 8 * (L::READY + s), 1 + (W4 ? CG * 4 : 1));  // activation bytes; weight bytes or expansion warps
             mbar_init(bar0 + 8 * (L::EMPTY + s), 1);
         }
         for (int s = 0; s < L::PS; ++s) {
@@ -247,8 +269,8 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     constexpr uint32_t tmem_base = 0;
     if (*s_tmem != tmem_base) *abort_flag = 1;
     // the weights are constants of the layer: their producer and the warps that expand them run ahead of earlier kernels
-    const bool expander = W4 && warp >= L::WORK0 && warp < L::WORK0 + 4 * L::EXP_GROUPS;
-    if (warp != 1 && warp != 16 && !expander) pdl_wait();
+    const bool expander = W4 && warp >= WORK0 && warp < HELP0;
+    if (warp != 1 && warp != HELP0 && !expander) pdl_wait();
 
     if (warp == 0 || warp == 3) {
         // ------------------------------------------------------------ MMA issuers (two warps of the leader)
@@ -310,33 +332,34 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             if (first >= pairs && elect_one()) commit_mmas<CG>(bar0 + 8 * L::ACC_FULL);  // (nothing to wait for)
             __syncwarp();
         }
-    } else if (warp == 1 || warp == 16) {
+    } else if (warp == 1 || warp == HELP0) {
         // ------------------------------------------------------------ weight rows of this CTA's channels
-        auto x_of = [&](int i) {  // first reduction index of k-block i
-            if (!p.conv) return i * BK;
-            const int tap = i / p.cblocks;
-            return tap * p.Cin + (i - tap * p.cblocks) * BK;
-        };
-        auto request = [&](int s, int sb, int u) {
-            if (W4) {  // a packed k-block, on a barrier of its own
-                const uint32_t full = bar0 + 8 * (L::FULL_P + s);
-                mbar_arrive_expect_tx(full, L::P_BYTES);
-                tma_load_2d(w0 + s * L::P_BYTES, &tmap_w, x_of(u) >> 1, n0, full);
-            } else {   // a pair of int8 ones
-                const int n = 2 * u + 1 < nkb ? 2 : 1;
+        auto x_of = [&](const KPos& at) { return at.tap * p.Cin + at.c * BK; };  // first reduction index of a k-block
+        auto request = [&](int s, int sb, int u, KPos at) {  // a pair of k-blocks
+            const int n = 2 * u + 1 < nkb ? 2 : 1;
+            if (W4) {  // on a barrier of its own
+                const uint32_t full = bar0 + 8 * (L::FULL_P + s), dst = w0 + s * L::P_BYTES;
+                mbar_arrive_expect_tx(full, (g.wide || n == 2) ? L::P_BYTES : L::P_BYTES / 2);
+                tma_load_2d(dst, &tmap_w, x_of(at) >> 1, n0, full);
+                if (!g.wide && n == 2) {
+                    at.advance(1, p.cblocks);
+                    tma_load_2d(dst + L::P_BYTES / 2, &tmap_w, x_of(at) >> 1, n0, full);
+                }
+            } else {
                 if (leader) mbar_arrive_expect_tx(bar0 + 8 * (L::READY + sb), n * CG * L::W_BYTES);
                 for (int h = 0; h < n; ++h) {
                     const uint32_t dst = w0 + (2 * s + h) * L::W_BYTES;
                     if (CG == 1)
-                        tma_load_2d(dst, &tmap_w, x_of(2 * u + h), n0, bar0 + 8 * (L::READY + sb));
+                        tma_load_2d(dst, &tmap_w, x_of(at), n0, bar0 + 8 * (L::READY + sb));
                     else
-                        tma_load_2d_pair(dst, &tmap_w, x_of(2 * u + h), n0, lead_bar0 + 8 * (L::READY + sb));
+                        tma_load_2d_pair(dst, &tmap_w, x_of(at), n0, lead_bar0 + 8 * (L::READY + sb));
+                    at.advance(1, p.cblocks);
                 }
             }
         };
-        produce(warp == 1 ? 0 : 1, lane, W4 ? L::PS : L::WS_MAX / 2, W4 ? nkb : pairs, bar0 + 8 * (W4 ? L::EMPTY_P : L::EMPTY),
+        produce(warp == 1 ? 0 : 1, lane, W4 ? L::PS : L::WS_MAX / 2, pairs, p.cblocks, bar0 + 8 * (W4 ? L::EMPTY_P : L::EMPTY),
                 W4 ? L::PS : L::NE, abort_flag, request);
-    } else if (warp == 2 || warp == 17) {
+    } else if (warp == 2 || warp == HELP0 + 1) {
         // ------------------------------------------------------------ int8 token rows by TMA
         const int m0 = tok0 + static_cast<int>(rank) * rows;
         int img = 0, wi = 0, hi = 0;
@@ -348,78 +371,84 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             hi = p.stride * ho - 1 + p.pad;
             wi = p.stride * (rem - ho * p.Wo) - 1 + p.pad;
         }
-        auto request = [&](int s, int sb, int u) {
+        auto request = [&](int s, int sb, int u, KPos at) {
             const uint32_t full = bar0 + 8 * (L::READY + sb), lead_full = lead_bar0 + 8 * (L::READY + sb);
             const int n = 2 * u + 1 < nkb ? 2 : 1;
             if (leader) mbar_arrive_expect_tx(full, n * CG * x_bytes);
             for (int h = 0; h < n; ++h) {
                 const uint32_t dst = x0 + (2 * s + h) * x_bytes;
-                const int i = 2 * u + h;
                 if (p.conv) {
-                    const int tap = i / p.cblocks, c = (i - tap * p.cblocks) * BK, kh = tap / 3, kw = tap - 3 * kh;
+                    const int kh = at.tap / 3, kw = at.tap - 3 * kh;
                     if (CG == 1)
-                        tma_load_im2col(dst, &tmap_x, c, wi, hi, img, kw, kh, full);
+                        tma_load_im2col(dst, &tmap_x, at.c * BK, wi, hi, img, kw, kh, full);
                     else
-                        tma_load_im2col_pair(dst, &tmap_x, c, wi, hi, img, kw, kh, lead_full);
+                        tma_load_im2col_pair(dst, &tmap_x, at.c * BK, wi, hi, img, kw, kh, lead_full);
                 } else if (CG == 1) {
-                    tma_load_2d(dst, &tmap_x, i * BK, m0, full);
+                    tma_load_2d(dst, &tmap_x, at.c * BK, m0, full);
                 } else {
-                    tma_load_2d_pair(dst, &tmap_x, i * BK, m0, lead_full);
+                    tma_load_2d_pair(dst, &tmap_x, at.c * BK, m0, lead_full);
                 }
+                at.advance(1, p.cblocks);
             }
         };
-        produce(warp == 2 ? 0 : 1, lane, g.x_slots / 2, pairs, bar0 + 8 * L::EMPTY, L::NE, abort_flag, request);
+        produce(warp == 2 ? 0 : 1, lane, g.x_slots / 2, pairs, p.cblocks, bar0 + 8 * L::EMPTY, L::NE, abort_flag, request);
     } else if (expander) {
         // ------------------------------------------------------------ packed int4 -> int8 (x16) in tensor memory
         // A thread owns a channel: its 64 packed bytes of a k-block become 32 columns of its lane.  Groups of four warps
-        // take alternate k-blocks; a group's next packed row is on its way into registers while the tensor-memory stores
-        // of this one complete.  (64-byte rows with the 64-byte swizzle: the reads are conflict-free.)
-        const int group = (warp - L::WORK0) >> 2, row = (warp & 3) * 32 + lane;
+        // take alternate pairs and fetch the next packed rows into registers before they wait for its slots.  (One k-block at a time, a turn took its group 1200 cycles, half of them for the waits and
+        // arrivals.)  The swizzle of the rows (128 bytes, or 64 where a pair is not contiguous) makes the reads
+        // conflict-free.
+        const int group = (warp - WORK0) >> 2, row = (warp & 3) * 32 + lane;
         constexpr uint32_t PS = L::PS > 0 ? L::PS : 1;
         const uint32_t a_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + g.a_col;
-        const uint8_t* base = smem + L::OFF_W + row * 64;
-        const uint32_t swz = (static_cast<uint32_t>(row >> 1) & 3u) << 4;
-        int sw = group;  // slot of the group's k-block (groups < slots)
-        uint4 w[4];
-        auto fetch = [&](int i) {
-            const uint32_t q = static_cast<uint32_t>(i), sp = q % PS;
+        const uint8_t* base = smem + L::OFF_W + row * (g.wide ? 128 : 64);
+        const uint32_t swz = g.wide ? (static_cast<uint32_t>(row) & 7u) << 4 : (static_cast<uint32_t>(row >> 1) & 3u) << 4;
+        const uint32_t second = g.wide ? 64u : L::P_BYTES / 2;  // from a row of the first k-block to the second's
+        int sw = 2 * group;  // slot of the pair's first k-block
+        if (sw >= g.w_slots) sw -= g.w_slots;
+        uint4 w[8];
+        auto fetch = [&](int j) {
+            const uint32_t q = static_cast<uint32_t>(j), sp = q % PS;
             const bool ok = mbar_wait(bar0 + 8 * (L::FULL_P + sp), (q / PS) & 1, abort_flag);
             const uint8_t* src = base + sp * L::P_BYTES;
 #pragma unroll
-            for (int j = 0; j < 4; ++j) w[j] = *reinterpret_cast<const uint4*>(src + ((static_cast<uint32_t>(j) << 4) ^ swz));
+            for (int k = 0; k < 8; ++k) {
+                // (wide: the second k-block is chunks 4 .. 7 of the row, and the swizzle runs over all eight)
+                const uint32_t off = static_cast<uint32_t>(k & 3) << 4;
+                w[k] = *reinterpret_cast<const uint4*>(src + (k < 4 ? off ^ swz : (g.wide ? (off | 64u) ^ swz : (off ^ swz) + second)));
+            }
             return ok;
         };
-        bool ok = group < nkb ? fetch(group) : true;
-        for (int i = group; i < nkb; i += L::EXP_GROUPS) {
-            if (ok && i >= g.w_slots) ok = wait_mmas<L>(bar0, i - g.w_slots, abort_flag);
-            if (!__all_sync(0xffffffffu, ok)) break;  // the warp leaves together
-            tc_fence_after_sync();
+        auto expand = [&](int h) {
             uint32_t c[32];
 #pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                const uint32_t v[4] = {w[j].x, w[j].y, w[j].z, w[j].w};
+            for (int k = 0; k < 4; ++k) {
+                const uint4& v4 = w[4 * h + k];
+                const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
 #pragma unroll
                 for (int q = 0; q < 4; ++q) {
-                    c[8 * j + 2 * q] = (v[q] << 4) & 0xF0F0F0F0u;
-                    c[8 * j + 2 * q + 1] = v[q] & 0xF0F0F0F0u;
+                    c[8 * k + 2 * q] = (v[q] << 4) & 0xF0F0F0F0u;
+                    c[8 * k + 2 * q + 1] = v[q] & 0xF0F0F0F0u;
                 }
             }
-            tmem_st_32x32(a_lane + sw * 32, c);
+            tmem_st_32x32(a_lane + (sw + h) * 32, c);
+        };
+        bool ok = group < pairs ? fetch(group) : true;
+        for (int j = group; j < pairs; j += EXP_GROUPS) {
+            if (ok && 2 * j >= g.w_slots) ok = wait_mmas<L>(bar0, 2 * j - g.w_slots, abort_flag);
+            if (!__all_sync(0xffffffffu, ok)) break;  // the warp leaves together
+            tc_fence_after_sync();
+            expand(0);
+            if (2 * j + 1 < nkb) expand(1);
             __syncwarp();
-            if (lane == 0) mbar_arrive(bar0 + 8 * (L::EMPTY_P + static_cast<uint32_t>(i) % PS));
-            if (i + L::EXP_GROUPS < nkb) ok = fetch(i + L::EXP_GROUPS);
+            if (lane == 0) mbar_arrive(bar0 + 8 * (L::EMPTY_P + static_cast<uint32_t>(j) % PS));
             tmem_st_wait();
             tc_fence_before_sync();
             __syncwarp();
-            if (lane == 0) arrive_at_leader<CG>(lead_bar0 + 8 * (L::READY + (i >> 1) % L::NE));
-            sw += L::EXP_GROUPS;
-            if (sw >= g.w_slots) sw -= g.w_slots;
-        }
-        // (a last pair of one k-block: the group whose turn the other would be arrives for it)
-        if ((nkb & 1) && nkb % L::EXP_GROUPS == group) {
-            if (ok && nkb >= g.w_slots) ok = wait_mmas<L>(bar0, nkb - g.w_slots, abort_flag);
-            __syncwarp();
-            if (ok && lane == 0) arrive_at_leader<CG>(lead_bar0 + 8 * (L::READY + (nkb >> 1) % L::NE));
+            if (lane == 0) arrive_at_leader<CG>(lead_bar0 + 8 * (L::READY + j % L::NE));
+            if (j + EXP_GROUPS < pairs) ok = fetch(j + EXP_GROUPS);
+            sw += 2 * EXP_GROUPS;
+            while (sw >= g.w_slots) sw -= g.w_slots;
         }
         pdl_wait();  // before these warps turn to the epilogue
     }
@@ -430,8 +459,8 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         // took its thread 370 cycles instead of 50.)
         mbar_wait(bar0 + 8 * L::ACC_FULL, 0, abort_flag);
         __syncwarp();
-        asm volatile("bar.sync 1, 416;" ::: "memory");
-    } else if (warp >= L::WORK0 && warp < L::WORK0 + 12) {
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * (WORKERS + 1)) : "memory");
+    } else if (warp >= WORK0 && warp < HELP0) {
         // ------------------------------------------------------------ epilogue: twelve warps, 8 tokens at a time
         const int n = n0 + (warp & 3) * 32 + lane;  // this lane's channel
         float comb = 0.f, bias = 0.f;
@@ -442,24 +471,24 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                 comb = (p.act_scale ? ld_pinned(p.act_scale) : 0.f) * ld_pinned(p.w_scale + n);
                 if (p.bias) bias = __half2float(p.bias[n]);
                 if (p.act_zero) bias = fmaf(static_cast<float>(zterm), comb, bias);
-                if (p.bos && p.Y && tok0 == 0 && warp < L::WORK0 + 4)
+                if (p.bos && p.Y && tok0 == 0 && warp < WORK0 + 4)
                     for (int b = 0; b < p.batch; ++b)
                         p.Y[static_cast<long long>(b) * MIXDQ_TOKENS_PER_PROMPT * p.ldy + n] = p.bos_out[n];
             }
         }
         if (W4) comb *= 0.0625f;  // the sums carry the factor 16 of the nibble placement: an exact power of two
-        asm volatile("bar.sync 1, 416;" ::: "memory");  // (warp 3 has seen the accumulator complete)
+        asm volatile("bar.sync 1, %0;" ::"n"(32 * (WORKERS + 1)) : "memory");  // (warp 3 has seen the accumulator complete)
         const bool ok = !*abort_flag;
         tc_fence_after_sync();
         const uint32_t acc = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16);
         const bool pairs_ok = ((p.N | static_cast<int>(p.ldy)) & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 3) == 0;
         const int cols = min(g.nt, p.M - tok0);
         if (ok && p.Y && pairs_ok && !p.acc_out) {
-            store_tokens(acc, ((warp - L::WORK0) >> 2) * 8, cols, comb, bias, p.Y + (n & ~1), p.ldy, tok0, p.M, n < p.N, p.bos != 0,
+            store_tokens(acc, ((warp - WORK0) >> 2) * 8, cols, comb, bias, p.Y + (n & ~1), p.ldy, tok0, p.M, n < p.N, p.bos != 0,
                          lane);
         } else if (ok) {
             // odd widths, and the raw sums of the parity hook
-            for (int c0 = ((warp - L::WORK0) >> 2) * 8; c0 < cols; c0 += 24) {
+            for (int c0 = ((warp - WORK0) >> 2) * 8; c0 < cols; c0 += 8 * EXP_GROUPS) {
                 uint32_t r[8];
                 tmem_ld_32x8(acc + c0, r);
                 tmem_ld_wait();
@@ -498,7 +527,7 @@ int launch_t(const CUtensorMap& tw, const CUtensorMap& tx, const TmaParams& tp, 
     auto kernel = chan_gemm_kernel<CG, W4>;
     if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), SMEM_MAX) != MIXDQ_OK) return MIXDQ_ERR_CUDA;
     const int x_bytes = g.nt / CG * BK;
-    // 12, 8 or 4 activation slots: the pair whose commit frees a slot, and the pair that last used the barrier of the one
+    // 16, 12, 8 or 4 activation slots: the pair whose commit frees a slot, and the pair that last used the barrier of the one
     // that will fill it, then belong to the same MMA issuer, so that the barrier's phase is over
     g.x_slots = std::min(L::XS_MAX, (SMEM_MAX - L::OFF_X) / x_bytes) & ~3;
     const int acc_cols = g.nt <= 128 ? 128 : 256;
@@ -538,10 +567,16 @@ int run_chan(const Params& p, int amode, const void* packed, int w_bits, const i
     tp.ldy = p.ldy;
     tp.acc_out = p.acc_out;
     tp.status = p.status;
-    tp.k_blocks = static_cast<int>(ceil_div(p.K, BK));
+    tp.k_blocks = tp.cblocks = static_cast<int>(ceil_div(p.K, BK));
     const int rows = tokens / cg;
     CUtensorMap tw, tx{};
-    int rc = w4 ? encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, BK / 2, CH, SWIZZLE_64)
+    ChanArgs g{};
+    g.nt = tokens;
+    g.c_tiles = static_cast<int>(ceil_div(p.N, CH * cg));
+    // 128 packed bytes of a row are two consecutive k-blocks, unless the channels of a filter tap end inside a k-block
+    g.wide = w4 && (!conv || p.Cin % BK == 0);
+    int rc = w4 ? encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, g.wide ? BK : BK / 2, CH,
+                                    g.wide ? SWIZZLE_128 : SWIZZLE_64)
                 : encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(p.K), p.N, pitch, BK, CH, SWIZZLE_128);
     if (rc != MIXDQ_OK) return rc;
     if (conv) {
@@ -559,9 +594,6 @@ int run_chan(const Params& p, int amode, const void* packed, int w_bits, const i
                                static_cast<uint32_t>(rows), SWIZZLE_128);
     }
     if (rc != MIXDQ_OK) return rc;
-    ChanArgs g{};
-    g.nt = tokens;
-    g.c_tiles = static_cast<int>(ceil_div(p.N, CH * cg));
     if (cg == 2) return w4 ? launch_t<2, true>(tw, tx, tp, g, stream) : launch_t<2, false>(tw, tx, tp, g, stream);
     return w4 ? launch_t<1, true>(tw, tx, tp, g, stream) : launch_t<1, false>(tw, tx, tp, g, stream);
 }

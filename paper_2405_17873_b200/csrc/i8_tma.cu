@@ -1214,12 +1214,13 @@ int plan_pair_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* splits
 // kernel runs one tile per CTA or CTA pair, so the tiles have to fit the SMs at once; a second wave costs more than the
 // form gains (4096 x 1280 x 640 int4: 11.3 us against 10.1).  Cycles of a tile of t tokens, from a fit to 104 layers (16 to
 // 16384 rows, 320 to 2560 channels, 3 to 180 k-blocks, linear and convolution; every tile that fits one wave; mean error
-// 6 per cent): fixed part + k-blocks x (issue + t) + epilogue of the tokens, where the share of the SMs in use slows each
-// k-block (they compete for the L2) and the start.  Chosen by it, the 104 layers ran within 2.2 per cent of each one's best
+// 5 per cent): fixed part + k-blocks x (issue + t) + epilogue of the tokens, where the share of the SMs in use slows each
+// k-block (they compete for the L2) and the start.  Chosen by it, the 104 layers ran within 1.9 per cent of each one's best
 // form and tile.
 //   * One CTA below 48 tokens or pairs below 64 never were the best (but for layers of so few rows).
 //   * int8 weights on pairs of more than 192 tokens leave room for four activation slots only: half the speed.
-//   * The single-CTA kernels' split reductions measured 5000 cycles over their estimate, the pair form's ten per cent under.
+//   * The other forms' estimates were six per cent short on these layers; the single-CTA kernels' split reductions measured
+//     5000 cycles over theirs, the pair form's ten per cent under.
 int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg)
 {
     const double nkb = k_blocks;
@@ -1233,8 +1234,9 @@ int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg)
             const int64_t ctas = c * c_tiles * ceil_div(M, t);
             if (ctas > num_sms) continue;
             const double busy = static_cast<double>(ctas) / num_sms;
-            const double cost = (w4 ? 3400.0 : 3700.0) + nkb * ((c == 1 ? (w4 ? 207.0 : 182.0) : (w4 ? 145.0 : 160.0)) + 1.1 * t + 92.0 * busy) +
-                                16.0 * t + (c == 1 ? 1270.0 : 3100.0) * busy;
+            const double per_kb = c == 1 ? (w4 ? 160.0 + 1.0 * t : 114.0 + 2.2 * t) : (w4 ? 72.0 + 1.5 * t : 96.0 + 1.4 * t);
+            const double cost = (w4 ? 3750.0 + 200.0 * c : 4500.0) + nkb * (per_kb + 72.0 * busy) + 15.0 * t +
+                                (c == 1 ? 1530.0 : 3300.0) * busy;
             if (best_tokens == 0 || cost < best) {
                 best = cost;
                 best_tokens = t;
@@ -1247,7 +1249,7 @@ int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg)
     const double single = o.single_cost + (o.single_splits > 1 ? 5000.0 : 0.0);
     const bool pair = o.pair_bn > 0 && o.pair_cost < 1.05 * single;
     const double other = pair ? o.pair_cost * (o.pair_splits > 1 ? 0.9 : 1.0) : single;
-    return best < other ? best_tokens : 0;
+    return best < 1.06 * other ? best_tokens : 0;
 }
 
 // Fused-quantization kernel (i8_fq.cu) or the two-kernel forms.  The fused kernel's k-block costs three to four

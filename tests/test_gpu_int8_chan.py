@@ -64,7 +64,7 @@ def test_asymmetric(bits, M, N, K):
 
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("B,H,W,Cin,Cout,stride", [(1, 4, 5, 32, 16, 1), (2, 17, 13, 160, 136, 2), (4, 16, 16, 640, 1280, 1),
-                                                   (3, 32, 30, 320, 640, 1), (1, 24, 24, 224, 321, 1)])
+                                                   (2, 32, 30, 320, 640, 1), (1, 24, 24, 224, 321, 1)])
 def test_conv3x3(bits, B, H, W, Cin, Cout, stride):
     Ho, Wo = (H - 1) // stride + 1, (W - 1) // stride + 1
     assert mixdq.int8_chan_tile(B * Ho * Wo, Cout, 9 * -(-Cin // 128), bits)[1] > 0
