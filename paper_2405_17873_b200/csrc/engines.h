@@ -78,10 +78,20 @@ int run_quant(const __half* X, long long ldx, long long rows, int K, const float
 int run_tma_prequantized(const Params& p, int amode, const void* packed, int w_bits, const int8_t* aq,
                          cudaStream_t stream);
 // Channel-major form (i8_chan.cu) on int8 codes: tiles of 128 cg channels x `tokens` tokens on cg = 1 or 2 CTAs.
+// plan_chan_tile: its tile's tokens where it is the fastest form for the layer, else 0; two: for both branches of a
+// shortcut-split layer at once (k_blocks of both), whose tile has at most CHAN_TWO_TOKENS.
+constexpr int CHAN_TWO_TOKENS = 128;
+struct ChanBranch {
+    const void* packed;
+    const int8_t* codes;
+    int cin;  // input channels (convolution) or reduction length of the branch
+    const float* act_scale;
+    int32_t* acc_out;
+};
 bool chan_tile_ok(int cg, int tokens);
-int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg);
-int run_chan(const Params& p, int amode, const void* packed, int w_bits, const int8_t* codes, int cg, int tokens,
-             cudaStream_t stream);
+int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg, bool two = false);
+int run_chan(const Params& p, int amode, const void* packed, int w_bits, const int8_t* codes, int cg, int tokens, cudaStream_t stream,
+             const ChanBranch* second = nullptr);
 // Shortcut-splitting (one activation scale per branch of a concatenated input): row elements [0, split_at)
 // and [split_at, row_len) are quantized, multiplied and summed separately and meet in a two-scale epilogue.
 // Linear layers and 3x3 convolutions whose halves both suit the two-kernel path.

@@ -72,7 +72,8 @@ struct Chan {
     static constexpr int EMPTY_P = FULL_P + PS;       // W4: packed rows read
     static constexpr int ACC_FULL = EMPTY_P + PS;
     static constexpr int GO = ACC_FULL + 1;           // leader: the MMA that overwrites the accumulator is issued
-    static constexpr int NUM_BARS = GO + 1;
+    static constexpr int GO2 = GO + 1;                // the same for the second branch's
+    static constexpr int NUM_BARS = GO2 + 1;
     static constexpr int OFF_BARS = RING_W;
     static constexpr int OFF_MISC = OFF_BARS + NUM_BARS * 8;
     static constexpr int OFF_X = (OFF_MISC + 16 + 1023) & ~1023;
@@ -84,6 +85,27 @@ struct ChanArgs {
     int x_slots, w_slots;
     int a_col;     // W4: first tensor-memory column of the expanded weights
     int wide;      // W4: a pair's packed rows are contiguous in memory and arrive as 128-byte rows
+    // two branches (shortcut-splitting, Sec. 4.1): the k-blocks from kb_lo on are the second branch's, with maps, geometry,
+    // scale and accumulator (column acc2) of its own; acc_out2: its sums (parity hook)
+    int kb_lo, cblocks2, Cin2, acc2;
+    const float* act_scale2;
+    int32_t* acc_out2;
+};
+
+// The k-blocks of a tile as pairs; with two branches each branch's pairs start at its own first k-block.
+template <bool TWO>
+struct Pairs {
+    int nkb, lo, kb_lo, n;  // k-blocks; TWO: pairs and k-blocks of the first branch; pairs in all
+    __device__ __forceinline__ Pairs(int nkb_, int kb_lo_)
+        : nkb(nkb_), lo(TWO ? (kb_lo_ + 1) >> 1 : 0), kb_lo(kb_lo_), n(TWO ? lo + ((nkb_ - kb_lo_ + 1) >> 1) : (nkb_ + 1) >> 1)
+    {
+    }
+    __device__ __forceinline__ bool second(int j) const { return TWO && j >= lo; }
+    __device__ __forceinline__ bool both(int j) const  // whether the pair has two k-blocks
+    {
+        if (!TWO) return 2 * j + 1 < nkb;
+        return j < lo ? 2 * j + 1 < kb_lo : 2 * (j - lo) + 1 < nkb - kb_lo;
+    }
 };
 
 // A load that stays where it is written (the compiler moves plain read-only loads down to their first use, past the
@@ -143,11 +165,13 @@ struct KPos {
 // Hence the two warps and the running position, and the first lap of the ring, which waits for nothing, goes out from all
 // lanes of the first of them at once (65 cycles apart).  free[unit % barriers] says that the slot of the unit `slots`
 // positions later is free; `barriers` is even and at least `slots`: a warp meets every phase.
-template <typename F>
-__device__ __forceinline__ void produce(int which, int lane, int slots, int units, int cblocks, uint32_t free, int barriers,
-                                        volatile int* abort_flag, F&& request)
+template <bool TWO, typename F>
+__device__ __forceinline__ void produce(int which, int lane, int slots, const Pairs<TWO>& pr, int cblocks, int cblocks2, uint32_t free,
+                                        int barriers, volatile int* abort_flag, F&& request)
 {
-    if (which == 0 && lane < slots && lane < units) request(lane, lane, lane, KPos(2 * lane, cblocks));
+    const int units = pr.n;
+    if (which == 0 && lane < slots && lane < units)
+        request(lane, lane, lane, pr.second(lane) ? KPos(2 * (lane - pr.lo), cblocks2) : KPos(2 * lane, cblocks));
     __syncwarp();
     if (slots + which >= units) return;
     int s = which, q = which, sb = which + slots;
@@ -155,7 +179,13 @@ __device__ __forceinline__ void produce(int which, int lane, int slots, int unit
     if (sb >= barriers) sb -= barriers;
     uint32_t par = 0;
     KPos at(2 * (slots + which), cblocks);
+    bool second = false;
     for (int i = slots + which; i < units; i += 2) {
+        if (TWO && !second && pr.second(i)) {
+            second = true;
+            cblocks = cblocks2;
+            at = KPos(2 * (i - pr.lo), cblocks2);
+        }
         const bool ok = mbar_wait(free + 8 * q, par, abort_flag);
         if (!__all_sync(0xffffffffu, ok)) break;
         if (elect_one()) request(s, sb, i, at);
@@ -176,20 +206,27 @@ __device__ __forceinline__ void produce(int which, int lane, int slots, int unit
 // One warp's share of the epilogue: its 32 lanes' channels x every third group of eight tokens.  Lanes 2 i and 2 i + 1 swap
 // halves of a packed token pair and each stores both channels of one token: a store covers 64 contiguous bytes of two
 // output rows.  col: Y at the lane's channel pair.
-__device__ __forceinline__ void store_tokens(uint32_t acc, int c0, int cols, float comb, float bias, __half* col, long long ldy,
-                                             int tok0, int M, bool in_n, bool bos, int lane)
+template <bool TWO>
+__device__ __forceinline__ void store_tokens(uint32_t acc, uint32_t acc2, int c0, int cols, float comb, float comb2, float bias,
+                                             __half* col, long long ldy, int tok0, int M, bool in_n, bool bos, int lane)
 {
     const uint32_t sel = (lane & 1) ? 0x3276u : 0x5410u;  // odd: token 1 (other's, own); even: token 0 (own, other's)
     const bool all_n = __all_sync(0xffffffffu, in_n);
     for (; c0 < cols; c0 += 8 * EXP_GROUPS) {
-        uint32_t r[8], own[4], out[4];
+        uint32_t r[8], r2[8], own[4], out[4];
         tmem_ld_32x8(acc + c0, r);
+        if (TWO) tmem_ld_32x8(acc2 + c0, r2);
         tmem_ld_wait();
         const int m0 = tok0 + c0 + (lane & 1);
 #pragma unroll
         for (int j = 0; j < 4; ++j) {
-            const __half2 h = __floats2half2_rn(fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j])), comb, bias),
-                                                fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j + 1])), comb, bias));
+            float a = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j])), comb, bias);
+            float b = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j + 1])), comb, bias);
+            if (TWO) {
+                a = fmaf(__int2float_rn(static_cast<int32_t>(r2[2 * j])), comb2, a);
+                b = fmaf(__int2float_rn(static_cast<int32_t>(r2[2 * j + 1])), comb2, b);
+            }
+            const __half2 h = __floats2half2_rn(a, b);
             own[j] = *reinterpret_cast<const uint32_t*>(&h);
         }
 #pragma unroll
@@ -211,9 +248,10 @@ __device__ __forceinline__ void store_tokens(uint32_t acc, int c0, int cols, flo
 }
 
 // Grid: CG CTAs (a cluster) per tile of 128 CG channels x nt tokens, channel tiles fastest.
-template <int CG, bool W4>
+template <int CG, bool W4, bool TWO>
 __global__ void __launch_bounds__(THREADS, 1)
-chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x, const TmaParams p,
+chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant__ CUtensorMap tmap_x,
+                 const __grid_constant__ CUtensorMap tmap_w2, const __grid_constant__ CUtensorMap tmap_x2, const TmaParams p,
                  const ChanArgs g)
 {
     using L = Chan<CG, W4>;
@@ -225,7 +263,8 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     const uint32_t rank = CG == 2 ? cluster_ctarank() : 0u;
     const bool leader = rank == 0;
     const int tile = static_cast<int>(blockIdx.x) / CG;
-    const int nkb = p.k_blocks, pairs = (nkb + 1) >> 1, rows = g.nt / CG;  // token rows this CTA holds
+    const Pairs<TWO> pr(p.k_blocks, g.kb_lo);
+    const int pairs = pr.n, rows = g.nt / CG;  // token rows this CTA holds
     const int tok0 = (tile / g.c_tiles) * g.nt;
     const int n0 = (tile % g.c_tiles) * (CG * CH) + static_cast<int>(rank) * CH;
     const uint32_t x_bytes = static_cast<uint32_t>(rows) * BK;
@@ -246,6 +285,7 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         }
         mbar_init(bar0 + 8 * L::ACC_FULL, L::ISSUERS);
         mbar_init(bar0 + 8 * L::GO, 1);
+        mbar_init(bar0 + 8 * L::GO2, 1);
         *abort_flag = (smem_u32(smem) & 1023u) ? 1 : 0;  // the swizzled tiles need the alignment the array is declared with
         fence_barrier_init();
     } else if (warp == 0) {
@@ -289,11 +329,14 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             bool ok = first == 0 || first >= pairs || mbar_wait(bar0 + 8 * L::GO, 0, abort_flag);
             for (int j = first; j < pairs; j += L::ISSUERS) {
                 ok = ok && mbar_wait(bar0 + 8 * (L::READY + sb), par, abort_flag);
+                if (TWO && j == pr.lo + 1) ok = ok && mbar_wait(bar0 + 8 * L::GO2, 0, abort_flag);
                 if (!__all_sync(0xffffffffu, ok)) break;
                 tc_fence_after_sync();
                 const uint64_t x_desc = x_desc0 + static_cast<uint32_t>(sx) * (x_bytes >> 4);
                 const uint64_t w_desc = w_desc0 + sw * (L::W_BYTES >> 4);
-                const bool both = 2 * j + 1 < nkb;
+                const bool both = pr.both(j);
+                const bool fresh = j == 0 || (TWO && j == pr.lo);  // overwrites its accumulator
+                const uint32_t acc = tmem_base + (pr.second(j) ? g.acc2 : 0);
                 if (elect_one()) {
 #pragma unroll
                     for (int h = 0; h < 2; ++h) {
@@ -301,19 +344,19 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                         const uint64_t xd = x_desc + h * (x_bytes >> 4);
 #pragma unroll
                         for (int k = 0; k < BK / 32; ++k) {
-                            const uint32_t add = (j != 0 || h != 0 || k != 0) ? 1u : 0u;
+                            const uint32_t add = (!fresh || h != 0 || k != 0) ? 1u : 0u;
                             const uint64_t wd = w_desc + h * (L::W_BYTES >> 4) + 2 * k;
                             if (W4)
-                                mma_i8_ts<CG>(tmem_base, tmem_base + g.a_col + sw * 32 + 32 * h + 8 * k, xd + 2 * k, idesc, add);
+                                mma_i8_ts<CG>(acc, tmem_base + g.a_col + sw * 32 + 32 * h + 8 * k, xd + 2 * k, idesc, add);
                             else if (CG == 1)
-                                mma_i8_ss(tmem_base, wd, xd + 2 * k, idesc, add);
+                                mma_i8_ss(acc, wd, xd + 2 * k, idesc, add);
                             else
-                                mma_i8_pair(tmem_base, wd, xd + 2 * k, idesc, add);
+                                mma_i8_pair(acc, wd, xd + 2 * k, idesc, add);
                         }
                     }
-                    if (j == 0 && pairs > 1) {
+                    if (fresh) {
                         tc_fence_before_sync();
-                        mbar_arrive(bar0 + 8 * L::GO);
+                        mbar_arrive(bar0 + 8 * (j == 0 ? L::GO : L::GO2));
                     }
                     commit_mmas<CG>(bar0 + 8 * (L::EMPTY + sb));
                     if (j + L::ISSUERS >= pairs) commit_mmas<CG>(bar0 + 8 * L::ACC_FULL);
@@ -334,31 +377,34 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         }
     } else if (warp == 1 || warp == HELP0) {
         // ------------------------------------------------------------ weight rows of this CTA's channels
-        auto x_of = [&](const KPos& at) { return at.tap * p.Cin + at.c * BK; };  // first reduction index of a k-block
         auto request = [&](int s, int sb, int u, KPos at) {  // a pair of k-blocks
-            const int n = 2 * u + 1 < nkb ? 2 : 1;
+            const int n = pr.both(u) ? 2 : 1;
+            const bool second = pr.second(u);
+            const CUtensorMap* map = second ? &tmap_w2 : &tmap_w;
+            const int cblocks = second ? g.cblocks2 : p.cblocks, cin = second ? g.Cin2 : p.Cin;
+            auto x_of = [&](const KPos& at) { return at.tap * cin + at.c * BK; };  // first reduction index of a k-block
             if (W4) {  // on a barrier of its own
                 const uint32_t full = bar0 + 8 * (L::FULL_P + s), dst = w0 + s * L::P_BYTES;
                 mbar_arrive_expect_tx(full, (g.wide || n == 2) ? L::P_BYTES : L::P_BYTES / 2);
-                tma_load_2d(dst, &tmap_w, x_of(at) >> 1, n0, full);
+                tma_load_2d(dst, map, x_of(at) >> 1, n0, full);
                 if (!g.wide && n == 2) {
-                    at.advance(1, p.cblocks);
-                    tma_load_2d(dst + L::P_BYTES / 2, &tmap_w, x_of(at) >> 1, n0, full);
+                    at.advance(1, cblocks);
+                    tma_load_2d(dst + L::P_BYTES / 2, map, x_of(at) >> 1, n0, full);
                 }
             } else {
                 if (leader) mbar_arrive_expect_tx(bar0 + 8 * (L::READY + sb), n * CG * L::W_BYTES);
                 for (int h = 0; h < n; ++h) {
                     const uint32_t dst = w0 + (2 * s + h) * L::W_BYTES;
                     if (CG == 1)
-                        tma_load_2d(dst, &tmap_w, x_of(at), n0, bar0 + 8 * (L::READY + sb));
+                        tma_load_2d(dst, map, x_of(at), n0, bar0 + 8 * (L::READY + sb));
                     else
-                        tma_load_2d_pair(dst, &tmap_w, x_of(at), n0, lead_bar0 + 8 * (L::READY + sb));
-                    at.advance(1, p.cblocks);
+                        tma_load_2d_pair(dst, map, x_of(at), n0, lead_bar0 + 8 * (L::READY + sb));
+                    at.advance(1, cblocks);
                 }
             }
         };
-        produce(warp == 1 ? 0 : 1, lane, W4 ? L::PS : L::WS_MAX / 2, pairs, p.cblocks, bar0 + 8 * (W4 ? L::EMPTY_P : L::EMPTY),
-                W4 ? L::PS : L::NE, abort_flag, request);
+        produce<TWO>(warp == 1 ? 0 : 1, lane, W4 ? L::PS : L::WS_MAX / 2, pr, p.cblocks, g.cblocks2,
+                     bar0 + 8 * (W4 ? L::EMPTY_P : L::EMPTY), W4 ? L::PS : L::NE, abort_flag, request);
     } else if (warp == 2 || warp == HELP0 + 1) {
         // ------------------------------------------------------------ int8 token rows by TMA
         const int m0 = tok0 + static_cast<int>(rank) * rows;
@@ -373,25 +419,27 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         }
         auto request = [&](int s, int sb, int u, KPos at) {
             const uint32_t full = bar0 + 8 * (L::READY + sb), lead_full = lead_bar0 + 8 * (L::READY + sb);
-            const int n = 2 * u + 1 < nkb ? 2 : 1;
+            const int n = pr.both(u) ? 2 : 1;
+            const bool second = pr.second(u);
+            const CUtensorMap* map = second ? &tmap_x2 : &tmap_x;
             if (leader) mbar_arrive_expect_tx(full, n * CG * x_bytes);
             for (int h = 0; h < n; ++h) {
                 const uint32_t dst = x0 + (2 * s + h) * x_bytes;
                 if (p.conv) {
                     const int kh = at.tap / 3, kw = at.tap - 3 * kh;
                     if (CG == 1)
-                        tma_load_im2col(dst, &tmap_x, at.c * BK, wi, hi, img, kw, kh, full);
+                        tma_load_im2col(dst, map, at.c * BK, wi, hi, img, kw, kh, full);
                     else
-                        tma_load_im2col_pair(dst, &tmap_x, at.c * BK, wi, hi, img, kw, kh, lead_full);
+                        tma_load_im2col_pair(dst, map, at.c * BK, wi, hi, img, kw, kh, lead_full);
                 } else if (CG == 1) {
-                    tma_load_2d(dst, &tmap_x, at.c * BK, m0, full);
+                    tma_load_2d(dst, map, at.c * BK, m0, full);
                 } else {
-                    tma_load_2d_pair(dst, &tmap_x, at.c * BK, m0, lead_full);
+                    tma_load_2d_pair(dst, map, at.c * BK, m0, lead_full);
                 }
-                at.advance(1, p.cblocks);
+                at.advance(1, second ? g.cblocks2 : p.cblocks);
             }
         };
-        produce(warp == 2 ? 0 : 1, lane, g.x_slots / 2, pairs, p.cblocks, bar0 + 8 * L::EMPTY, L::NE, abort_flag, request);
+        produce<TWO>(warp == 2 ? 0 : 1, lane, g.x_slots / 2, pr, p.cblocks, g.cblocks2, bar0 + 8 * L::EMPTY, L::NE, abort_flag, request);
     } else if (expander) {
         // ------------------------------------------------------------ packed int4 -> int8 (x16) in tensor memory
         // A thread owns a channel: its 64 packed bytes of a k-block become 32 columns of its lane.  Groups of four warps
@@ -439,7 +487,7 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             if (!__all_sync(0xffffffffu, ok)) break;  // the warp leaves together
             tc_fence_after_sync();
             expand(0);
-            if (2 * j + 1 < nkb) expand(1);
+            if (pr.both(j)) expand(1);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar0 + 8 * (L::EMPTY_P + static_cast<uint32_t>(j) % PS));
             tmem_st_wait();
@@ -463,12 +511,13 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     } else if (warp >= WORK0 && warp < HELP0) {
         // ------------------------------------------------------------ epilogue: twelve warps, 8 tokens at a time
         const int n = n0 + (warp & 3) * 32 + lane;  // this lane's channel
-        float comb = 0.f, bias = 0.f;
+        float comb = 0.f, comb2 = 0.f, bias = 0.f;
         int zterm = 0;  // (128 - zero) * sum of the channel's weight codes
         if (n < p.N) {
             if (p.act_zero) zterm = (128 - __ldg(p.act_zero)) * __ldg(p.w_code_sums + n);
             if (p.w_scale) {
                 comb = (p.act_scale ? ld_pinned(p.act_scale) : 0.f) * ld_pinned(p.w_scale + n);
+                if (TWO) comb2 = ld_pinned(g.act_scale2) * ld_pinned(p.w_scale + n);
                 if (p.bias) bias = __half2float(p.bias[n]);
                 if (p.act_zero) bias = fmaf(static_cast<float>(zterm), comb, bias);
                 if (p.bos && p.Y && tok0 == 0 && warp < WORK0 + 4)
@@ -476,7 +525,10 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
                         p.Y[static_cast<long long>(b) * MIXDQ_TOKENS_PER_PROMPT * p.ldy + n] = p.bos_out[n];
             }
         }
-        if (W4) comb *= 0.0625f;  // the sums carry the factor 16 of the nibble placement: an exact power of two
+        if (W4) {  // the sums carry the factor 16 of the nibble placement: an exact power of two
+            comb *= 0.0625f;
+            comb2 *= 0.0625f;
+        }
         asm volatile("bar.sync 1, %0;" ::"n"(32 * (WORKERS + 1)) : "memory");  // (warp 3 has seen the accumulator complete)
         const bool ok = !*abort_flag;
         tc_fence_after_sync();
@@ -484,22 +536,29 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         const bool pairs_ok = ((p.N | static_cast<int>(p.ldy)) & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 3) == 0;
         const int cols = min(g.nt, p.M - tok0);
         if (ok && p.Y && pairs_ok && !p.acc_out) {
-            store_tokens(acc, ((warp - WORK0) >> 2) * 8, cols, comb, bias, p.Y + (n & ~1), p.ldy, tok0, p.M, n < p.N, p.bos != 0,
-                         lane);
+            store_tokens<TWO>(acc, acc + g.acc2, ((warp - WORK0) >> 2) * 8, cols, comb, comb2, bias, p.Y + (n & ~1), p.ldy, tok0, p.M,
+                              n < p.N, p.bos != 0, lane);
         } else if (ok) {
             // odd widths, and the raw sums of the parity hook
             for (int c0 = ((warp - WORK0) >> 2) * 8; c0 < cols; c0 += 8 * EXP_GROUPS) {
-                uint32_t r[8];
+                uint32_t r[8], r2[8];
                 tmem_ld_32x8(acc + c0, r);
+                if (TWO) tmem_ld_32x8(acc + g.acc2 + c0, r2);
                 tmem_ld_wait();
 #pragma unroll
                 for (int j = 0; j < 8; ++j) {
                     int m = tok0 + c0 + j;
                     if (m >= p.M || n >= p.N) continue;
                     const int32_t a = static_cast<int32_t>(r[j]);
+                    float v = fmaf(__int2float_rn(a), comb, bias);
                     if (p.acc_out) p.acc_out[static_cast<long long>(m) * p.N + n] = (W4 ? (a >> 4) : a) + zterm;
+                    if (TWO) {
+                        const int32_t a2 = static_cast<int32_t>(r2[j]);
+                        v = fmaf(__int2float_rn(a2), comb2, v);
+                        if (g.acc_out2) g.acc_out2[static_cast<long long>(m) * p.N + n] = W4 ? (a2 >> 4) : a2;
+                    }
                     if (p.bos) m += m / (MIXDQ_TOKENS_PER_PROMPT - 1) + 1;
-                    if (p.Y) p.Y[m * p.ldy + n] = __float2half_rn(fmaf(__int2float_rn(a), comb, bias));
+                    if (p.Y) p.Y[m * p.ldy + n] = __float2half_rn(v);
                 }
             }
         }
@@ -520,22 +579,47 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     }
 }
 
-template <int CG, bool W4>
-int launch_t(const CUtensorMap& tw, const CUtensorMap& tx, const TmaParams& tp, ChanArgs g, cudaStream_t stream)
+template <int CG, bool W4, bool TWO>
+int launch_t(const CUtensorMap* maps, const TmaParams& tp, ChanArgs g, cudaStream_t stream)
 {
     using L = Chan<CG, W4>;
-    auto kernel = chan_gemm_kernel<CG, W4>;
+    auto kernel = chan_gemm_kernel<CG, W4, TWO>;
     if (ensure_dynamic_smem(reinterpret_cast<const void*>(kernel), SMEM_MAX) != MIXDQ_OK) return MIXDQ_ERR_CUDA;
     const int x_bytes = g.nt / CG * BK;
-    // 16, 12, 8 or 4 activation slots: the pair whose commit frees a slot, and the pair that last used the barrier of the one
+    // 12, 8 or 4 activation slots: the pair whose commit frees a slot, and the pair that last used the barrier of the one
     // that will fill it, then belong to the same MMA issuer, so that the barrier's phase is over
     g.x_slots = std::min(L::XS_MAX, (SMEM_MAX - L::OFF_X) / x_bytes) & ~3;
-    const int acc_cols = g.nt <= 128 ? 128 : 256;
+    const int acc_cols = g.nt <= 128 ? (TWO ? 256 : 128) : 256;
+    g.acc2 = TWO ? 128 : 0;
     g.w_slots = W4 ? (512 - acc_cols) / 32 : L::WS_MAX;
     g.a_col = acc_cols;
     const int tiles = g.c_tiles * static_cast<int>(ceil_div(tp.M, g.nt));
     return launch_pdl_cluster(kernel, dim3(static_cast<unsigned>(CG * tiles)), dim3(THREADS),
-                              static_cast<size_t>(L::OFF_X + g.x_slots * x_bytes), stream, CG, 1u, tw, tx, tp, g);
+                              static_cast<size_t>(L::OFF_X + g.x_slots * x_bytes), stream, CG, 1u, maps[0], maps[1], maps[2], maps[3],
+                              tp, g);
+}
+
+template <bool TWO>
+int launch(const CUtensorMap* maps, const TmaParams& tp, const ChanArgs& g, int cg, bool w4, cudaStream_t stream)
+{
+    if (cg == 2) return w4 ? launch_t<2, true, TWO>(maps, tp, g, stream) : launch_t<2, false, TWO>(maps, tp, g, stream);
+    return w4 ? launch_t<1, true, TWO>(maps, tp, g, stream) : launch_t<1, false, TWO>(maps, tp, g, stream);
+}
+
+// Tensor maps of one branch: its weights [N, taps * cin] and its activations, int8 [M, cin] or the NHWC image of cin channels
+// (with its border when pad is set).
+int encode_branch(CUtensorMap* tw, CUtensorMap* tx, const Params& p, bool conv, int pad, int cin, const void* packed, bool w4, bool wide,
+                  const int8_t* codes, int rows)
+{
+    const int64_t K = (conv ? 9ll : 1ll) * cin;
+    const int64_t pitch = row_pitch_bytes(K, w4 ? 4 : 8, MIXDQ_LAYOUT_DEVICE);
+    const int rc = w4 ? encode_tmap_2d_u8(tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, wide ? BK : BK / 2, CH,
+                                          wide ? SWIZZLE_128 : SWIZZLE_64)
+                      : encode_tmap_2d_u8(tw, packed, static_cast<uint64_t>(K), p.N, pitch, BK, CH, SWIZZLE_128);
+    if (rc != MIXDQ_OK) return rc;
+    if (conv) return encode_tmap_im2col3x3(tx, codes, false, p.batch, p.H + 2 * pad, p.W + 2 * pad, cin, pad, p.stride, BK, rows);
+    return encode_tmap_2d_u8(tx, codes, static_cast<uint64_t>(cin), static_cast<uint64_t>(p.M), static_cast<uint64_t>(cin), BK,
+                             static_cast<uint32_t>(rows), SWIZZLE_128);
 }
 
 }  // namespace
@@ -545,13 +629,14 @@ bool chan_tile_ok(int cg, int tokens)
     return (cg == 1 || cg == 2) && tokens >= 16 * cg && tokens % (16 * cg) == 0 && tokens <= TOK_MAX && tokens / cg <= ROWS_MAX;
 }
 
-// codes: int8 activations, [M, K] rows, or the NHWC image (with its border when p.act_zero).
-int run_chan(const Params& p, int amode, const void* packed, int w_bits, const int8_t* codes, int cg, int tokens, cudaStream_t stream)
+// codes: int8 activations, [M, K] rows, or the NHWC image (with its border when p.act_zero).  second: the other branch of a
+// shortcut-split layer (p.K or p.Cin, p.act_scale, p.acc_out, packed and codes are then the first branch's).
+int run_chan(const Params& p, int amode, const void* packed, int w_bits, const int8_t* codes, int cg, int tokens, cudaStream_t stream,
+             const ChanBranch* second)
 {
     const bool w4 = w_bits == 4, conv = amode == A_CONV3;
-    if (!chan_tile_ok(cg, tokens) || p.addend) return MIXDQ_ERR_INVALID_ARG;
+    if (!chan_tile_ok(cg, tokens) || p.addend || (second && tokens > CHAN_TWO_TOKENS)) return MIXDQ_ERR_INVALID_ARG;
     const int pad = (conv && p.act_zero) ? 1 : 0;
-    const int64_t pitch = row_pitch_bytes(p.K, w_bits, MIXDQ_LAYOUT_DEVICE);
     TmaParams tp{};
     tp.M = p.M;
     tp.N = p.N;
@@ -567,35 +652,35 @@ int run_chan(const Params& p, int amode, const void* packed, int w_bits, const i
     tp.ldy = p.ldy;
     tp.acc_out = p.acc_out;
     tp.status = p.status;
-    tp.k_blocks = tp.cblocks = static_cast<int>(ceil_div(p.K, BK));
-    const int rows = tokens / cg;
-    CUtensorMap tw, tx{};
+    const int cin = conv ? p.Cin : p.K, rows = tokens / cg;
     ChanArgs g{};
     g.nt = tokens;
     g.c_tiles = static_cast<int>(ceil_div(p.N, CH * cg));
     // 128 packed bytes of a row are two consecutive k-blocks, unless the channels of a filter tap end inside a k-block
-    g.wide = w4 && (!conv || p.Cin % BK == 0);
-    int rc = w4 ? encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, g.wide ? BK : BK / 2, CH,
-                                    g.wide ? SWIZZLE_128 : SWIZZLE_64)
-                : encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(p.K), p.N, pitch, BK, CH, SWIZZLE_128);
-    if (rc != MIXDQ_OK) return rc;
+    g.wide = w4 && (!conv || (cin % BK == 0 && (!second || second->cin % BK == 0)));
+    tp.cblocks = static_cast<int>(ceil_div(cin, BK));
+    tp.k_blocks = (conv ? 9 : 1) * tp.cblocks;
     if (conv) {
-        rc = encode_tmap_im2col3x3(&tx, codes, false, p.batch, p.H + 2 * pad, p.W + 2 * pad, p.Cin, pad, p.stride, BK, rows);
         tp.conv = 1;
         tp.pad = pad;
         tp.stride = p.stride;
-        tp.cblocks = static_cast<int>(ceil_div(p.Cin, BK));
         tp.Cin = p.Cin;
         tp.HoWo = p.Ho * p.Wo;
         tp.Wo = p.Wo;
-        tp.k_blocks = 9 * tp.cblocks;
-    } else {
-        rc = encode_tmap_2d_u8(&tx, codes, static_cast<uint64_t>(p.K), static_cast<uint64_t>(p.M), static_cast<uint64_t>(p.K), BK,
-                               static_cast<uint32_t>(rows), SWIZZLE_128);
     }
+    CUtensorMap maps[4]{};  // weights, activations; the second branch's
+    int rc = encode_branch(&maps[0], &maps[1], p, conv, pad, cin, packed, w4, g.wide, codes, rows);
     if (rc != MIXDQ_OK) return rc;
-    if (cg == 2) return w4 ? launch_t<2, true>(tw, tx, tp, g, stream) : launch_t<2, false>(tw, tx, tp, g, stream);
-    return w4 ? launch_t<1, true>(tw, tx, tp, g, stream) : launch_t<1, false>(tw, tx, tp, g, stream);
+    if (!second) return launch<false>(maps, tp, g, cg, w4, stream);
+    rc = encode_branch(&maps[2], &maps[3], p, conv, pad, second->cin, second->packed, w4, g.wide, second->codes, rows);
+    if (rc != MIXDQ_OK) return rc;
+    g.kb_lo = tp.k_blocks;
+    g.cblocks2 = static_cast<int>(ceil_div(second->cin, BK));
+    g.Cin2 = conv ? second->cin : 0;
+    g.act_scale2 = second->act_scale;
+    g.acc_out2 = second->acc_out;
+    tp.k_blocks += (conv ? 9 : 1) * g.cblocks2;
+    return launch<true>(maps, tp, g, cg, w4, stream);
 }
 
 }  // namespace i8

@@ -1221,7 +1221,7 @@ int plan_pair_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* splits
 //   * int8 weights on pairs of more than 192 tokens leave room for four activation slots only: half the speed.
 //   * The other forms' estimates were six per cent short on these layers; the single-CTA kernels' split reductions measured
 //     5000 cycles over theirs, the pair form's ten per cent under.
-int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg)
+int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg, bool two)
 {
     const double nkb = k_blocks;
     double best = 0;
@@ -1229,7 +1229,7 @@ int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg)
     for (int c = 1; c <= 2; ++c) {
         const int64_t c_tiles = ceil_div(N, 128 * c);
         for (int t = 16 * c; t <= (c == 2 && !w4 ? 192 : 128 * c); t += 16 * c) {
-            if (t < 32 * c && M > 64) continue;
+            if ((t < 32 * c && M > 64) || (two && t > CHAN_TWO_TOKENS)) continue;
             if (t >= M + 16 * c) break;  // (nothing but padding more than the tile before)
             const int64_t ctas = c * c_tiles * ceil_div(M, t);
             if (ctas > num_sms) continue;
@@ -1245,7 +1245,7 @@ int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg)
         }
     }
     if (best_tokens == 0) return 0;
-    const TokenPlan o = token_plan(M, N, k_blocks, w4, num_sms, true);
+    const TokenPlan o = token_plan(M, N, k_blocks, w4, num_sms, !two);
     const double single = o.single_cost + (o.single_splits > 1 ? 5000.0 : 0.0);
     const bool pair = o.pair_bn > 0 && o.pair_cost < 1.05 * single;
     const double other = pair ? o.pair_cost * (o.pair_splits > 1 ? 0.9 : 1.0) : single;
@@ -1596,7 +1596,7 @@ int run_tma_split(const Params& p, int amode, int split_at, const void* packed_l
                         p.X, ldx, in_rows, row_len, split_at, scale_lo, scale_hi, aq_lo, aq_hi);
     if (rc != MIXDQ_OK) return rc;
 
-    // One launch where the two-CTA form suits the layer: both branches' k-blocks in one kernel, an accumulator per
+    // One launch where the channel-major or the two-CTA form suits the layer: both branches' k-blocks in one kernel, an accumulator per
     // branch in tensor memory, the two-scale epilogue straight from there (no int32 round trip through memory).
     const int num_sms = sm_count();
     if (num_sms <= 0) return MIXDQ_ERR_CUDA;
@@ -1604,6 +1604,17 @@ int run_tma_split(const Params& p, int amode, int split_at, const void* packed_l
     const int c_lo = split_at, c_hi = row_len - split_at;
     const int kb_lo = static_cast<int>(conv ? 9 * ceil_div(c_lo, BK) : ceil_div(c_lo, BK));
     const int kb_hi = static_cast<int>(conv ? 9 * ceil_div(c_hi, BK) : ceil_div(c_hi, BK));
+    int cg;
+    const int tokens = plan_chan_tile(p.M, p.N, kb_lo + kb_hi, w4, num_sms, &cg, true);
+    if (tokens > 0) {
+        Params q = p;
+        q.Cin = conv ? c_lo : 0;
+        q.K = conv ? 9 * c_lo : c_lo;
+        q.act_scale = scale_lo;
+        q.acc_out = p.Y ? nullptr : acc_lo_out;
+        const ChanBranch second{packed_hi, aq_hi, c_hi, scale_hi, p.Y ? nullptr : acc_hi_out};
+        return run_chan(q, amode, packed_lo, w_bits, aq_lo, cg, tokens, stream, &second);
+    }
     const int pair_bn = plan_pair_tile(p.M, p.N, kb_lo + kb_hi, w4, num_sms, nullptr);
     if (pair_bn > 0) {
         CUtensorMap ta[2], tw[2], ty{};

@@ -1,12 +1,14 @@
 """The channel-major int8 kernel (weights on the rows of the tensor-core tile) on one- and two-CTA tiles: odd and even
 numbers of k-blocks from one to more than every ring holds, ragged channels, tokens and reduction tails, odd widths,
-every source of activations (rows, skipped first tokens, im2col, asymmetric codes)."""
+every source of activations (rows, skipped first tokens, im2col, asymmetric codes), both branches of shortcut-split
+layers."""
 import numpy as np
 import pytest
 import torch
 
 from oracle import mixdq_oracle as orc
 from paper_2405_17873_b200 import mixdq, synth
+import test_gpu_int8_split as split
 from helpers import assert_close, dev, device_weights, host, oracle_weights, status_word
 
 pytestmark = pytest.mark.gpu
@@ -105,3 +107,16 @@ def test_bos(bits, batch, N, K):
     assert int(host(st)[0]) == 0
     assert np.array_equal(host(acc), acc_ref)
     assert_close(host(y), y_ref)
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("M,C_lo,C_hi,N", [(1, 16, 16, 16), (100, 144, 272, 129), (1024, 1280, 1280, 1280), (250, 2064, 128, 648)])
+def test_two_branches_linear(bits, M, C_lo, C_hi, N):
+    split._run_linear(M, C_lo, C_hi, N, bits, seed=M + C_lo)
+
+
+@pytest.mark.parametrize("bits", [8, 4])
+@pytest.mark.parametrize("B,H,W,C_lo,C_hi,N,stride", [(2, 16, 16, 160, 96, 136, 1), (1, 8, 16, 32, 32, 16, 1), (4, 16, 16, 384, 256, 1280, 1),
+                                                      (2, 32, 32, 128, 640, 328, 2)])
+def test_two_branches_conv3x3(bits, B, H, W, C_lo, C_hi, N, stride):
+    split._run_conv(B, H, W, C_lo, C_hi, N, bits, stride, seed=H + C_lo + N)
