@@ -72,9 +72,10 @@ int mixdq_int8_tile_plan(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int
                          int* reduction_splits);
 
 /* Diagnostic (the paper has no counterpart): the tile of the channel-major form (output channels on the rows of the
- * tensor-core tile), which runs layers whose tiles fit the SMs at once: *tile_channels is 128, or 256 when two CTAs
- * share a tile, *tile_tokens a multiple of 16 per CTA; both 0 where the tiles of mixdq_int8_tile_plan are faster.
- * Arguments as there.  Taken with a workspace by every int8 layer but the second branch of a shortcut-split layer.
+ * tensor-core tile), which runs layers whose tiles fit the SMs at once and int4 layers of several waves:
+ * *tile_channels is 128, or 256 when two CTAs share a tile, *tile_tokens a multiple of 16 per CTA; both 0 where the
+ * tiles of mixdq_int8_tile_plan are faster.  Arguments as there.  Taken with a workspace by every int8 layer but the
+ * second branch of a shortcut-split layer; the BOS-aware projection and split layers only where one wave suffices.
  * Nothing is launched. */
 int mixdq_int8_chan_tile(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int* tile_channels, int* tile_tokens);
 

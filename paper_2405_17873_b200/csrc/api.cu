@@ -212,9 +212,9 @@ extern "C" int mixdq_int8_chan_tile(int64_t M, int64_t N, int64_t k_blocks, int 
     if (w_bits != 4 && w_bits != 8) return MIXDQ_ERR_UNSUPPORTED;
     const int sms = sm_count();
     if (sms <= 0) return MIXDQ_ERR_CUDA;
-    int cg = 1;
-    *tile_tokens = i8::plan_chan_tile(static_cast<int>(M), static_cast<int>(N), static_cast<int>(k_blocks), w_bits == 4, sms, &cg);
-    *tile_channels = *tile_tokens > 0 ? 128 * cg : 0;
+    const i8::ChanPlan plan = i8::plan_chan(static_cast<int>(M), static_cast<int>(N), static_cast<int>(k_blocks), w_bits == 4, sms);
+    *tile_tokens = plan.tokens;
+    *tile_channels = 128 * plan.cg;
     return MIXDQ_OK;
 }
 

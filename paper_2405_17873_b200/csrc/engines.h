@@ -78,8 +78,6 @@ int run_quant(const __half* X, long long ldx, long long rows, int K, const float
 int run_tma_prequantized(const Params& p, int amode, const void* packed, int w_bits, const int8_t* aq,
                          cudaStream_t stream);
 // Channel-major form (i8_chan.cu) on int8 codes: tiles of 128 cg channels x `tokens` tokens on cg = 1 or 2 CTAs.
-// plan_chan_tile: its tile's tokens where it is the fastest form for the layer, else 0; two: for both branches of a
-// shortcut-split layer at once (k_blocks of both), whose tile has at most CHAN_TWO_TOKENS.
 constexpr int CHAN_TWO_TOKENS = 128;
 struct ChanBranch {
     const void* packed;
@@ -89,9 +87,18 @@ struct ChanBranch {
     int32_t* acc_out;
 };
 bool chan_tile_ok(int cg, int tokens);
-int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg, bool two = false);
 int run_chan(const Params& p, int amode, const void* packed, int w_bits, const int8_t* codes, int cg, int tokens, cudaStream_t stream,
              const ChanBranch* second = nullptr);
+// The same for int4 layers of several waves (i8_chan_many.cu): CTA pairs walk tiles of 256 channels x `tokens` tokens.
+bool chan_many_tile_ok(int tokens, int k_blocks);
+int run_chan_many(const Params& p, int amode, const void* packed, const int8_t* codes, int tokens, int num_sms, cudaStream_t stream);
+// The channel-major form that is the fastest for the layer, if one is (tokens 0: none).  two: for both branches of a
+// shortcut-split layer at once (k_blocks of both), whose tile has at most CHAN_TWO_TOKENS.
+struct ChanPlan {
+    int tokens = 0, cg = 0;
+    bool many = false;  // run_chan_many
+};
+ChanPlan plan_chan(int M, int N, int k_blocks, bool w4, int num_sms, bool two = false, bool many_ok = true);
 // Shortcut-splitting (one activation scale per branch of a concatenated input): row elements [0, split_at)
 // and [split_at, row_len) are quantized, multiplied and summed separately and meet in a two-scale epilogue.
 // Linear layers and 3x3 convolutions whose halves both suit the two-kernel path.

@@ -32,15 +32,13 @@
 #include <algorithm>
 #include <cmath>
 
-#include "cta_pair.cuh"
-#include "i8_tiles.cuh"
+#include "i8_chan.cuh"
 
 namespace mixdq {
 namespace i8 {
 
 namespace {
 
-constexpr int CH = 128;        // channels of one CTA
 constexpr int TOK_MAX = 256;   // tokens of a tile
 constexpr int ROWS_MAX = 128;  // token rows of one CTA
 constexpr int EXP_GROUPS = 3;  // of four warps: expansion (W4), then epilogue
@@ -108,33 +106,6 @@ struct Pairs {
     }
 };
 
-// A load that stays where it is written (the compiler moves plain read-only loads down to their first use, past the
-// barriers these are meant to overlap).
-__device__ __forceinline__ float ld_pinned(const float* p)
-{
-    float v;
-    asm volatile("ld.global.nc.f32 %0, [%1];" : "=f"(v) : "l"(p));
-    return v;
-}
-
-template <int CG>
-__device__ __forceinline__ void arrive_at_leader(uint32_t bar)
-{
-    if (CG == 1)
-        mbar_arrive(bar);
-    else
-        mbar_arrive_cluster(bar);
-}
-
-template <int CG>
-__device__ __forceinline__ void commit_mmas(uint32_t bar)
-{
-    if (CG == 1)
-        tc_commit(bar);
-    else
-        tc_commit_pair(bar, 3);
-}
-
 // Waits until the MMAs of the pair of k-block `was` have finished.
 template <class L>
 __device__ __forceinline__ bool wait_mmas(uint32_t bar0, int was, volatile int* abort_flag)
@@ -142,22 +113,6 @@ __device__ __forceinline__ bool wait_mmas(uint32_t bar0, int was, volatile int* 
     const uint32_t q = static_cast<uint32_t>(was) >> 1;
     return mbar_wait(bar0 + 8 * (L::EMPTY + q % L::NE), (q / L::NE) & 1, abort_flag);
 }
-
-// Where a k-block lies: reduction elements [c * BK, ...) of filter tap `tap` (a linear layer is one endless tap).
-struct KPos {
-    int tap, c;
-    __device__ __forceinline__ KPos(int i, int cblocks) : tap(0), c(i)
-    {
-        if (i >= cblocks) {  // (not for a linear layer: a division takes 120 cycles of the first request's way)
-            tap = i / cblocks;
-            c = i - tap * cblocks;
-        }
-    }
-    __device__ __forceinline__ void advance(int n, int cblocks)
-    {
-        for (c += n; c >= cblocks; c -= cblocks) ++tap;
-    }
-};
 
 // A TMA producer, one of two warps that take alternate units, pairs of k-blocks; request(slot, barrier, unit,
 // position) asks for one.  A warp that runs alone takes some five cycles per instruction, so a
@@ -199,50 +154,6 @@ __device__ __forceinline__ void produce(int which, int lane, int slots, const Pa
         if (q >= barriers) {
             q -= barriers;
             par ^= 1;
-        }
-    }
-}
-
-// One warp's share of the epilogue: its 32 lanes' channels x every third group of eight tokens.  Lanes 2 i and 2 i + 1 swap
-// halves of a packed token pair and each stores both channels of one token: a store covers 64 contiguous bytes of two
-// output rows.  col: Y at the lane's channel pair.
-template <bool TWO>
-__device__ __forceinline__ void store_tokens(uint32_t acc, uint32_t acc2, int c0, int cols, float comb, float comb2, float bias,
-                                             __half* col, long long ldy, int tok0, int M, bool in_n, bool bos, int lane)
-{
-    const uint32_t sel = (lane & 1) ? 0x3276u : 0x5410u;  // odd: token 1 (other's, own); even: token 0 (own, other's)
-    const bool all_n = __all_sync(0xffffffffu, in_n);
-    for (; c0 < cols; c0 += 8 * EXP_GROUPS) {
-        uint32_t r[8], r2[8], own[4], out[4];
-        tmem_ld_32x8(acc + c0, r);
-        if (TWO) tmem_ld_32x8(acc2 + c0, r2);
-        tmem_ld_wait();
-        const int m0 = tok0 + c0 + (lane & 1);
-#pragma unroll
-        for (int j = 0; j < 4; ++j) {
-            float a = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j])), comb, bias);
-            float b = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j + 1])), comb, bias);
-            if (TWO) {
-                a = fmaf(__int2float_rn(static_cast<int32_t>(r2[2 * j])), comb2, a);
-                b = fmaf(__int2float_rn(static_cast<int32_t>(r2[2 * j + 1])), comb2, b);
-            }
-            const __half2 h = __floats2half2_rn(a, b);
-            own[j] = *reinterpret_cast<const uint32_t*>(&h);
-        }
-#pragma unroll
-        for (int j = 0; j < 4; ++j) out[j] = __byte_perm(own[j], __shfl_xor_sync(0xffffffffu, own[j], 1), sel);
-        if (all_n && !bos && c0 + 8 <= cols) {  // (uniform: the whole group of tokens exists)
-            __half* dst = col + m0 * ldy;
-#pragma unroll
-            for (int j = 0; j < 4; ++j) *reinterpret_cast<uint32_t*>(dst + 2 * j * ldy) = out[j];
-        } else if (in_n) {
-#pragma unroll
-            for (int j = 0; j < 4; ++j) {
-                int m = m0 + 2 * j;
-                if (m >= M) continue;
-                if (bos) m += m / (MIXDQ_TOKENS_PER_PROMPT - 1) + 1;
-                *reinterpret_cast<uint32_t*>(col + m * ldy) = out[j];
-            }
         }
     }
 }
@@ -449,45 +360,23 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         const int group = (warp - WORK0) >> 2, row = (warp & 3) * 32 + lane;
         constexpr uint32_t PS = L::PS > 0 ? L::PS : 1;
         const uint32_t a_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + g.a_col;
-        const uint8_t* base = smem + L::OFF_W + row * (g.wide ? 128 : 64);
-        const uint32_t swz = g.wide ? (static_cast<uint32_t>(row) & 7u) << 4 : (static_cast<uint32_t>(row >> 1) & 3u) << 4;
-        const uint32_t second = g.wide ? 64u : L::P_BYTES / 2;  // from a row of the first k-block to the second's
+        const PackedRows rows_of(row, g.wide);
         int sw = 2 * group;  // slot of the pair's first k-block
         if (sw >= g.w_slots) sw -= g.w_slots;
         uint4 w[8];
         auto fetch = [&](int j) {
             const uint32_t q = static_cast<uint32_t>(j), sp = q % PS;
             const bool ok = mbar_wait(bar0 + 8 * (L::FULL_P + sp), (q / PS) & 1, abort_flag);
-            const uint8_t* src = base + sp * L::P_BYTES;
-#pragma unroll
-            for (int k = 0; k < 8; ++k) {
-                // (wide: the second k-block is chunks 4 .. 7 of the row, and the swizzle runs over all eight)
-                const uint32_t off = static_cast<uint32_t>(k & 3) << 4;
-                w[k] = *reinterpret_cast<const uint4*>(src + (k < 4 ? off ^ swz : (g.wide ? (off | 64u) ^ swz : (off ^ swz) + second)));
-            }
+            rows_of.load(smem + L::OFF_W + sp * L::P_BYTES, w);
             return ok;
-        };
-        auto expand = [&](int h) {
-            uint32_t c[32];
-#pragma unroll
-            for (int k = 0; k < 4; ++k) {
-                const uint4& v4 = w[4 * h + k];
-                const uint32_t v[4] = {v4.x, v4.y, v4.z, v4.w};
-#pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    c[8 * k + 2 * q] = (v[q] << 4) & 0xF0F0F0F0u;
-                    c[8 * k + 2 * q + 1] = v[q] & 0xF0F0F0F0u;
-                }
-            }
-            tmem_st_32x32(a_lane + (sw + h) * 32, c);
         };
         bool ok = group < pairs ? fetch(group) : true;
         for (int j = group; j < pairs; j += EXP_GROUPS) {
             if (ok && 2 * j >= g.w_slots) ok = wait_mmas<L>(bar0, 2 * j - g.w_slots, abort_flag);
             if (!__all_sync(0xffffffffu, ok)) break;  // the warp leaves together
             tc_fence_after_sync();
-            expand(0);
-            if (pr.both(j)) expand(1);
+            expand_row(w, a_lane + sw * 32);
+            if (pr.both(j)) expand_row(w + 4, a_lane + (sw + 1) * 32);
             __syncwarp();
             if (lane == 0) mbar_arrive(bar0 + 8 * (L::EMPTY_P + static_cast<uint32_t>(j) % PS));
             tmem_st_wait();
@@ -509,7 +398,7 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         __syncwarp();
         asm volatile("bar.sync 1, %0;" ::"n"(32 * (WORKERS + 1)) : "memory");
     } else if (warp >= WORK0 && warp < HELP0) {
-        // ------------------------------------------------------------ epilogue: twelve warps, 8 tokens at a time
+        // ------------------------------------------------------------ epilogue: twelve warps
         const int n = n0 + (warp & 3) * 32 + lane;  // this lane's channel
         float comb = 0.f, comb2 = 0.f, bias = 0.f;
         int zterm = 0;  // (128 - zero) * sum of the channel's weight codes
@@ -536,8 +425,14 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
         const bool pairs_ok = ((p.N | static_cast<int>(p.ldy)) & 1) == 0 && (reinterpret_cast<uintptr_t>(p.Y) & 3) == 0;
         const int cols = min(g.nt, p.M - tok0);
         if (ok && p.Y && pairs_ok && !p.acc_out) {
-            store_tokens<TWO>(acc, acc + g.acc2, ((warp - WORK0) >> 2) * 8, cols, comb, comb2, bias, p.Y + (n & ~1), p.ldy, tok0, p.M,
-                              n < p.N, p.bos != 0, lane);
+            const int who = (warp - WORK0) >> 2;
+            __half* col = p.Y + (n & ~1);
+            if (cols > 32)
+                store_tokens<TWO, 16>(acc, acc + g.acc2, 16 * who, 16 * EXP_GROUPS, cols, comb, comb2, bias, col, p.ldy, tok0, p.M, n < p.N,
+                                      p.bos != 0, lane);
+            else
+                store_tokens<TWO, 8>(acc, acc + g.acc2, 8 * who, 8 * EXP_GROUPS, cols, comb, comb2, bias, col, p.ldy, tok0, p.M, n < p.N,
+                                     p.bos != 0, lane);
         } else if (ok) {
             // odd widths, and the raw sums of the parity hook
             for (int c0 = ((warp - WORK0) >> 2) * 8; c0 < cols; c0 += 8 * EXP_GROUPS) {
@@ -606,9 +501,11 @@ int launch(const CUtensorMap* maps, const TmaParams& tp, const ChanArgs& g, int 
     return w4 ? launch_t<1, true, TWO>(maps, tp, g, stream) : launch_t<1, false, TWO>(maps, tp, g, stream);
 }
 
+}  // namespace
+
 // Tensor maps of one branch: its weights [N, taps * cin] and its activations, int8 [M, cin] or the NHWC image of cin channels
 // (with its border when pad is set).
-int encode_branch(CUtensorMap* tw, CUtensorMap* tx, const Params& p, bool conv, int pad, int cin, const void* packed, bool w4, bool wide,
+int encode_chan_branch(CUtensorMap* tw, CUtensorMap* tx, const Params& p, bool conv, int pad, int cin, const void* packed, bool w4, bool wide,
                   const int8_t* codes, int rows)
 {
     const int64_t K = (conv ? 9ll : 1ll) * cin;
@@ -621,8 +518,6 @@ int encode_branch(CUtensorMap* tw, CUtensorMap* tx, const Params& p, bool conv, 
     return encode_tmap_2d_u8(tx, codes, static_cast<uint64_t>(cin), static_cast<uint64_t>(p.M), static_cast<uint64_t>(cin), BK,
                              static_cast<uint32_t>(rows), SWIZZLE_128);
 }
-
-}  // namespace
 
 bool chan_tile_ok(int cg, int tokens)
 {
@@ -669,10 +564,10 @@ int run_chan(const Params& p, int amode, const void* packed, int w_bits, const i
         tp.Wo = p.Wo;
     }
     CUtensorMap maps[4]{};  // weights, activations; the second branch's
-    int rc = encode_branch(&maps[0], &maps[1], p, conv, pad, cin, packed, w4, g.wide, codes, rows);
+    int rc = encode_chan_branch(&maps[0], &maps[1], p, conv, pad, cin, packed, w4, g.wide, codes, rows);
     if (rc != MIXDQ_OK) return rc;
     if (!second) return launch<false>(maps, tp, g, cg, w4, stream);
-    rc = encode_branch(&maps[2], &maps[3], p, conv, pad, second->cin, second->packed, w4, g.wide, second->codes, rows);
+    rc = encode_chan_branch(&maps[2], &maps[3], p, conv, pad, second->cin, second->packed, w4, g.wide, second->codes, rows);
     if (rc != MIXDQ_OK) return rc;
     g.kb_lo = tp.k_blocks;
     g.cblocks2 = static_cast<int>(ceil_div(second->cin, BK));

@@ -1210,8 +1210,8 @@ int plan_pair_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* splits
     return t.pair_bn;
 }
 
-// Channel-major form (i8_chan.cu): its tile's tokens, or 0 where the forms with the tokens on the rows are faster.  The
-// kernel runs one tile per CTA or CTA pair, so the tiles have to fit the SMs at once; a second wave costs more than the
+// Channel-major forms: which, and its tile, or none where the forms with the tokens on the rows are faster.  The one of
+// i8_chan.cu runs one tile per CTA or CTA pair, so the tiles have to fit the SMs at once; a second wave costs more than the
 // form gains (4096 x 1280 x 640 int4: 11.3 us against 10.1).  Cycles of a tile of t tokens, from a fit to 104 layers (16 to
 // 16384 rows, 320 to 2560 channels, 3 to 180 k-blocks, linear and convolution; every tile that fits one wave; mean error
 // 5 per cent): fixed part + k-blocks x (issue + t) + epilogue of the tokens, where the share of the SMs in use slows each
@@ -1221,11 +1221,11 @@ int plan_pair_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* splits
 //   * int8 weights on pairs of more than 192 tokens leave room for four activation slots only: half the speed.
 //   * The other forms' estimates were six per cent short on these layers; the single-CTA kernels' split reductions measured
 //     5000 cycles over theirs, the pair form's ten per cent under.
-int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg, bool two)
+ChanPlan plan_chan(int M, int N, int k_blocks, bool w4, int num_sms, bool two, bool many_ok)
 {
     const double nkb = k_blocks;
     double best = 0;
-    int best_tokens = 0;
+    ChanPlan r;
     for (int c = 1; c <= 2; ++c) {
         const int64_t c_tiles = ceil_div(N, 128 * c);
         for (int t = 16 * c; t <= (c == 2 && !w4 ? 192 : 128 * c); t += 16 * c) {
@@ -1237,19 +1237,35 @@ int plan_chan_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* cg, bo
             const double per_kb = c == 1 ? (w4 ? 160.0 + 1.0 * t : 114.0 + 2.2 * t) : (w4 ? 72.0 + 1.5 * t : 96.0 + 1.4 * t);
             const double cost = (w4 ? 3750.0 + 200.0 * c : 4500.0) + nkb * (per_kb + 72.0 * busy) + 15.0 * t +
                                 (c == 1 ? 1530.0 : 3300.0) * busy;
-            if (best_tokens == 0 || cost < best) {
+            if (r.tokens == 0 || cost < best) {
                 best = cost;
-                best_tokens = t;
-                *cg = c;
+                r.tokens = t;
+                r.cg = c;
             }
         }
     }
-    if (best_tokens == 0) return 0;
+    // Pairs that walk several tiles (i8_chan_many.cu, int4).  Fitted to 24 layers of one to twelve rounds, tiles of 96 to 256
+    // tokens: a k-block costs what its MMAs take (two cycles a token, never under 310), a tile's epilogue 900 + 15.5 cycles a
+    // token, beside the next tile's main loop where there are two accumulators (up to 192 tokens), else after its own.
+    const int pairs = num_sms / 2;
+    for (int t = 96; many_ok && w4 && !two && pairs > 0 && t <= 256; t += 32) {
+        if (!chan_many_tile_ok(t, k_blocks)) break;
+        const double rounds = std::ceil(static_cast<double>(ceil_div(N, 256) * ceil_div(M, t)) / pairs);
+        const double main = nkb * std::max(310.0, 2.1 * t + 20.0), epi = 900.0 + 15.5 * t;
+        const double cost = 7400.0 + (t > 192 ? rounds * (main + epi) : std::max(rounds * main + epi, main + rounds * epi));
+        if (r.tokens == 0 || cost < best) {
+            best = cost;
+            r.tokens = t;
+            r.cg = 2;
+            r.many = true;
+        }
+    }
+    if (r.tokens == 0) return r;
     const TokenPlan o = token_plan(M, N, k_blocks, w4, num_sms, !two);
     const double single = o.single_cost + (o.single_splits > 1 ? 5000.0 : 0.0);
     const bool pair = o.pair_bn > 0 && o.pair_cost < 1.05 * single;
     const double other = pair ? o.pair_cost * (o.pair_splits > 1 ? 0.9 : 1.0) : single;
-    return best < 1.06 * other ? best_tokens : 0;
+    return best < 1.06 * other ? r : ChanPlan{};
 }
 
 // Fused-quantization kernel (i8_fq.cu) or the two-kernel forms.  The fused kernel's k-block costs three to four
@@ -1374,8 +1390,7 @@ int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* sc
         // Below 2048 rows the quantization pass is short (1.7 us for 1024 x 640) and the channel-major GEMM after it makes
         // up for it: 1024 x 640 x 640 W4 5.2 us against 8.2, W8 5.4 against 6.6.  From there on they come out equal (4096 x
         // 640 x 640 W4: 9.2 and 9.3 us) or the fused kernel ahead (W8 9.2 and 7.5, K = 320 8.0 and 7.1).
-        int cg;
-        if (fq_bn > 0 && (p.M >= 2048 || plan_chan_tile(p.M, p.N, kb, w_bits == 4, num_sms, &cg) == 0))
+        if (fq_bn > 0 && (p.M >= 2048 || plan_chan(p.M, p.N, kb, w_bits == 4, num_sms).tokens == 0))
             return run_fq(p, packed, w_bits, fq_bn, stream);
     }
 
@@ -1407,10 +1422,10 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
     const int num_sms = sm_count();
     if (num_sms <= 0) return MIXDQ_ERR_CUDA;
     if (!p.addend && !p.test_drop_b_kblock) {
-        int cg = 1;
         const int kb = static_cast<int>(conv ? 9 * ceil_div(p.Cin, BK) : ceil_div(p.K, BK));
-        const int tokens = plan_chan_tile(p.M, p.N, kb, w4, num_sms, &cg);
-        if (tokens > 0) return run_chan(p, amode, packed, w_bits, aq, cg, tokens, stream);
+        const ChanPlan plan = plan_chan(p.M, p.N, kb, w4, num_sms, false, amode != A_BOS);
+        if (plan.many) return run_chan_many(p, amode, packed, aq, plan.tokens, num_sms, stream);
+        if (plan.tokens > 0) return run_chan(p, amode, packed, w_bits, aq, plan.cg, plan.tokens, stream);
     }
 
     // 2. tensor maps
@@ -1604,16 +1619,15 @@ int run_tma_split(const Params& p, int amode, int split_at, const void* packed_l
     const int c_lo = split_at, c_hi = row_len - split_at;
     const int kb_lo = static_cast<int>(conv ? 9 * ceil_div(c_lo, BK) : ceil_div(c_lo, BK));
     const int kb_hi = static_cast<int>(conv ? 9 * ceil_div(c_hi, BK) : ceil_div(c_hi, BK));
-    int cg;
-    const int tokens = plan_chan_tile(p.M, p.N, kb_lo + kb_hi, w4, num_sms, &cg, true);
-    if (tokens > 0) {
+    const ChanPlan plan = plan_chan(p.M, p.N, kb_lo + kb_hi, w4, num_sms, true);
+    if (plan.tokens > 0) {
         Params q = p;
         q.Cin = conv ? c_lo : 0;
         q.K = conv ? 9 * c_lo : c_lo;
         q.act_scale = scale_lo;
         q.acc_out = p.Y ? nullptr : acc_lo_out;
         const ChanBranch second{packed_hi, aq_hi, c_hi, scale_hi, p.Y ? nullptr : acc_hi_out};
-        return run_chan(q, amode, packed_lo, w_bits, aq_lo, cg, tokens, stream, &second);
+        return run_chan(q, amode, packed_lo, w_bits, aq_lo, plan.cg, plan.tokens, stream, &second);
     }
     const int pair_bn = plan_pair_tile(p.M, p.N, kb_lo + kb_hi, w4, num_sms, nullptr);
     if (pair_bn > 0) {

@@ -120,3 +120,31 @@ def test_two_branches_linear(bits, M, C_lo, C_hi, N):
                                                       (2, 32, 32, 128, 640, 328, 2)])
 def test_two_branches_conv3x3(bits, B, H, W, C_lo, C_hi, N, stride):
     split._run_conv(B, H, W, C_lo, C_hi, N, bits, stride, seed=H + C_lo + N)
+
+
+# int4 layers of several waves: a CTA pair's tiles follow each other through the rings, on one accumulator and on two
+@pytest.mark.parametrize("M,N,K", [(3000, 5124, 272), (2050, 5121, 656), (4500, 2564, 1296), (1024, 10240, 1280), (4100, 1800, 5136)])
+def test_linear_of_several_waves(M, N, K):
+    channels, tokens = mixdq.int8_chan_tile(M, N, -(-K // 128), 4)
+    assert channels == 256 and -(-M // tokens) * -(-N // 256) > 74
+    X, W, b = _layer(M, N, K)
+    X = synth.one_sided_f16((M, K), seed=5, shift=0.3)
+    s_ref, _, codes = oracle_weights(W, 4, True)
+    sa_ref, z_ref = orc.act_minmax_params(X)
+    acc_ref, y_ref = orc.linear_a8_asym(X, codes, s_ref, sa_ref, z_ref, b)
+    Xd = dev(X)
+    s, _, packed = device_weights(W, 4, True)
+    sums = mixdq.weight_code_sums(packed, N, K, 4)
+    sa, z = mixdq.act_asym_params(Xd)
+    ws, st = mixdq.new_workspace(mixdq.workspace_bytes(M, N, K, 4, 8)), status_word()
+    acc = mixdq.linear_a8_asym_acc_i32(Xd, packed, N, 4, sums, sa, z, workspace=ws, status=st)
+    y = mixdq.linear_a8_asym(Xd, packed, N, 4, s, sums, sa, z, dev(b), ws, st)
+    torch.cuda.synchronize()
+    assert int(host(st)[0]) == 0
+    assert np.array_equal(host(acc), acc_ref)
+    assert_close(host(y), y_ref)
+
+
+@pytest.mark.parametrize("B,H,W,Cin,Cout,stride", [(4, 64, 64, 320, 320, 1), (3, 65, 63, 96, 648, 1), (2, 96, 97, 128, 1284, 2)])
+def test_conv3x3_of_several_waves(B, H, W, Cin, Cout, stride):
+    test_conv3x3(4, B, H, W, Cin, Cout, stride)
