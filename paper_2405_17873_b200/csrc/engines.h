@@ -135,6 +135,10 @@ int run(Params p, int amode, const void* packed, int w_bits, cudaStream_t stream
 size_t expanded_weight_bytes(int64_t N, int64_t K);
 bool pair_path_ok(const Params& p, int amode, int w_bits);
 int run_pair(const Params& p, int amode, const void* packed, int w_bits, cudaStream_t stream);
+// One wave of channel-major tiles, 128 cg channels x `tokens` tokens, no workspace; see wo_chan.cu.
+bool chan_tile_ok(int cg, int tokens);
+bool chan_path_ok(const Params& p, int amode, int w_bits);
+int run_chan(const Params& p, int amode, const void* packed, int w_bits, int cg, int tokens, cudaStream_t stream);
 // Many-token path on tcgen05 (fp16 MMA, weights expanded into shared memory); see wo_tc.cu.
 bool tc_path_ok(const Params& p, int amode, int w_bits);
 int run_tc(const Params& p, int amode, const void* packed, int w_bits, int batch, cudaStream_t stream);

@@ -90,72 +90,12 @@ struct ChanArgs {
     int32_t* acc_out2;
 };
 
-// The k-blocks of a tile as pairs; with two branches each branch's pairs start at its own first k-block.
-template <bool TWO>
-struct Pairs {
-    int nkb, lo, kb_lo, n;  // k-blocks; TWO: pairs and k-blocks of the first branch; pairs in all
-    __device__ __forceinline__ Pairs(int nkb_, int kb_lo_)
-        : nkb(nkb_), lo(TWO ? (kb_lo_ + 1) >> 1 : 0), kb_lo(kb_lo_), n(TWO ? lo + ((nkb_ - kb_lo_ + 1) >> 1) : (nkb_ + 1) >> 1)
-    {
-    }
-    __device__ __forceinline__ bool second(int j) const { return TWO && j >= lo; }
-    __device__ __forceinline__ bool both(int j) const  // whether the pair has two k-blocks
-    {
-        if (!TWO) return 2 * j + 1 < nkb;
-        return j < lo ? 2 * j + 1 < kb_lo : 2 * (j - lo) + 1 < nkb - kb_lo;
-    }
-};
-
 // Waits until the MMAs of the pair of k-block `was` have finished.
 template <class L>
 __device__ __forceinline__ bool wait_mmas(uint32_t bar0, int was, volatile int* abort_flag)
 {
     const uint32_t q = static_cast<uint32_t>(was) >> 1;
     return mbar_wait(bar0 + 8 * (L::EMPTY + q % L::NE), (q / L::NE) & 1, abort_flag);
-}
-
-// A TMA producer, one of two warps that take alternate units, pairs of k-blocks; request(slot, barrier, unit,
-// position) asks for one.  A warp that runs alone takes some five cycles per instruction, so a
-// loop over k-blocks costs 370 cycles a turn whatever the size of the request, and an integer division in it 120 more.
-// Hence the two warps and the running position, and the first lap of the ring, which waits for nothing, goes out from all
-// lanes of the first of them at once (65 cycles apart).  free[unit % barriers] says that the slot of the unit `slots`
-// positions later is free; `barriers` is even and at least `slots`: a warp meets every phase.
-template <bool TWO, typename F>
-__device__ __forceinline__ void produce(int which, int lane, int slots, const Pairs<TWO>& pr, int cblocks, int cblocks2, uint32_t free,
-                                        int barriers, volatile int* abort_flag, F&& request)
-{
-    const int units = pr.n;
-    if (which == 0 && lane < slots && lane < units)
-        request(lane, lane, lane, pr.second(lane) ? KPos(2 * (lane - pr.lo), cblocks2) : KPos(2 * lane, cblocks));
-    __syncwarp();
-    if (slots + which >= units) return;
-    int s = which, q = which, sb = which + slots;
-    if (s >= slots) s -= slots;
-    if (sb >= barriers) sb -= barriers;
-    uint32_t par = 0;
-    KPos at(2 * (slots + which), cblocks);
-    bool second = false;
-    for (int i = slots + which; i < units; i += 2) {
-        if (TWO && !second && pr.second(i)) {
-            second = true;
-            cblocks = cblocks2;
-            at = KPos(2 * (i - pr.lo), cblocks2);
-        }
-        const bool ok = mbar_wait(free + 8 * q, par, abort_flag);
-        if (!__all_sync(0xffffffffu, ok)) break;
-        if (elect_one()) request(s, sb, i, at);
-        __syncwarp();
-        at.advance(4, cblocks);
-        s += 2;
-        while (s >= slots) s -= slots;
-        sb += 2;
-        if (sb >= barriers) sb -= barriers;
-        q += 2;
-        if (q >= barriers) {
-            q -= barriers;
-            par ^= 1;
-        }
-    }
 }
 
 // Grid: CG CTAs (a cluster) per tile of 128 CG channels x nt tokens, channel tiles fastest.
@@ -428,10 +368,10 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             const int who = (warp - WORK0) >> 2;
             __half* col = p.Y + (n & ~1);
             if (cols > 32)
-                store_tokens<TWO, 16>(acc, acc + g.acc2, 16 * who, 16 * EXP_GROUPS, cols, comb, comb2, bias, col, p.ldy, tok0, p.M, n < p.N,
+                store_tokens<TWO ? ACC_TWO_BRANCHES : ACC_INT, 16>(acc, acc + g.acc2, 16 * who, 16 * EXP_GROUPS, cols, comb, comb2, bias, col, p.ldy, tok0, p.M, n < p.N,
                                       p.bos != 0, lane);
             else
-                store_tokens<TWO, 8>(acc, acc + g.acc2, 8 * who, 8 * EXP_GROUPS, cols, comb, comb2, bias, col, p.ldy, tok0, p.M, n < p.N,
+                store_tokens<TWO ? ACC_TWO_BRANCHES : ACC_INT, 8>(acc, acc + g.acc2, 8 * who, 8 * EXP_GROUPS, cols, comb, comb2, bias, col, p.ldy, tok0, p.M, n < p.N,
                                      p.bos != 0, lane);
         } else if (ok) {
             // odd widths, and the raw sums of the parity hook

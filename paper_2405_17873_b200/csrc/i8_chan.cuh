@@ -1,5 +1,5 @@
 // Parts shared by the channel-major int8 kernels (i8_chan.cu: one tile per CTA or CTA pair; i8_chan_many.cu: pairs that walk
-// several tiles).
+// several tiles; wo_chan.cu: fp16 activations).
 #pragma once
 
 #include "cta_pair.cuh"
@@ -52,6 +52,66 @@ struct KPos {
         for (c += n; c >= cblocks; c -= cblocks) ++tap;
     }
 };
+
+// The k-blocks of a tile as pairs; with two branches each branch's pairs start at its own first k-block.
+template <bool TWO>
+struct Pairs {
+    int nkb, lo, kb_lo, n;  // k-blocks; TWO: pairs and k-blocks of the first branch; pairs in all
+    __device__ __forceinline__ Pairs(int nkb_, int kb_lo_)
+        : nkb(nkb_), lo(TWO ? (kb_lo_ + 1) >> 1 : 0), kb_lo(kb_lo_), n(TWO ? lo + ((nkb_ - kb_lo_ + 1) >> 1) : (nkb_ + 1) >> 1)
+    {
+    }
+    __device__ __forceinline__ bool second(int j) const { return TWO && j >= lo; }
+    __device__ __forceinline__ bool both(int j) const  // whether the pair has two k-blocks
+    {
+        if (!TWO) return 2 * j + 1 < nkb;
+        return j < lo ? 2 * j + 1 < kb_lo : 2 * (j - lo) + 1 < nkb - kb_lo;
+    }
+};
+
+// A TMA producer, one of two warps that take alternate units, pairs of k-blocks; request(slot, barrier, unit,
+// position) asks for one.  A warp that runs alone takes some five cycles per instruction, so a
+// loop over k-blocks costs 370 cycles a turn whatever the size of the request, and an integer division in it 120 more.
+// Hence the two warps and the running position, and the first lap of the ring, which waits for nothing, goes out from all
+// lanes of the first of them at once (65 cycles apart).  free[unit % barriers] says that the slot of the unit `slots`
+// positions later is free; `barriers` is even and at least `slots`: a warp meets every phase.
+template <bool TWO, typename F>
+__device__ __forceinline__ void produce(int which, int lane, int slots, const Pairs<TWO>& pr, int cblocks, int cblocks2, uint32_t free,
+                                        int barriers, volatile int* abort_flag, F&& request)
+{
+    const int units = pr.n;
+    if (which == 0 && lane < slots && lane < units)
+        request(lane, lane, lane, pr.second(lane) ? KPos(2 * (lane - pr.lo), cblocks2) : KPos(2 * lane, cblocks));
+    __syncwarp();
+    if (slots + which >= units) return;
+    int s = which, q = which, sb = which + slots;
+    if (s >= slots) s -= slots;
+    if (sb >= barriers) sb -= barriers;
+    uint32_t par = 0;
+    KPos at(2 * (slots + which), cblocks);
+    bool second = false;
+    for (int i = slots + which; i < units; i += 2) {
+        if (TWO && !second && pr.second(i)) {
+            second = true;
+            cblocks = cblocks2;
+            at = KPos(2 * (i - pr.lo), cblocks2);
+        }
+        const bool ok = mbar_wait(free + 8 * q, par, abort_flag);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        if (elect_one()) request(s, sb, i, at);
+        __syncwarp();
+        at.advance(4, cblocks);
+        s += 2;
+        while (s >= slots) s -= slots;
+        sb += 2;
+        if (sb >= barriers) sb -= barriers;
+        q += 2;
+        if (q >= barriers) {
+            q -= barriers;
+            par ^= 1;
+        }
+    }
+}
 
 // The packed int4 rows of a pair of k-blocks as they lie in shared memory: 128-byte rows (both k-blocks of a channel, 128-byte
 // swizzle) where the pair is contiguous in memory, else two tiles of 64-byte rows (64-byte swizzle).  The swizzle makes the
@@ -106,7 +166,12 @@ __device__ __forceinline__ void tmem_ld_tokens(uint32_t taddr, uint32_t (&r)[G])
 // swap halves of a packed token pair and each stores both channels of one token: a store covers 64 contiguous bytes of two
 // output rows.  col: Y at the lane's channel pair.  A turn is bound by its latencies (tensor-memory load, conversions, swap):
 // sixteen tokens a turn where there are enough of them.
-template <bool TWO, int G>
+enum : int {
+    ACC_INT = 0,           // y = acc * comb + bias
+    ACC_TWO_BRANCHES = 1,  // y = acc2 * comb2 + (acc * comb + bias)
+    ACC_FLOAT = 2,         // fp32 sums in two accumulators: y = (acc + acc2) * comb + bias
+};
+template <int KIND, int G>
 __device__ __forceinline__ void store_tokens(uint32_t acc, uint32_t acc2, int c0, int step, int cols, float comb, float comb2, float bias,
                                              __half* col, long long ldy, int tok0, int M, bool in_n, bool bos, int lane)
 {
@@ -115,14 +180,20 @@ __device__ __forceinline__ void store_tokens(uint32_t acc, uint32_t acc2, int c0
     for (; c0 < cols; c0 += step) {
         uint32_t r[G], r2[G], own[G / 2];
         tmem_ld_tokens<G>(acc + c0, r);
-        if (TWO) tmem_ld_tokens<G>(acc2 + c0, r2);
+        if (KIND != ACC_INT) tmem_ld_tokens<G>(acc2 + c0, r2);
         tmem_ld_wait();
         const int m0 = tok0 + c0 + (lane & 1);
 #pragma unroll
         for (int j = 0; j < G / 2; ++j) {
-            float a = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j])), comb, bias);
-            float b = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j + 1])), comb, bias);
-            if (TWO) {
+            float a, b;
+            if (KIND == ACC_FLOAT) {
+                a = fmaf(__uint_as_float(r[2 * j]) + __uint_as_float(r2[2 * j]), comb, bias);
+                b = fmaf(__uint_as_float(r[2 * j + 1]) + __uint_as_float(r2[2 * j + 1]), comb, bias);
+            } else {
+                a = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j])), comb, bias);
+                b = fmaf(__int2float_rn(static_cast<int32_t>(r[2 * j + 1])), comb, bias);
+            }
+            if (KIND == ACC_TWO_BRANCHES) {
                 a = fmaf(__int2float_rn(static_cast<int32_t>(r2[2 * j])), comb2, a);
                 b = fmaf(__int2float_rn(static_cast<int32_t>(r2[2 * j + 1])), comb2, b);
             }

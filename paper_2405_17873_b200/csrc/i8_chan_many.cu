@@ -349,7 +349,7 @@ chan_many_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             const uint32_t acc = tmem_base + buf * g.nt + (static_cast<uint32_t>((warp & 3) * 32) << 16);
             const int cols = min(g.nt, p.M - tok0);
             if (p.Y && pairs_ok && !p.acc_out) {
-                store_tokens<false, 16>(acc, 0, (ew >> 2) * 16, 32, cols, comb, 0.f, bias, p.Y + (n & ~1), p.ldy, tok0, p.M, n < p.N, false,
+                store_tokens<ACC_INT, 16>(acc, 0, (ew >> 2) * 16, 32, cols, comb, 0.f, bias, p.Y + (n & ~1), p.ldy, tok0, p.M, n < p.N, false,
                                     lane);
             } else {
                 // odd widths, and the raw sums of the parity hook
