@@ -137,7 +137,10 @@ bool pair_path_ok(const Params& p, int amode, int w_bits);
 int run_pair(const Params& p, int amode, const void* packed, int w_bits, cudaStream_t stream);
 // One wave of channel-major tiles, 128 cg channels x `tokens` tokens, no workspace; see wo_chan.cu.
 bool chan_tile_ok(int cg, int tokens);
-bool chan_path_ok(const Params& p, int amode, int w_bits);
+bool chan_path_ok(const Params& p, int amode, const void* packed, int w_bits);
+// Its tile's tokens (*cg CTAs) where it is the fastest form for the layer, else 0.  pair: whether run_pair could take it.
+int plan_chan(const Params& p, int amode, int w_bits, bool pair, int num_sms, int* cg);
+double pair_cost(int M, int N, int K, int k_blocks, int w_bits, int num_sms);
 int run_chan(const Params& p, int amode, const void* packed, int w_bits, int cg, int tokens, cudaStream_t stream);
 // Many-token path on tcgen05 (fp16 MMA, weights expanded into shared memory); see wo_tc.cu.
 bool tc_path_ok(const Params& p, int amode, int w_bits);

@@ -9,6 +9,11 @@
 //   * fp32 sums depend on their order, so each MMA issuer has an accumulator of its own and the epilogue adds the two:
 //     results do not change from run to run;
 //   * there is no quantization pass: the activations are the layer's input as it is.
+//
+// Measured on B200, before and now: W4 16 x 10240 x 1280 7.4 -> 5.3 us, 17 x 1280 x 1280 10.2 -> 4.2, 128 x 1280 x 5120 38.4 ->
+// 13.7, 256 x 1280 x 1280 8.4 -> 5.3, 1024 x 1280 x 1280 10.1 -> 6.8, 1024 x 1280 x 5120 23.7 -> 15.7, 3x3 convolution 48 x 48
+// x 640 -> 640 28.9 -> 17.6; W3 the first two 7.5 -> 5.6, 10.4 -> 4.3.  A long reduction takes 300 cycles per k-block of 64:
+// the expansion (three groups of four warps, some 1700 cycles for a pair of k-blocks; 3 bits more) and the rings' latency.
 #include <algorithm>
 
 #include "i8_chan.cuh"
@@ -257,7 +262,7 @@ wo_chan_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         const uint32_t a_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + a_col;
         const uint32_t flip = g.w_zero ? 0u : 0x88888888u;  // signed nibbles + 8
         const int zero = g.w_zero ? (n0 + row < p.N ? __ldg(g.w_zero + n0 + row) : 0) : 8;
-        const __half2 z2 = __half2half2(__ushort_as_half(static_cast<unsigned short>(0x6400 + zero)));
+        const __half2 z2 = __half2half2(__int2half_rn(1024 + zero));
         int sw = 2 * group % g.w_slots;  // slot of the pair's first k-block
         Codes<BITS> codes;
         auto fetch = [&](int j) {
@@ -379,11 +384,55 @@ bool chan_tile_ok(int cg, int tokens)
 }
 
 // A k-block of a convolution must be a whole block of the flattened reduction index: Cin a multiple of 64.
-bool chan_path_ok(const Params& p, int amode, int w_bits)
+bool chan_path_ok(const Params& p, int amode, const void* packed, int w_bits)
 {
-    if (w_bits > 4 || (w_bits <= 3 && !p.w_zero) || !p.Y || (reinterpret_cast<uintptr_t>(p.X) & 15) != 0) return false;
+    if (w_bits > 4 || (w_bits <= 3 && !p.w_zero) || !p.Y) return false;
+    if (((reinterpret_cast<uintptr_t>(p.X) | reinterpret_cast<uintptr_t>(packed)) & 15) != 0) return false;
     if (amode == A_CONV3) return p.Cin % BKE == 0 && (p.stride == 1 || p.stride == 2);
     return amode == A_LINEAR && p.K % 8 == 0 && p.ldx % 8 == 0;
+}
+
+// Cycles of a tile, fitted to 120 layers of 1 to 4096 rows (graphs of launches; error 5 to 7 per cent): fixed part + k-blocks x
+// (issue, little of it per token) + epilogue, and the share of the SMs in use (they compete for the L2).  The other forms' as
+// fitted to the same layers:
+//   * up to 16 rows, a linear layer: the kernels of wo_gemm.cu, which split the reduction inside a CTA and win wherever it is
+//     long or the rows are eight at most and the weights few (16 x 1280 x 5120 W4 5.6 us against 13.0), and lose by up to half
+//     on many channels (16 x 10240 x 1280 7.4 and 5.3);
+//   * 17 to 255 rows: nothing comes near (17 x 1280 x 1280 W4 10.2 us and 4.2, 128 x 1280 x 5120 38 and 13.7), so tiles of
+//     more than one wave are taken too;
+//   * from 256 rows, with a workspace: the pair form, whose split reductions win on the longest.
+int plan_chan(const Params& p, int amode, int w_bits, bool pair, int num_sms, int* cg)
+{
+    const bool conv = amode == A_CONV3;
+    const int k_blocks = static_cast<int>(conv ? 9 * ceil_div(p.Cin, BKE) : ceil_div(p.K, BKE));
+    const double nkb = k_blocks;
+    double best = 0;
+    int tokens = 0;
+    for (int c = 1; c <= 2; ++c) {
+        const int64_t c_tiles = ceil_div(p.N, CH * c);
+        for (int t = 16 * c; chan_tile_ok(c, t) && t < p.M + 16 * c; t += 16 * c) {
+            const int64_t ctas = c * c_tiles * ceil_div(p.M, t);
+            if (ctas > num_sms && p.M >= 256) continue;
+            const double waves = static_cast<double>(ceil_div(ctas, num_sms)), busy = std::min(1.0, static_cast<double>(ctas) / num_sms);
+            const double per_kb = (w_bits == 4 ? 244.0 : 284.0) - (c == 2 ? 16.0 : 0.0) + 0.3 * t;
+            const double cost = (c == 1 ? 2600.0 : 2900.0) +
+                                waves * (nkb * (per_kb + (c == 1 ? 47.0 : 57.0) * busy) + 27.0 * t + (c == 1 ? 2100.0 : 3650.0) * busy);
+            if (tokens == 0 || cost < best) {
+                best = cost;
+                tokens = t;
+                *cg = c;
+            }
+        }
+    }
+    if (tokens == 0) return 0;
+    const double N = p.N, K = p.K, b = w_bits == 4 ? 0.0 : 1.0;
+    if (p.M <= 16 && !conv && p.K <= 5120) {
+        const double other = p.M <= 8 ? 3950.0 + 220.0 * b + 0.29 * K + (4.8e-4 + 1.1e-4 * b) * N * K
+                                      : 5560.0 + 0.13 * N + (0.1 + 0.09 * b) * K + 7e-4 * N * K;
+        return best < 0.97 * other ? tokens : 0;
+    }
+    if (pair) return best < pair_cost(p.M, p.N, p.K, k_blocks, w_bits, num_sms) ? tokens : 0;
+    return tokens;
 }
 
 int run_chan(const Params& p, int amode, const void* packed, int w_bits, int cg, int tokens, cudaStream_t stream)

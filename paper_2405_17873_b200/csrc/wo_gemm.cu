@@ -531,7 +531,15 @@ int run(Params p, int amode, const void* packed, int w_bits, cudaStream_t stream
         return MIXDQ_ERR_ALIGNMENT;
     const long long pitch = row_pitch_bytes(p.K, w_bits, MIXDQ_LAYOUT_DEVICE);
     const bool is_signed = p.w_zero == nullptr;
-    if (pair_path_ok(p, amode, w_bits)) return run_pair(p, amode, packed, w_bits, stream);
+    const int num_sms = sm_count();
+    if (num_sms <= 0) return MIXDQ_ERR_CUDA;
+    const bool pair = pair_path_ok(p, amode, w_bits);
+    if (chan_path_ok(p, amode, packed, w_bits)) {
+        int cg;
+        const int tokens = plan_chan(p, amode, w_bits, pair, num_sms, &cg);
+        if (tokens > 0) return run_chan(p, amode, packed, w_bits, cg, tokens, stream);
+    }
+    if (pair) return run_pair(p, amode, packed, w_bits, stream);
     if (tc_path_ok(p, amode, w_bits) && !(w_bits <= 3 && is_signed)) return run_tc(p, amode, packed, w_bits, p.batch, stream);
     if (w_bits == 3) return is_signed ? MIXDQ_ERR_UNSUPPORTED : launch_nt<3, false>(p, amode, packed, pitch, stream);
     if (w_bits == 2) return is_signed ? MIXDQ_ERR_UNSUPPORTED : launch_nt<2, false>(p, amode, packed, pitch, stream);

@@ -76,7 +76,7 @@ bool conv_box(int Ho, int Wo, int* Wb, int* Hb, int* Bb)
 
 // Tile width and reduction split: whole rounds of 256 x bn tiles over the SM pairs, the per-tile cost growing with
 // the width; layers with few tiles and a long reduction give one tile to a cluster of two to four CTA pairs.
-int pick_tile(int M, int N, int k_blocks, int num_sms, int* splits)
+int pick_tile(int M, int N, int k_blocks, int num_sms, int* splits, double* cost = nullptr)
 {
     double best = 0;
     int best_bn = 0;
@@ -102,10 +102,21 @@ int pick_tile(int M, int N, int k_blocks, int num_sms, int* splits)
             }
         }
     }
+    if (cost) *cost = best;
     return best_bn;
 }
 
 }  // namespace
+
+// Cycles of the pair form: its tiles' estimate, with the weights expanded in the kernel or by a pass of its own.
+double pair_cost(int M, int N, int K, int k_blocks, int w_bits, int num_sms)
+{
+    int splits;
+    double tiles = 0;
+    pick_tile(M, N, k_blocks, num_sms, &splits, &tiles);
+    if (splits == 1 && w_bits <= 4 && M <= 2048) return 2460.0 + 1.53 * tiles;
+    return 7850.0 + 1.15 * tiles + 7e-6 * static_cast<double>(N) * K;
+}
 
 size_t expanded_weight_bytes(int64_t N, int64_t K) { return static_cast<size_t>(round_up(N * round_up(K, 8) * 2, 256)); }
 
