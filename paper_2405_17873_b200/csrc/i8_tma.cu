@@ -35,11 +35,18 @@ __device__ __forceinline__ uint32_t q4(float a, float b, float c, float d, float
     return __byte_perm(__byte_perm(qa, qb, 0x0040), __byte_perm(qc, qd, 0x0040), 0x5410);
 }
 
-// 16 consecutive fp16 values (16-byte aligned) to 16 code bytes.
-__device__ __forceinline__ uint4 quantize16(const __half* __restrict__ p, float inv, float lo, float hi, uint32_t zoff)
+// 16 consecutive fp16 values (16-byte aligned), and their code bytes.
+struct Half16 {
+    uint4 v0, v1;
+    __device__ __forceinline__ explicit Half16(const __half* __restrict__ p)
+        : v0(__ldg(reinterpret_cast<const uint4*>(p))), v1(__ldg(reinterpret_cast<const uint4*>(p) + 1))
+    {
+    }
+};
+
+__device__ __forceinline__ uint4 quantize16(const Half16& x, float inv, float lo, float hi, uint32_t zoff)
 {
-    const uint4* src = reinterpret_cast<const uint4*>(p);
-    const uint4 v0 = __ldg(src), v1 = __ldg(src + 1);
+    const uint4 &v0 = x.v0, &v1 = x.v1;
     const __half2* h0 = reinterpret_cast<const __half2*>(&v0);
     const __half2* h1 = reinterpret_cast<const __half2*>(&v1);
     float2 f[8];
@@ -56,26 +63,34 @@ __device__ __forceinline__ uint4 quantize16(const __half* __restrict__ p, float 
     return o;
 }
 
-// One thread per 16 consecutive elements of a row.  bos != 0: output row r reads input row
-// (r / 76) * 77 + r % 76 + 1, i.e. the BOS token of every prompt is left out.
+// One thread per 16 consecutive elements.  A small layer's pass is a chain of latencies in front of its GEMM, so that the
+// addresses are found before the wait for the previous kernel and the values requested before the scale's reciprocal.
+// DENSE: consecutive rows are consecutive in memory.  Else one thread per 16 elements of a row; bos != 0: output row r reads
+// input row (r / 76) * 77 + r % 76 + 1, i.e. the BOS token of every prompt is left out.
 // act_zero != nullptr: asymmetric codes with that zero-point (see q4).
-__global__ void quant_kernel(const __half* __restrict__ X, long long ldx, long long rows, int K, int bos,
+template <bool DENSE>
+__global__ void quant_kernel(const __half* __restrict__ X, long long ldx, long long tasks, int K, int bos,
                              const float* __restrict__ act_scale, const int32_t* __restrict__ act_zero,
                              int8_t* __restrict__ out)
 {
     pdl_launch_dependents();
-    pdl_wait();
-    const int cpr = K >> 4;
     const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    if (idx >= rows * cpr) return;
-    const long long r = idx / cpr;
-    const int c = static_cast<int>(idx - r * cpr);
-    long long src_row = r;
-    if (bos) {
-        const long long prompt = r / (MIXDQ_TOKENS_PER_PROMPT - 1);
-        src_row = prompt * MIXDQ_TOKENS_PER_PROMPT + (r - prompt * (MIXDQ_TOKENS_PER_PROMPT - 1)) + 1;
+    const bool mine = idx < tasks;
+    const __half* src = X + idx * 16;
+    if (!DENSE && mine) {
+        const int cpr = K >> 4;
+        const long long r = idx / cpr;
+        const int c = static_cast<int>(idx - r * cpr);
+        long long src_row = r;
+        if (bos) {
+            const long long prompt = r / (MIXDQ_TOKENS_PER_PROMPT - 1);
+            src_row = prompt * MIXDQ_TOKENS_PER_PROMPT + (r - prompt * (MIXDQ_TOKENS_PER_PROMPT - 1)) + 1;
+        }
+        src = X + src_row * ldx + c * 16;
     }
-    const float inv = __fdiv_rn(1.f, __ldg(act_scale));
+    pdl_wait();
+    if (!mine) return;
+    const Half16 x(src);
     float lo = kMagic - 127.f, hi = kMagic + 127.f;
     uint32_t zoff = 0;
     if (act_zero) {
@@ -84,7 +99,17 @@ __global__ void quant_kernel(const __half* __restrict__ X, long long ldx, long l
         hi = kMagic + static_cast<float>(255 - z);
         zoff = static_cast<uint32_t>(z - 128);
     }
-    *reinterpret_cast<uint4*>(out + r * K + c * 16) = quantize16(X + src_row * ldx + c * 16, inv, lo, hi, zoff);
+    const float inv = __fdiv_rn(1.f, __ldg(act_scale));
+    *reinterpret_cast<uint4*>(out + idx * 16) = quantize16(x, inv, lo, hi, zoff);
+}
+
+int launch_quant(const __half* X, long long ldx, long long rows, int K, bool bos, const float* act_scale, const int32_t* act_zero,
+                 int8_t* out, cudaStream_t stream)
+{
+    const long long tasks = rows * (K / 16);
+    const dim3 grid(static_cast<unsigned>(ceil_div(tasks, 256))), block(256);
+    if (ldx == K && !bos) return launch_pdl(quant_kernel<true>, grid, block, 0, stream, 1, X, ldx, tasks, K, 0, act_scale, act_zero, out);
+    return launch_pdl(quant_kernel<false>, grid, block, 0, stream, 1, X, ldx, tasks, K, bos ? 1 : 0, act_scale, act_zero, out);
 }
 
 // The int8 image of an asymmetrically quantized convolution input, with its padding written out: X fp16 NHWC
@@ -96,25 +121,25 @@ __global__ void quant_pad_kernel(const __half* __restrict__ X, int B, int H, int
                                  int8_t* __restrict__ out)
 {
     pdl_launch_dependents();
-    pdl_wait();
     const int cpr = Cin >> 4;
     const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    if (idx >= static_cast<long long>(B) * (H + 2) * (W + 2) * cpr) return;
     const long long pix = idx / cpr;
     const int c = static_cast<int>(idx - pix * cpr);
     const int wp = static_cast<int>(pix % (W + 2));
     const long long t = pix / (W + 2);
     const int hp = static_cast<int>(t % (H + 2));
     const long long b = t / (H + 2);
+    pdl_wait();
+    if (idx >= static_cast<long long>(B) * (H + 2) * (W + 2) * cpr) return;
     const int z = __ldg(act_zero);
     uint4 o;
     if (hp == 0 || hp == H + 1 || wp == 0 || wp == W + 1) {
         const uint32_t word = (static_cast<uint32_t>(z - 128) & 0xffu) * 0x01010101u;
         o = make_uint4(word, word, word, word);
     } else {
+        const Half16 x(X + ((b * H + (hp - 1)) * W + (wp - 1)) * Cin + c * 16);
         const float inv = __fdiv_rn(1.f, __ldg(act_scale));
-        const __half* src = X + ((b * H + (hp - 1)) * W + (wp - 1)) * Cin + c * 16;
-        o = quantize16(src, inv, kMagic - static_cast<float>(z), kMagic + static_cast<float>(255 - z),
+        o = quantize16(x, inv, kMagic - static_cast<float>(z), kMagic + static_cast<float>(255 - z),
                        static_cast<uint32_t>(z - 128));
     }
     *reinterpret_cast<uint4*>(out + pix * Cin + c * 16) = o;
@@ -129,15 +154,16 @@ __global__ void quant_split_kernel(const __half* __restrict__ X, long long ldx, 
                                    int8_t* __restrict__ out_lo, int8_t* __restrict__ out_hi)
 {
     pdl_launch_dependents();
-    pdl_wait();
     const int cpr = K >> 4;
     const long long idx = blockIdx.x * static_cast<long long>(blockDim.x) + threadIdx.x;
-    if (idx >= rows * cpr) return;
     const long long r = idx / cpr;
     const int c = static_cast<int>(idx - r * cpr) * 16;
     const bool hi_side = c >= split;
+    pdl_wait();
+    if (idx >= rows * cpr) return;
+    const Half16 x(X + r * ldx + c);
     const float inv = __fdiv_rn(1.f, __ldg(hi_side ? scale_hi : scale_lo));
-    const uint4 q = quantize16(X + r * ldx + c, inv, kMagic - 127.f, kMagic + 127.f, 0u);
+    const uint4 q = quantize16(x, inv, kMagic - 127.f, kMagic + 127.f, 0u);
     int8_t* dst = hi_side ? out_hi + r * (K - split) + (c - split) : out_lo + r * split + c;
     *reinterpret_cast<uint4*>(dst) = q;
 }
@@ -1406,8 +1432,7 @@ int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* sc
         rc = launch_pdl(quant_pad_kernel, dim3(static_cast<unsigned>(ceil_div(tasks, 256))), dim3(256), 0, stream, 1,
                         p.X, p.batch, p.H, p.W, p.Cin, p.act_scale, p.act_zero, aq);
     else
-        rc = launch_pdl(quant_kernel, dim3(static_cast<unsigned>(ceil_div(tasks, 256))), dim3(256), 0, stream, 1,
-                        p.X, ldx, in_rows, row_len, amode == A_BOS ? 1 : 0, p.act_scale, p.act_zero, aq);
+        rc = launch_quant(p.X, ldx, in_rows, row_len, amode == A_BOS, p.act_scale, p.act_zero, aq, stream);
     if (rc != MIXDQ_OK) return rc;
     return run_tma_gemm(p, amode, packed, w_bits, aq, stream);
 }
@@ -1548,9 +1573,7 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
 int run_quant(const __half* X, long long ldx, long long rows, int K, const float* act_scale, int8_t* out,
               cudaStream_t stream)
 {
-    const long long tasks = rows * (K / 16);
-    return launch_pdl(quant_kernel, dim3(static_cast<unsigned>(ceil_div(tasks, 256))), dim3(256), 0, stream, 1, X, ldx,
-                      rows, K, 0, act_scale, static_cast<const int32_t*>(nullptr), out);
+    return launch_quant(X, ldx, rows, K, false, act_scale, nullptr, out, stream);
 }
 
 // Step 2 alone, on int8 activations the caller keeps (the stored form of an activation tensor).
