@@ -83,8 +83,9 @@ int mixdq_int8_chan_tile(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int
  * its own, Sec. 4.1 "Hardware Profiling"): width of the 128-row output tiles when mixdq_linear, called with a
  * workspace, 8-bit symmetric activations and a row-major X, runs a layer of M rows, N channels and K inputs as ONE
  * kernel that quantizes its activation tiles itself; 0 when the layer runs as quantization pass + GEMM (the
- * one-kernel form pays only for short reductions, K <= 640, on one wave of tiles).  Below 2048 rows a layer for which
- * mixdq_int8_chan_tile reports a tile runs as two kernels all the same.  Negative: an error code.
+ * one-kernel form pays only for short reductions, K <= 640, on one wave of tiles).  Layers that fit single-CTA tiles of
+ * mixdq_int8_chan_tile, int4 layers of four or five reduction blocks and small int8 ones run as two kernels all the same.
+ * Negative: an error code.
  * For tests and benchmarks: nothing is launched. */
 int mixdq_linear_fused_quant_tile(int64_t M, int64_t N, int64_t K, int w_bits);
 

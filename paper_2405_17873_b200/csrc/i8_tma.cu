@@ -1413,10 +1413,16 @@ int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* sc
         const int num_sms = sm_count();
         const int kb = static_cast<int>(ceil_div(p.K, BK));
         const int fq_bn = num_sms > 0 ? plan_fq_tile(p.M, p.N, kb, w_bits == 4, num_sms) : 0;
-        // Below 2048 rows the quantization pass is short (1.7 us for 1024 x 640) and the channel-major GEMM after it makes
-        // up for it: 1024 x 640 x 640 W4 5.2 us against 8.2, W8 5.4 against 6.6.  From there on they come out equal (4096 x
-        // 640 x 640 W4: 9.2 and 9.3 us) or the fused kernel ahead (W8 9.2 and 7.5, K = 320 8.0 and 7.1).
-        if (fq_bn > 0 && (p.M >= 2048 || plan_chan(p.M, p.N, kb, w_bits == 4, num_sms).tokens == 0))
+        // It repeats the quantization in every tile column and lost ground to the shorter pass and the channel-major GEMM.
+        // Those win wherever the layer fits single-CTA tiles (3000 x 640 x 640 W4 6.7 us against 8.7, 2048 x 320 x 320 5.1 and
+        // 6.2); on CTA pairs for int4 from four k-blocks (4096 x 640 x 640 8.1 and 9.1; 384 long 7.4 and 7.0), whose expansion
+        // the fused kernel repeats too, up to some 8000 rows (8192 x 320 x 640 9.6 and 9.1); for int8 not there (4096 x 640 x
+        // 640 8.1 and 7.5).  Layers left to the forms with tokens on the rows: int8 of four or five k-blocks up to 3072 rows
+        // (2048 x 640 x 640 6.4 and 6.9, 3000 7.1 and 7.3).
+        const ChanPlan chan = fq_bn > 0 ? plan_chan(p.M, p.N, kb, w_bits == 4, num_sms) : ChanPlan{};
+        const bool two = chan.tokens == 0 ? kb >= 4 && p.M <= 3072
+                                          : chan.cg == 1 || (w_bits == 4 && kb >= 4 && p.M < 8192);
+        if (fq_bn > 0 && !two)
             return run_fq(p, packed, w_bits, fq_bn, stream);
     }
 
