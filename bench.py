@@ -766,7 +766,7 @@ def run_ours(args):
         alg_bytes = sum(sweep.algorithmic_bytes(pl) for pl in tc_layers)
         roofline = {"bound": "tensor", "achieved": achieved, "peak": peak, "unit": "TOP/s", "frac": achieved / peak,
                     "traffic": traffic,
-                    "kernel": "i8 tcgen05 kind::i8 GEMM kernels (pair_gemm_kernel on two-CTA tiles, tma_gemm_kernel, "
+                    "kernel": "i8 tcgen05 kind::i8 GEMM kernels (chan_gemm_kernel, chan_many_kernel, pair_gemm_kernel, tma_gemm_kernel, "
                               "tma_gemm_persistent_kernel) with their quant_kernel pre-pass, all tensor-core int8 layers of "
                               "the step",
                     "peak_source": f"{peaks['source']} bf16 sustained x {INT8_TO_BF16_NOMINAL:g} (nominal int8:bf16)",
