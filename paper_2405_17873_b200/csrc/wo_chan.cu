@@ -1,4 +1,4 @@
-// Weight-only (W2 / W3 / W4, fp16 activations) layers of one wave, channel-major: the weights on the 128 rows of the
+// Weight-only (W2 / W3 / W4 / W8, fp16 activations) layers of one wave, channel-major: the weights on the 128 rows of the
 // tensor-core tile, expanded to fp16 (code - zero, exact integers) straight into tensor memory, the tokens on its N side.
 //
 // Why.  The two-CTA form with the tokens on the rows (i8_pair.cu, MODE 3) writes every expanded weight row to shared memory
@@ -12,7 +12,8 @@
 //
 // Measured on B200, before and now: W4 16 x 10240 x 1280 7.4 -> 5.3 us, 17 x 1280 x 1280 10.2 -> 4.2, 128 x 1280 x 5120 38.4 ->
 // 13.7, 256 x 1280 x 1280 8.4 -> 5.3, 1024 x 1280 x 1280 10.1 -> 6.8, 1024 x 1280 x 5120 23.7 -> 15.7, 3x3 convolution 48 x 48
-// x 640 -> 640 28.9 -> 17.6; W3 the first two 7.5 -> 5.6, 10.4 -> 4.3.  A long reduction takes 300 cycles per k-block of 64:
+// x 640 -> 640 28.9 -> 17.6; W3 the first two 7.5 -> 5.6, 10.4 -> 4.3; W8
+// 16 x 10240 x 1280 7.4 -> 5.0, 17 x 1280 x 1280 10.2 -> 4.1, 1024 x 1280 x 1280 10.9 -> 6.6, 1024 x 1280 x 5120 25.0 -> 15.9.  A long reduction takes 300 cycles per k-block of 64:
 // the expansion (three groups of four warps, some 1700 cycles for a pair of k-blocks; 3 bits more) and the rings' latency.
 #include <algorithm>
 
@@ -67,7 +68,8 @@ struct Codes {
     __device__ __forceinline__ void load(const uint8_t* slot, int row)
     {
         // 64-byte rows come with the 64-byte swizzle; rows of 48 bytes are conflict-free, of 32 two-way, as they are
-        const uint32_t swz = BITS == 4 ? (static_cast<uint32_t>(row >> 1) & 3u) << 4 : 0u;
+        // (8 bits: 128-byte rows, 128-byte swizzle)
+        const uint32_t swz = BITS == 8 ? (static_cast<uint32_t>(row) & 7u) << 4 : (BITS == 4 ? (static_cast<uint32_t>(row >> 1) & 3u) << 4 : 0u);
         const uint8_t* src = slot + row * (16 * BITS);
 #pragma unroll
         for (int k = 0; k < BITS; ++k) v[k] = *reinterpret_cast<const uint4*>(src + ((static_cast<uint32_t>(k) << 4) ^ swz));
@@ -76,7 +78,7 @@ struct Codes {
     {
         return i == 0 ? q.x : (i == 1 ? q.y : (i == 2 ? q.z : q.w));
     }
-    // Eight codes of group j of k-block h as nibbles of a word.
+    // Eight codes of group j of k-block h as nibbles of a word (not for 8 bits).
     __device__ __forceinline__ uint32_t group(int h, int j, uint32_t flip) const
     {
         if constexpr (BITS == 4) {
@@ -98,8 +100,16 @@ __device__ __forceinline__ void expand_codes(const Codes<BITS>& codes, int h, ui
     uint32_t c[32];
 #pragma unroll
     for (int j = 0; j < 8; ++j) {
-        const uint32_t w = codes.group(h, j, flip);
-        const uint32_t lo4 = w & 0x0F0F0F0Fu, hi4 = (w >> 4) & 0x0F0F0F0Fu;
+        uint32_t lo4, hi4;  // codes 0 .. 3 and 4 .. 7 of the group as bytes
+        if constexpr (BITS == 8) {
+            const uint4& v = codes.v[4 * h + (j >> 1)];
+            lo4 = ((j & 1) ? v.z : v.x) ^ flip;
+            hi4 = ((j & 1) ? v.w : v.y) ^ flip;
+        } else {
+            const uint32_t w = codes.group(h, j, flip);
+            lo4 = w & 0x0F0F0F0Fu;
+            hi4 = (w >> 4) & 0x0F0F0F0Fu;
+        }
         const uint32_t b[4] = {__byte_perm(lo4, 0x64646464u, 0x5140), __byte_perm(lo4, 0x64646464u, 0x7362),
                                __byte_perm(hi4, 0x64646464u, 0x5140), __byte_perm(hi4, 0x64646464u, 0x7362)};
 #pragma unroll
@@ -260,8 +270,8 @@ wo_chan_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         // before they wait for its slots.
         const int group = (warp - WORK0) >> 2, row = (warp & 3) * 32 + lane;
         const uint32_t a_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + a_col;
-        const uint32_t flip = g.w_zero ? 0u : 0x88888888u;  // signed nibbles + 8
-        const int zero = g.w_zero ? (n0 + row < p.N ? __ldg(g.w_zero + n0 + row) : 0) : 8;
+        const uint32_t flip = g.w_zero ? 0u : (BITS == 8 ? 0x80808080u : 0x88888888u);  // signed codes + 128 or 8
+        const int zero = g.w_zero ? (n0 + row < p.N ? __ldg(g.w_zero + n0 + row) : 0) : (BITS == 8 ? 128 : 8);
         const __half2 z2 = __half2half2(__int2half_rn(1024 + zero));
         int sw = 2 * group % g.w_slots;  // slot of the pair's first k-block
         Codes<BITS> codes;
@@ -386,7 +396,7 @@ bool chan_tile_ok(int cg, int tokens)
 // A k-block of a convolution must be a whole block of the flattened reduction index: Cin a multiple of 64.
 bool chan_path_ok(const Params& p, int amode, const void* packed, int w_bits)
 {
-    if (w_bits > 4 || (w_bits <= 3 && !p.w_zero) || !p.Y) return false;
+    if ((w_bits <= 3 && !p.w_zero) || !p.Y) return false;
     if (((reinterpret_cast<uintptr_t>(p.X) | reinterpret_cast<uintptr_t>(packed)) & 15) != 0) return false;
     if (amode == A_CONV3) return p.Cin % BKE == 0 && (p.stride == 1 || p.stride == 2);
     return amode == A_LINEAR && p.K % 8 == 0 && p.ldx % 8 == 0;
@@ -427,7 +437,7 @@ int plan_chan(const Params& p, int amode, int w_bits, bool pair, int num_sms, in
     if (tokens == 0) return 0;
     const double N = p.N, K = p.K, b = w_bits == 4 ? 0.0 : 1.0;
     if (p.M <= 16 && !conv && p.K <= 5120) {
-        const double other = p.M <= 8 ? 3950.0 + 220.0 * b + 0.29 * K + (4.8e-4 + 1.1e-4 * b) * N * K
+        const double other = p.M <= 8 ? 3950.0 + 220.0 * b + 0.29 * K + (w_bits == 8 ? 3.4e-4 : 4.8e-4 + 1.1e-4 * b) * N * K
                                       : 5560.0 + 0.13 * N + (0.1 + 0.09 * b) * K + 7e-4 * N * K;
         return best < 0.97 * other ? tokens : 0;
     }
@@ -465,12 +475,13 @@ int run_chan(const Params& p, int amode, const void* packed, int w_bits, int cg,
     if (rc != MIXDQ_OK) return rc;
     const int64_t pitch = row_pitch_bytes(p.K, w_bits, MIXDQ_LAYOUT_DEVICE);
     rc = encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(pitch), static_cast<uint64_t>(p.N), static_cast<uint64_t>(pitch),
-                           static_cast<uint32_t>(16 * w_bits), CH, w_bits == 4 ? SWIZZLE_64 : SWIZZLE_NONE);
+                           static_cast<uint32_t>(16 * w_bits), CH, w_bits == 8 ? SWIZZLE_128 : (w_bits == 4 ? SWIZZLE_64 : SWIZZLE_NONE));
     if (rc != MIXDQ_OK) return rc;
     WoArgs g{};
     g.nt = tokens;
     g.c_tiles = static_cast<int>(ceil_div(p.N, CH * cg));
     g.w_zero = p.w_zero;
+    if (w_bits == 8) return launch<8>(cg, tw, tx, tp, g, stream);
     if (w_bits == 4) return launch<4>(cg, tw, tx, tp, g, stream);
     if (w_bits == 3) return launch<3>(cg, tw, tx, tp, g, stream);
     return launch<2>(cg, tw, tx, tp, g, stream);
