@@ -199,9 +199,9 @@ int mixdq_conv3x3_workspace_bytes(int64_t B, int64_t H, int64_t W, int64_t Cin, 
  * them BEFORE they wait for earlier work on the stream, so that their start overlaps the previous
  * kernel's end; they must therefore be complete when a layer call that reads them is enqueued.  Buffers
  * written by mixdq_pack_weights, mixdq_weight_minmax_params and mixdq_weight_code_sums on the SAME stream
- * satisfy this by themselves (those calls end with a full stream dependency).  Constants produced any
- * other way (a copy, a kernel of the caller's, another stream) need a stream synchronization or an event
- * wait between their producer and the first layer call that uses them.  Everything else -- X, the
+ * satisfy this by themselves (the library's next kernel on that stream starts after they are complete, captured into
+ * a graph or not).  Constants produced any other way (a copy, a kernel of the caller's, another stream) need a stream
+ * synchronization or an event wait between their producer and the first layer call that uses them.  Everything else -- X, the
  * activation scale and zero-point, the workspace, Y -- follows ordinary stream order.
  */
 

@@ -11,6 +11,7 @@ CSRC = os.path.join(HERE, "csrc")
 LIB = os.path.join(HERE, "libmixdq.so")
 BIND_SRC = os.path.join(CSRC, "bind.cpp")
 BIND = os.path.join(HERE, "_mixdq_native.so")
+NVCC = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
 INCLUDE = os.path.join(os.path.dirname(HERE), "include")
 
 
@@ -18,20 +19,23 @@ def sources():
     return sorted(glob.glob(os.path.join(CSRC, "*.cu")))
 
 
-def _stale() -> bool:
-    if not os.path.exists(LIB):
-        return True
-    t = os.path.getmtime(LIB)
-    deps = sources() + glob.glob(os.path.join(CSRC, "*.cuh")) + glob.glob(os.path.join(CSRC, "*.h")) + \
-        glob.glob(os.path.join(INCLUDE, "*.h"))
-    return any(os.path.getmtime(d) > t for d in deps)
+def _newest(files) -> float:
+    return max(os.path.getmtime(f) for f in files)
+
+
+def _fresh(target: str, files) -> bool:
+    return os.path.exists(target) and os.path.getmtime(target) >= _newest(files)
+
+
+def _headers():
+    return [f for pattern in (os.path.join(CSRC, "*.cuh"), os.path.join(CSRC, "*.h"), os.path.join(INCLUDE, "*.h"))
+            for f in glob.glob(pattern)]
 
 
 def _build_binding(force: bool) -> None:
     """The extension module links against libmixdq.so beside it; torch's libraries are found in the process, which has
     imported torch before it imports this package."""
-    newest = max(os.path.getmtime(f) for f in (BIND_SRC, os.path.join(INCLUDE, "mixdq.h")))
-    if not force and os.path.exists(BIND) and os.path.getmtime(BIND) >= newest:
+    if not force and _fresh(BIND, (BIND_SRC, os.path.join(INCLUDE, "mixdq.h"))):
         return
     import sysconfig
 
@@ -51,16 +55,21 @@ def build(force: bool = False, verbose: bool = False) -> str:
 
 
 def _build_library(force: bool, verbose: bool) -> None:
-    if not (force or _stale()):
-        return
-    nvcc = os.environ.get("NVCC", "/usr/local/cuda/bin/nvcc")
+    if force or not _fresh(LIB, sources() + _headers()):
+        subprocess.run([NVCC, "-shared", "-cudart", "static", "-o", LIB] + objects(force, verbose), check=True)
+
+
+def objects(force: bool = False, verbose: bool = False) -> list:
+    """The library's object files; those older than their source or any header are compiled."""
     objs = []
     procs = []
     os.makedirs(os.path.join(HERE, "_build"), exist_ok=True)
     for src in sources():
         obj = os.path.join(HERE, "_build", os.path.basename(src)[:-3] + ".o")
         objs.append(obj)
-        cmd = [nvcc, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
+        if not force and _fresh(obj, [src] + _headers()):
+            continue
+        cmd = [NVCC, "-O3", "-std=c++17", "-gencode", "arch=compute_100a,code=sm_100a", "-lineinfo",
                "-Xcompiler", "-fPIC", "-c", src, "-o", obj]
         if verbose:
             cmd.insert(1, "-Xptxas=-v")
@@ -73,7 +82,7 @@ def _build_library(force: bool, verbose: bool) -> None:
         failed |= pr.returncode != 0
     if failed:
         raise RuntimeError("nvcc failed")
-    subprocess.run([nvcc, "-shared", "-cudart", "static", "-o", LIB] + objs, check=True)
+    return objs
 
 
 if __name__ == "__main__":

@@ -87,10 +87,17 @@ int ensure_dynamic_smem(const void* kernel, int bytes);
 int sm_count();
 
 // A call on `stream` has written constants of a layer: the library's next kernel there must not start before they are
-// complete.  False: no room for another stream's note (the caller orders the two by other means).
+// complete.  False: no note is left (the stream is capturing or the per-thread one, or there are too many notes), and the
+// caller orders the two by other means.
 bool note_constants_written(cudaStream_t stream);
-// Whether there is such a note for `stream`; takes it.
-bool take_constants_note(cudaStream_t stream);
+// Whether the next kernel on `stream` has to be launched plainly, and the note that this launch, once it has succeeded,
+// takes away.  A launch into a graph takes none: the graph runs later, and the stream's next kernel may not be in it.
+struct ConstantsNote {
+    bool plain = false;
+    uint64_t serial = 0;  // 0: nothing to take
+};
+ConstantsNote standing_constants_note(cudaStream_t stream);
+void take_constants_note(const ConstantsNote& note);
 
 #ifdef __CUDACC__
 
@@ -133,9 +140,10 @@ inline int launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
     cfg.blockDim = block;
     cfg.dynamicSmemBytes = smem;
     cfg.stream = stream;
+    const ConstantsNote note = standing_constants_note(stream);
     cudaLaunchAttribute attr[2];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = take_constants_note(stream) ? 0 : 1;
+    attr[0].val.programmaticStreamSerializationAllowed = note.plain ? 0 : 1;
     attr[1].id = cudaLaunchAttributeClusterDimension;
     attr[1].val.clusterDim.x = cluster_x;
     attr[1].val.clusterDim.y = 1;
@@ -148,6 +156,7 @@ inline int launch_ex(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t sme
         (void)cudaGetLastError();
         return MIXDQ_ERR_CUDA;
     }
+    take_constants_note(note);
     return MIXDQ_OK;
 }
 

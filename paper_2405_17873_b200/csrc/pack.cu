@@ -254,8 +254,9 @@ using namespace mixdq;
 // wait for earlier kernels of the stream, so a kernel that WRITES such constants must be complete, not merely
 // finishing, when a layer kernel behind it starts.  The entry points below that produce constants therefore leave a
 // note for the stream, and the library's next kernel on it is launched plainly, without the programmatic overlap
-// (launch_ex).  Where no note can be left, this empty kernel, launched plainly, stands between the two.  (It used to
-// end every one of these calls: two launches and some 3 us of a 10240 x 1280 layer's preparation.)
+// (launch_ex).  Where no note can be left (while the stream captures, on the per-thread stream), this empty kernel,
+// launched plainly, stands between the two.  (It used to end every one of these calls: two launches and some 3 us of a
+// 10240 x 1280 layer's preparation.)
 __global__ void constants_complete_kernel() {}
 
 static int finish_constants(cudaStream_t st)

@@ -194,37 +194,86 @@ int allow_large_clusters(const void* kernel)
 
 namespace {
 
+// Notes by (device, handle): a handle alone does not name a stream, the default stream is handle 0 on every device.  (A
+// stream's id would do, but asking for it ends a capture with an error.)  A destroyed stream's handle may come back: the
+// new stream's first launch then is a plain one for nothing.
+struct Note {
+    int device;
+    cudaStream_t stream;
+    uint64_t serial;  // another one each time: a launch takes the note that it saw, not one left since
+};
+
 constexpr size_t kMaxNotes = 64;
 std::mutex g_notes_mutex;
-cudaStream_t g_notes[kMaxNotes];
+Note g_notes[kMaxNotes];
 std::atomic<size_t> g_note_count{0};  // read without the lock by every launch
+uint64_t g_note_serial = 0;
+
+bool capturing(cudaStream_t stream)
+{
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    if (cudaStreamIsCapturing(stream, &status) == cudaSuccess) return status != cudaStreamCaptureStatusNone;
+    (void)cudaGetLastError();
+    return true;  // (the default stream while another one captures: nothing can be launched on it)
+}
+
+// The default stream has two handles.
+cudaStream_t one_handle(cudaStream_t stream) { return stream == cudaStreamLegacy ? nullptr : stream; }
+
+// With the lock held.
+Note* find_note(int device, cudaStream_t stream)
+{
+    for (size_t i = 0, n = g_note_count.load(std::memory_order_relaxed); i < n; ++i)
+        if (g_notes[i].device == device && g_notes[i].stream == stream) return &g_notes[i];
+    return nullptr;
+}
 
 }  // namespace
 
 bool note_constants_written(cudaStream_t stream)
 {
+    // The per-thread handle is another stream in every thread.  While a stream captures, nothing runs: a note left then
+    // would be spent on a kernel of another graph or of none.
+    const int device = current_device();
+    if (device < 0 || stream == cudaStreamPerThread || capturing(stream)) return false;
     std::lock_guard<std::mutex> lock(g_notes_mutex);
-    const size_t n = g_note_count.load(std::memory_order_relaxed);
-    for (size_t i = 0; i < n; ++i)
-        if (g_notes[i] == stream) return true;
-    if (n == kMaxNotes) return false;
-    g_notes[n] = stream;
-    g_note_count.store(n + 1, std::memory_order_release);
+    Note* note = find_note(device, one_handle(stream));
+    if (!note) {
+        const size_t n = g_note_count.load(std::memory_order_relaxed);
+        if (n == kMaxNotes) return false;
+        note = &g_notes[n];
+        note->device = device;
+        note->stream = one_handle(stream);
+        g_note_count.store(n + 1, std::memory_order_release);
+    }
+    note->serial = ++g_note_serial;
     return true;
 }
 
-bool take_constants_note(cudaStream_t stream)
+ConstantsNote standing_constants_note(cudaStream_t stream)
 {
-    if (g_note_count.load(std::memory_order_acquire) == 0) return false;
+    ConstantsNote r;
+    if (g_note_count.load(std::memory_order_acquire) == 0) return r;
+    const int device = current_device();
+    std::lock_guard<std::mutex> lock(g_notes_mutex);
+    if (const Note* note = find_note(device, one_handle(stream))) {
+        r.plain = true;
+        r.serial = capturing(stream) ? 0 : note->serial;
+    }
+    return r;
+}
+
+void take_constants_note(const ConstantsNote& note)
+{
+    if (note.serial == 0) return;
     std::lock_guard<std::mutex> lock(g_notes_mutex);
     const size_t n = g_note_count.load(std::memory_order_relaxed);
     for (size_t i = 0; i < n; ++i)
-        if (g_notes[i] == stream) {
+        if (g_notes[i].serial == note.serial) {
             g_notes[i] = g_notes[n - 1];
             g_note_count.store(n - 1, std::memory_order_release);
-            return true;
+            return;
         }
-    return false;
 }
 
 int sm_count()

@@ -253,8 +253,8 @@ def test_conv1x1_equals_linear():
 
 @pytest.mark.parametrize("bits", [8, 4])
 def test_pack_then_layer_on_one_stream_without_synchronization(bits):
-    """The layer kernels load their weights before they wait for earlier kernels of the stream; the pack entry
-    points end with a full stream dependency so that a layer call enqueued right behind them, with no
+    """The layer kernels load their weights before they wait for earlier kernels of the stream; behind a pack entry
+    point the first one is launched without that overlap, so that a layer call enqueued right there, with no
     synchronization, still reads complete weights.  The same packed buffer is rewritten for every round."""
     M, K, N = 256, 1280, 640
     X = synth.normal_f16((M, K), 1.0, seed=77)
@@ -279,3 +279,31 @@ def test_pack_then_layer_on_one_stream_without_synchronization(bits):
         s_ref, _, codes = oracle_weights(W, bits, True)
         _, y_ref = orc.linear_a8(X, codes, s_ref, sx_ref, None)
         assert_close(host(outs[r]), y_ref)
+
+
+def test_pack_then_capture_on_one_stream():
+    """A layer call captured right behind an eager pack on the same stream, the replay, and an eager call behind that."""
+    M, K, N = 256, 1280, 640
+    X, W = synth.normal_f16((M, K), 1.0, seed=77), synth.normal_f16((N, K), 0.02, seed=780)
+    Xd, Wd = dev(X), dev(W)
+    sx, st, ws = mixdq.act_scale(Xd), status_word(), workspace_for(M, N, K, 8)
+    s = torch.zeros(N, dtype=torch.float32, device="cuda")
+    packed = torch.zeros(mixdq.packed_bytes(N, K, 8), dtype=torch.uint8, device="cuda")
+    captured, eager = (torch.zeros((M, N), dtype=torch.float16, device="cuda") for _ in range(2))
+    torch.cuda.synchronize()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.stream(stream):
+        mixdq.weight_minmax_params(Wd, 8, True, scale_out=s)
+        mixdq.pack_weights(Wd, 8, s, out=packed)
+        graph.capture_begin()
+        mixdq.linear(Xd, packed, N, 8, s, None, 8, sx, None, workspace=ws, status=st, out=captured)
+        graph.capture_end()
+        graph.replay()
+        mixdq.linear(Xd, packed, N, 8, s, None, 8, sx, None, workspace=ws, status=st, out=eager)
+    torch.cuda.synchronize()
+    assert int(host(st)[0]) == 0
+    _, _, codes = oracle_weights(W, 8, True)
+    s_ref, _ = orc.weight_minmax_params(W, 8, True)
+    _, y_ref = orc.linear_a8(X, codes, s_ref, orc.act_scale(orc.act_absmax(X), 8), None)
+    assert_close(host(captured), y_ref)
+    assert np.array_equal(host(captured).view(np.uint16), host(eager).view(np.uint16))
