@@ -35,7 +35,7 @@ def _headers():
 def _build_binding(force: bool) -> None:
     """The extension module links against libmixdq.so beside it; torch's libraries are found in the process, which has
     imported torch before it imports this package."""
-    if not force and _fresh(BIND, (BIND_SRC, os.path.join(INCLUDE, "mixdq.h"))):
+    if not force and _fresh(BIND, (BIND_SRC, os.path.join(CSRC, "unlocked.h"), os.path.join(INCLUDE, "mixdq.h"))):
         return
     import sysconfig
 

@@ -18,6 +18,7 @@
 #include <torch/csrc/autograd/python_variable.h>
 
 #include "../../include/mixdq.h"
+#include "unlocked.h"
 
 namespace {
 
@@ -152,11 +153,7 @@ struct Output {
 template <typename F>
 void call(const char* what, F&& f)
 {
-    int rc;
-    PyThreadState* state = PyEval_SaveThread();
-    rc = f();
-    PyEval_RestoreThread(state);
-    check(rc, what);
+    check(unlocked(f), what);
 }
 
 void need_dim(const at::Tensor& t, int dim)

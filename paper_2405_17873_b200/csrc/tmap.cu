@@ -3,6 +3,7 @@
 // a machine without a GPU driver.
 #include <atomic>
 #include <mutex>
+#include <new>
 #include <unordered_set>
 
 #include "common.cuh"
@@ -165,7 +166,11 @@ int set_once(const void* kernel, cudaFuncAttribute attribute, int value, std::mu
     std::lock_guard<std::mutex> lock(mu);
     if (done[dev].count(kernel)) return MIXDQ_OK;
     MIXDQ_CUDA_TRY(cudaFuncSetAttribute(kernel, attribute, value));
-    done[dev].insert(kernel);
+    try {
+        done[dev].insert(kernel);
+    } catch (const std::bad_alloc&) {
+        // set all the same, and again by the next call: nothing may be thrown through the C interface
+    }
     return MIXDQ_OK;
 }
 

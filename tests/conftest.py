@@ -8,6 +8,13 @@ if ROOT not in sys.path:
     sys.path.insert(0, ROOT)
 
 
+@pytest.fixture(scope="session")
+def recorded_library(tmp_path_factory):
+    """Path of the library on the runtime that only records (recorded.py)."""
+    import recorded
+    return recorded.link(str(tmp_path_factory.mktemp("recorded") / "libmixdq_recorded.so"))
+
+
 def pytest_configure(config):
     config.addinivalue_line("markers", "gpu: needs a CUDA device (B200)")
 

@@ -39,7 +39,10 @@ cudaError_t launch(const void* f, cudaStream_t stream, int overlap)
         g_fail_launch = false;
         return error(cudaErrorLaunchFailure);
     }
+    const bool fail = g_fail_alloc;
+    g_fail_alloc = false;  // (what is recorded here is not the library's)
     g_launches.push_back({kernels()[f], stream, overlap});
+    g_fail_alloc = fail;
     return cudaSuccess;
 }
 

@@ -1,41 +1,18 @@
 """The order of packing calls and the layer calls behind them, seen in how their kernels are launched.
 
 A layer kernel loads its weights before it waits for earlier kernels of its stream, so the first one behind a packing call
-must not be launched with programmatic overlap, unless an empty kernel stands between the two.  The library's object files
-are linked with a runtime that only records (fake_cudart.cpp): nothing here runs on a GPU."""
-import ctypes as C
-import os
-import subprocess
+must not be launched with programmatic overlap, unless an empty kernel stands between the two.  On the recording runtime
+(recorded.py): nothing here runs on a GPU."""
 import threading
 
 import pytest
 
-HERE = os.path.dirname(os.path.abspath(__file__))
-BUFFER = C.c_void_p(0x100000)  # never dereferenced
+from recorded import BUFFER, Recorded
+
 LEGACY, PER_THREAD = 1, 2
-EMPTY = "constants_complete_kernel"
 
 
-@pytest.fixture(scope="session")
-def fake_lib(tmp_path_factory):
-    """Path of the library on the recording runtime."""
-    from paper_2405_17873_b200 import build
-    out = str(tmp_path_factory.mktemp("fake") / "libmixdq_fake.so")
-    subprocess.run(["g++", "-O1", "-std=c++17", "-fPIC", "-shared", "-I/usr/local/cuda/include", os.path.join(HERE, "fake_cudart.cpp")]
-                   + build.objects() + ["-Wl,-Bsymbolic", "-o", out], check=True)
-    return out
-
-
-class Lib:
-    def __init__(self, path):
-        from paper_2405_17873_b200 import mixdq
-        self.so = C.CDLL(path)
-        for name, (res, args) in mixdq._SIGNATURES.items():
-            if hasattr(self.so, name):
-                getattr(self.so, name).restype, getattr(self.so, name).argtypes = res, args
-        self.so.fake_kernel.restype = C.c_char_p
-        self.so.fake_capturing.argtypes = [C.c_void_p, C.c_int]
-
+class Lib(Recorded):
     def pack(self, stream=0):
         assert self.so.mixdq_pack_weights(BUFFER, 64, 128, 8, BUFFER, None, 1, BUFFER, stream) == 0
 
@@ -43,17 +20,13 @@ class Lib:
         return self.so.mixdq_linear_q8(BUFFER, 64, 128, BUFFER, 64, 8, BUFFER, BUFFER, None, BUFFER, None, stream)
 
     def launches(self):
-        """(kernel, launched with overlap) of every launch since the last call."""
-        names = [self.so.fake_kernel(i).decode() for i in range(self.so.fake_launches())]
-        got = [("empty" if EMPTY in n else "pack" if "pack_kernel" in n else "layer", bool(self.so.fake_overlap(i)))
-               for i, n in enumerate(names)]
-        self.so.fake_clear()
-        return got
+        kind = lambda name: "empty" if "constants_complete_kernel" in name else "pack" if "pack_kernel" in name else "layer"
+        return [(kind(name), overlap) for name, overlap in super().launches()]
 
 
 @pytest.fixture
-def lib(fake_lib):
-    lib = Lib(fake_lib)
+def lib(recorded_library):
+    lib = Lib(recorded_library)
     for d in (1, 0):  # no note of another test stands
         lib.so.fake_device(d)
         for stream in (0, 0x70):
