@@ -34,16 +34,20 @@ def _headers():
 
 def _build_binding(force: bool) -> None:
     """The extension module links against libmixdq.so beside it; torch's libraries are found in the process, which has
-    imported torch before it imports this package."""
-    if not force and _fresh(BIND, (BIND_SRC, os.path.join(CSRC, "unlocked.h"), os.path.join(INCLUDE, "mixdq.h"))):
-        return
+    imported torch before it imports this package.  What it was compiled against is compiled into it."""
     import sysconfig
 
     import torch
+    built_for = f"_mixdq_native for torch {torch.__version__}, Python {sys.version_info.major}.{sys.version_info.minor}"
+    if not force and _fresh(BIND, (BIND_SRC, os.path.join(CSRC, "unlocked.h"), os.path.join(INCLUDE, "mixdq.h"))):
+        with open(BIND, "rb") as f:
+            if built_for.encode() + b"\0" in f.read():
+                return
     root = os.path.dirname(torch.__file__)
     subprocess.run(["g++", "-O2", "-std=c++17", "-fPIC", "-shared", "-isystem", os.path.join(root, "include"),
                     "-isystem", os.path.join(root, "include", "torch", "csrc", "api", "include"),
-                    "-isystem", "/usr/local/cuda/include", "-I" + sysconfig.get_paths()["include"], BIND_SRC, "-o", BIND,
+                    "-isystem", "/usr/local/cuda/include", "-I" + sysconfig.get_paths()["include"],
+                    f'-DMIXDQ_BUILT_FOR="{built_for}"', BIND_SRC, "-o", BIND,
                     "-L" + HERE, "-l:" + os.path.basename(LIB), "-L" + os.path.join(root, "lib"), "-lc10", "-lc10_cuda",
                     "-ltorch_cpu", "-ltorch_cuda", "-ltorch_python", "-Wl,-rpath,$ORIGIN"], check=True)
 

@@ -667,5 +667,7 @@ PyMODINIT_FUNC PyInit__mixdq_native(void)
     PyObject* f = PyCFunction_New(&kSetError, nullptr);
     if (!f || PyModule_AddObjectRef(m, "_set_error_class", f) < 0) return nullptr;
     Py_DECREF(f);
+    // (build.py looks for the text: a binding made for another torch or Python is out of date whatever its time)
+    if (PyModule_AddStringConstant(m, "built_for", MIXDQ_BUILT_FOR) < 0) return nullptr;
     return m;
 }

@@ -38,6 +38,18 @@ def test_no_link_time_dependency_on_the_driver():
     assert "libcuda.so" not in out and "libtorch" not in out
 
 
+def test_binding_of_another_torch_is_out_of_date(lib, monkeypatch):
+    import torch
+    from paper_2405_17873_b200 import build
+    compiled = []
+    monkeypatch.setattr(build.subprocess, "run", lambda cmd, **kw: compiled.append(cmd))
+    build._build_binding(force=False)
+    assert not compiled
+    monkeypatch.setattr(torch, "__version__", "0.0.0")
+    build._build_binding(force=False)
+    assert len(compiled) == 1 and compiled[0][0] == "g++"
+
+
 def test_version_and_strerror(lib):
     assert lib.mixdq_version() >= 100
     assert lib.mixdq_strerror(0) == b"success"
