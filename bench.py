@@ -359,13 +359,10 @@ def _fracs(rate, measured, nominal, probe=None):
     return d
 
 
-def _tile_name(M, N, k_blocks, bits):
+def _tile_name(M, N, k_blocks, bits, kind):
     from paper_2405_17873_b200 import mixdq
-    channels, tokens = mixdq.int8_chan_tile(M, N, k_blocks, bits)
-    if tokens:
-        return f"{channels} channels x {tokens} tokens"
-    rows, cols, sp = mixdq.int8_tile_plan(M, N, k_blocks, bits, with_splits=True)
-    return f"{rows}x{cols}" + (f", reduction over {sp} CTA pairs" if sp > 1 else "")
+    form, tokens, channels, splits = mixdq.int8_layer_plan(M, N, k_blocks, bits, kind)
+    return f"{channels} channels x {tokens} tokens ({form})" + (f", reduction over {splits} CTA pairs" if splits > 1 else "")
 
 
 def config_records(torch, mixdq, synth, stream, peaks, probe_int8):
@@ -390,7 +387,7 @@ def config_records(torch, mixdq, synth, stream, peaks, probe_int8):
         bd = None if b is None else dev(b)
         us = _time_graph(torch, stream, lambda: mixdq.linear(Xd, pk, N, bits, s, None, 8, sx, bd, ws, status, out=Y))
         tops = 2.0 * M * N * K / us / 1e6
-        tile = _tile_name(M, N, (K + 127) // 128, bits)
+        tile = _tile_name(M, N, (K + 127) // 128, bits, "linear")
         out.append({"config": tag, "M": M, "N": N, "K": K, "w_bits": bits, "a_bits": 8, "us": round(us, 2),
                     "tops": round(tops, 1), "bound": "tensor", "l2": "warm",
                     "tile": tile,
@@ -747,10 +744,13 @@ def run_ours(args):
                 torch.cuda.synchronize()
             us = t0.elapsed_time(t1) * 1e3 / (reps * rounds)
             tops = pl.spec.ops(args.batch) / us / 1e6
-            kb = 9 * ((pl.spec.Cin + 127) // 128) if pl.spec.kind == "conv3x3" else (pl.spec.K + 127) // 128
+            conv = pl.spec.kind == "conv3x3"
+            at, row = 0 if pl.packed_hi is None else synth.shortcut_split_at(pl.spec), pl.spec.Cin if conv else pl.spec.K
+            kb = (9 if conv else 1) * sum((c + 127) // 128 for c in (at, row - at))
+            asked = "split" if at else ("codes" if conv or args.act_asym else "linear")
             per_layer.append({"layer": name, "kind": pl.spec.kind, "M": pl.spec.rows(args.batch), "N": pl.spec.N,
                               "K": pl.spec.K, "w_bits": pl.spec.w_bits,
-                              "tile": _tile_name(pl.spec.rows(args.batch), pl.spec.N, kb, pl.spec.w_bits),
+                              "tile": _tile_name(pl.spec.rows(args.batch), pl.spec.N, kb, pl.spec.w_bits, asked),
                               "us": round(us, 2),
                               "tops": round(tops, 1), "frac_of_burst_peak": round(tops / burst, 3),
                               "frac_of_sustained_peak": round(tops / (peaks["bf16_tflops_sustained"] * INT8_TO_BF16_NOMINAL), 3),

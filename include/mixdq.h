@@ -83,11 +83,27 @@ int mixdq_int8_chan_tile(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int
  * its own, Sec. 4.1 "Hardware Profiling"): width of the 128-row output tiles when mixdq_linear, called with a
  * workspace, 8-bit symmetric activations and a row-major X, runs a layer of M rows, N channels and K inputs as ONE
  * kernel that quantizes its activation tiles itself; 0 when the layer runs as quantization pass + GEMM (the
- * one-kernel form pays only for short reductions, K <= 640, on one wave of tiles).  Layers that fit single-CTA tiles of
- * mixdq_int8_chan_tile, int4 layers of four or five reduction blocks and small int8 ones run as two kernels all the same.
- * Negative: an error code.
+ * one-kernel form pays only for short reductions, K <= 640, on one wave of tiles).  Negative: an error code.
  * For tests and benchmarks: nothing is launched. */
 int mixdq_linear_fused_quant_tile(int64_t M, int64_t N, int64_t K, int w_bits);
+
+/* Diagnostic (the paper has no counterpart): the kernel that runs an int8 layer of M rows, N channels and k_blocks
+ * reduction blocks of 128 (as in mixdq_int8_tile_plan) with a workspace or on stored codes.  The layer calls decide by the
+ * same function.  kind: */
+#define MIXDQ_LAYER_LINEAR 0  /* mixdq_linear on fp16 rows with symmetric activations */
+#define MIXDQ_LAYER_CODES 1   /* stored codes, 3x3 convolutions, asymmetric activations */
+#define MIXDQ_LAYER_KV 2      /* mixdq_crossattn_kv */
+#define MIXDQ_LAYER_SPLIT 3   /* a shortcut-split layer; k_blocks of both branches */
+/* Returns one of these, or a negative error code: */
+#define MIXDQ_FORM_SINGLE 0     /* 128-token tiles on single CTAs */
+#define MIXDQ_FORM_PAIR 1       /* 256-token tiles on CTA pairs, *reduction_splits pairs to a tile */
+#define MIXDQ_FORM_CHAN 2       /* channel-major tiles, all on the SMs at once */
+#define MIXDQ_FORM_CHAN_MANY 3  /* channel-major tiles on CTA pairs that walk several each */
+#define MIXDQ_FORM_FUSED 4      /* one kernel that quantizes its activation tiles itself */
+#define MIXDQ_FORM_BRANCHES 5   /* a shortcut-split layer as a GEMM for each branch (tile sizes 0) */
+/* All pointers HOST.  Nothing is launched. */
+int mixdq_int8_layer_plan(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int kind, int* tile_tokens,
+                          int* tile_channels, int* reduction_splits);
 
 /* Static, NUL-terminated description of an error code (host pointer, never NULL). */
 const char* mixdq_strerror(int code);

@@ -197,9 +197,8 @@ extern "C" int mixdq_int8_tile_plan(int64_t M, int64_t N, int64_t k_blocks, int 
         *reduction_splits = splits;
     } else {
         *reduction_splits = 0;  // (decided at launch: a cluster of up to eight CTAs when the tiles are few)
-        const bool wide = w_bits == 8 && (N >= 1024 || N % 256 == 0) && ceil_div(M, 128) * ceil_div(N, 256) >= 100;
         *tile_rows = 128;
-        *tile_cols = wide ? 256 : i8::plan_narrow_tile(static_cast<int>(M), static_cast<int>(N), static_cast<int>(k_blocks), sms);
+        *tile_cols = i8::plan_single_tile(static_cast<int>(M), static_cast<int>(N), static_cast<int>(k_blocks), w_bits == 4, sms);
     }
     return MIXDQ_OK;
 }
@@ -225,7 +224,26 @@ extern "C" int mixdq_linear_fused_quant_tile(int64_t M, int64_t N, int64_t K, in
     const int sms = sm_count();
     if (sms <= 0) return MIXDQ_ERR_CUDA;
     if (K % 16 != 0) return 0;  // (the TMA-fed kernels need 16-byte rows of codes)
-    return i8::plan_fq_tile(static_cast<int>(M), static_cast<int>(N), static_cast<int>(ceil_div(K, 128)), w_bits == 4, sms);
+    const i8::LayerPlan plan = i8::plan_layer(i8::LayerKind::ROWS, static_cast<int>(M), static_cast<int>(N),
+                                              static_cast<int>(ceil_div(K, 128)), w_bits == 4, sms);
+    return plan.form == i8::Form::FUSED ? plan.channels : 0;
+}
+
+extern "C" int mixdq_int8_layer_plan(int64_t M, int64_t N, int64_t k_blocks, int w_bits, int kind, int* tile_tokens,
+                                     int* tile_channels, int* reduction_splits)
+{
+    if (!tile_tokens || !tile_channels || !reduction_splits || M <= 0 || N <= 0 || k_blocks <= 0 || M > 0x7fffffff ||
+        N > 0x7fffffff || k_blocks > 0x7fffffff || kind < MIXDQ_LAYER_LINEAR || kind > MIXDQ_LAYER_SPLIT)
+        return MIXDQ_ERR_INVALID_ARG;
+    if (w_bits != 4 && w_bits != 8) return MIXDQ_ERR_UNSUPPORTED;
+    const int sms = sm_count();
+    if (sms <= 0) return MIXDQ_ERR_CUDA;
+    const i8::LayerPlan plan = i8::plan_layer(static_cast<i8::LayerKind>(kind), static_cast<int>(M), static_cast<int>(N),
+                                              static_cast<int>(k_blocks), w_bits == 4, sms);
+    *tile_tokens = plan.tokens;
+    *tile_channels = plan.channels;
+    *reduction_splits = plan.splits;
+    return static_cast<int>(plan.form);
 }
 
 extern "C" const char* mixdq_strerror(int code)

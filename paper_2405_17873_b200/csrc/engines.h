@@ -6,6 +6,8 @@
 #include <stddef.h>
 #include <stdint.h>
 
+#include "../../include/mixdq.h"
+
 namespace mixdq {
 
 // How the rows of the A operand are found in memory.
@@ -63,14 +65,33 @@ int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* sc
 // M x N over k_blocks k-blocks of 128, else 0 (the single-CTA kernels run).  *splits (optional): how many CTA
 // pairs share one tile's reduction (1: persistent pairs; without the pointer only that form is considered).
 int plan_pair_tile(int M, int N, int k_blocks, bool w4, int num_sms, int* splits = nullptr);
-// Tile width of the fused-quantization kernel (one launch per layer, 128 x width tiles) when the planner prefers
-// it for a linear layer with symmetric activations, else 0 (quantization pass + GEMM).
-int plan_fq_tile(int M, int N, int k_blocks, bool w4, int num_sms);
 // The one-kernel form itself on 128 x bn tiles (bn a multiple of 32, 32 .. 256): a linear layer with symmetric
 // activations, K % 16 == 0, ldx % 8 == 0, X 16-byte aligned; p.Y and / or p.acc_out.
 int run_fq(const Params& p, const void* packed, int w_bits, int bn, cudaStream_t stream);
-// Tile width (128, 96 or 64) of the one-tile kernel on 128-wide slots.
-int plan_narrow_tile(int M, int N, int k_blocks, int num_sms);
+// Tile width (256, 128, 96 or 64) of the single-CTA kernels.
+int plan_single_tile(int M, int N, int k_blocks, bool w4, int num_sms);
+// What runs an int8 layer that has a workspace or stored codes: the calls and the queries all ask here.
+enum class Form {
+    SINGLE = MIXDQ_FORM_SINGLE,        // 128 x channels tiles on single CTAs (i8_tma.cu)
+    PAIR = MIXDQ_FORM_PAIR,            // 256 x channels tiles on CTA pairs, `splits` pairs to a tile (i8_pair.cu)
+    CHAN = MIXDQ_FORM_CHAN,            // channel-major, one wave (i8_chan.cu)
+    CHAN_MANY = MIXDQ_FORM_CHAN_MANY,  // channel-major, several waves (i8_chan_many.cu)
+    FUSED = MIXDQ_FORM_FUSED,          // one kernel that quantizes its own activation tiles (i8_fq.cu)
+    BRANCHES = MIXDQ_FORM_BRANCHES,    // shortcut-split layer: a GEMM for each branch, CODES then SECOND_BRANCH
+};
+enum class LayerKind {
+    ROWS = MIXDQ_LAYER_LINEAR,   // fp16 rows, symmetric activations
+    CODES = MIXDQ_LAYER_CODES,   // stored codes, convolutions, asymmetric activations
+    BOS = MIXDQ_LAYER_KV,
+    SPLIT = MIXDQ_LAYER_SPLIT,   // k_blocks of both branches
+    SECOND_BRANCH,
+};
+struct LayerPlan {
+    Form form = Form::SINGLE;
+    int tokens = 0, channels = 0;  // of a tile
+    int splits = 1;
+};
+LayerPlan plan_layer(LayerKind kind, int M, int N, int k_blocks, bool w4, int num_sms);
 // The two steps as calls of their own, for activations that are stored as int8 between layers: the codes of
 // X [rows, K] into a dense int8 matrix, and the GEMM / implicit-GEMM convolution on such codes (p.X unused).
 int run_quant(const __half* X, long long ldx, long long rows, int K, const float* act_scale, int8_t* out,

@@ -1294,27 +1294,11 @@ ChanPlan plan_chan(int M, int N, int k_blocks, bool w4, int num_sms, bool two, b
     return best < 1.06 * other ? r : ChanPlan{};
 }
 
-// Fused-quantization kernel (i8_fq.cu) or the two-kernel forms.  The fused kernel's k-block costs three to four
-// times the two-kernel main loop's (its converter warps' turn bounds it), and its fixed cost is one kernel's
-// instead of two: it wins where the reduction is short (at most five k-blocks), the activations large enough for
-// the quantization pass to matter, and the tiles fit the SMs in one wave.  Measured on B200, fused against
-// two-kernel: 4096 x 640 x 640 W4 9.5 / 10.5 us, W8 7.8 / 9.2; 4096 x 640 x 320 7.5 / 9.9 and 6.5 / 8.7;
-// 1024 x 640 x 640 W8 6.8 / 8.7, W4 8.3 / 8.7; losing: 1024 x 1280 x 640 (8.9 / 7.1), 16384 x 320 x 640 (two
-// waves: 18.5 / 15.5), anything from ten k-blocks up (1024 x 1280 x 1280: 12.2 / 8.5).
-// Width: the narrowest multiple of 32 whose tiles still fit one wave (less MMA and epilogue work per CTA).
-int plan_fq_tile(int M, int N, int k_blocks, bool w4, int num_sms)
-{
-    (void)w4;
-    if (k_blocks > 5 || N > 1024 || M < 1024) return 0;
-    const int64_t row_tiles = ceil_div(M, BM);
-    for (int bn = 64; bn <= 256; bn += 32)
-        if (row_tiles * ceil_div(N, bn) <= num_sms) return bn;
-    return 0;
-}
+namespace {
 
 // Width of the one-tile kernel's tiles for a layer the single-CTA kernels run on 128-wide slots: 128, or 96 / 64
 // when that raises the number of CTAs while they still fit the SMs in one wave and the reduction is not split.
-int plan_narrow_tile(int M, int N, int k_blocks, int num_sms)
+int narrow_tile(int M, int N, int k_blocks, int num_sms)
 {
     const int64_t row_tiles = ceil_div(M, BM);
     const int64_t t128 = row_tiles * ceil_div(N, 128);
@@ -1324,6 +1308,85 @@ int plan_narrow_tile(int M, int N, int k_blocks, int num_sms)
         if (t < num_sms && t > t128) return cand;
     }
     return 128;
+}
+
+}  // namespace
+
+// 256-wide tiles halve the activation traffic per output but need enough tiles to cover the SMs (int4 runs on 128-wide ones
+// only: its packed ring needs the room, and it measured no slower).
+int plan_single_tile(int M, int N, int k_blocks, bool w4, int num_sms)
+{
+    const bool wide = !w4 && (N >= 1024 || N % 256 == 0) && ceil_div(M, BM) * ceil_div(N, 256) >= 100;
+    return wide ? 256 : narrow_tile(M, N, k_blocks, num_sms);
+}
+
+namespace {
+
+// Fused-quantization kernel (i8_fq.cu): the width of its tiles where it could win, else 0.  Its k-block costs three to four
+// times the two-kernel main loop's (its converter warps' turn bounds it), and its fixed cost is one kernel's instead of
+// two: it needs a short reduction (at most five k-blocks; 1024 x 1280 x 1280: 12.2 us against 8.5), activations large enough
+// for the quantization pass to matter, and tiles that fit the SMs in one wave (16384 x 320 x 640, two waves: 18.5 / 15.5).
+// Width: the narrowest multiple of 32 whose tiles still fit one wave (less MMA and epilogue work per CTA).
+int fq_tile(int M, int N, int k_blocks, int num_sms)
+{
+    if (k_blocks > 5 || N > 1024 || M < 1024) return 0;
+    const int64_t row_tiles = ceil_div(M, BM);
+    for (int bn = 64; bn <= 256; bn += 32)
+        if (row_tiles * ceil_div(N, bn) <= num_sms) return bn;
+    return 0;
+}
+
+// Whether quantization pass + GEMM are faster than the fused kernel on a layer that has a tile of it.  The fused kernel
+// repeats the quantization in every tile column and lost ground to the shorter pass and the channel-major GEMM.  Those win
+// wherever the layer fits single-CTA tiles (3000 x 640 x 640 W4 6.7 us against 8.7, 2048 x 320 x 320 5.1 and 6.2); on CTA
+// pairs for int4 from four k-blocks (4096 x 640 x 640 8.1 and 9.1; 384 long 7.4 and 7.0), whose expansion the fused kernel
+// repeats too, up to some 8000 rows (8192 x 320 x 640 9.6 and 9.1); for int8 not there (4096 x 640 x 640 8.1 and 7.5).
+// Layers left to the forms with tokens on the rows: int8 of four or five k-blocks up to 3072 rows (2048 x 640 x 640 6.4 and
+// 6.9, 3000 7.1 and 7.3).
+bool two_kernels_win(const ChanPlan& chan, int M, int k_blocks, bool w4)
+{
+    if (chan.tokens == 0) return k_blocks >= 4 && M <= 3072;
+    return chan.cg == 1 || (w4 && k_blocks >= 4 && M < 8192);
+}
+
+}  // namespace
+
+LayerPlan plan_layer(LayerKind kind, int M, int N, int k_blocks, bool w4, int num_sms)
+{
+    LayerPlan r;
+    const bool split = kind == LayerKind::SPLIT;
+    if (kind != LayerKind::SECOND_BRANCH) {
+        const ChanPlan chan = plan_chan(M, N, k_blocks, w4, num_sms, split, kind != LayerKind::BOS);
+        const int fq = kind == LayerKind::ROWS ? fq_tile(M, N, k_blocks, num_sms) : 0;
+        if (fq > 0 && !two_kernels_win(chan, M, k_blocks, w4)) {
+            r.form = Form::FUSED;
+            r.tokens = BM;
+            r.channels = fq;
+            return r;
+        }
+        if (chan.tokens > 0) {
+            r.form = chan.many ? Form::CHAN_MANY : Form::CHAN;
+            r.tokens = chan.tokens;
+            r.channels = 128 * chan.cg;
+            return r;
+        }
+        int splits = 1;
+        const int pair = kind == LayerKind::BOS ? 0 : plan_pair_tile(M, N, k_blocks, w4, num_sms, split ? nullptr : &splits);
+        if (pair > 0) {
+            r.form = Form::PAIR;
+            r.tokens = 2 * BM;
+            r.channels = pair;
+            r.splits = splits;
+            return r;
+        }
+    }
+    if (split) {
+        r.form = Form::BRANCHES;
+        return r;
+    }
+    r.tokens = BM;
+    r.channels = kind == LayerKind::SECOND_BRANCH ? 128 : plan_single_tile(M, N, k_blocks, w4, num_sms);
+    return r;
 }
 
 size_t tma_scratch_bytes(int64_t in_rows, int64_t K_row) { return static_cast<size_t>(round_up(in_rows * K_row, 256)); }
@@ -1369,7 +1432,8 @@ bool tma_path_ok(const Params& p, int amode, int w_bits)
 
 // Step 2 of the two-kernel path: the TMA-fed GEMM (or implicit-GEMM convolution) on int8 activations `aq`
 // that an earlier kernel of the stream has written ([M, K] dense, or the NHWC image, padded when p.act_zero).
-static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bits, int8_t* aq, cudaStream_t stream);
+static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bits, const LayerPlan& plan, const int8_t* aq,
+                        cudaStream_t stream);
 
 // One-kernel form: the GEMM kernel quantizes its own activation tiles (i8_fq.cu).
 int run_fq(const Params& p, const void* packed, int w_bits, int bn, cudaStream_t stream)
@@ -1406,25 +1470,33 @@ int run_fq(const Params& p, const void* packed, int w_bits, int bn, cudaStream_t
     return launch_fq(tx, tw, ty, tp, w4, bn, stream);
 }
 
+// The plan of a call; the self-test of the bounded waits runs on the single-CTA kernels.
+static int plan_call(const Params& p, int amode, bool fp16_rows, int w_bits, LayerPlan* plan)
+{
+    const int num_sms = sm_count();
+    if (num_sms <= 0) return MIXDQ_ERR_CUDA;
+    const bool w4 = w_bits == 4;
+    const int k_blocks = static_cast<int>(amode == A_CONV3 ? 9 * ceil_div(p.Cin, BK) : ceil_div(p.K, BK));
+    if (p.test_drop_b_kblock) {
+        *plan = LayerPlan{};
+        plan->tokens = BM;
+        plan->channels = plan_single_tile(p.M, p.N, k_blocks, w4, num_sms);
+        return MIXDQ_OK;
+    }
+    const LayerKind kind = p.addend ? LayerKind::SECOND_BRANCH
+                                    : (amode == A_BOS ? LayerKind::BOS
+                                                      : (fp16_rows && amode == A_LINEAR && !p.act_zero ? LayerKind::ROWS : LayerKind::CODES));
+    *plan = plan_layer(kind, p.M, p.N, k_blocks, w4, num_sms);
+    return MIXDQ_OK;
+}
+
 int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* scratch, cudaStream_t stream)
 {
     int8_t* aq = static_cast<int8_t*>(scratch);
-    if (amode == A_LINEAR && !p.act_zero && !p.addend && !p.test_drop_b_kblock) {
-        const int num_sms = sm_count();
-        const int kb = static_cast<int>(ceil_div(p.K, BK));
-        const int fq_bn = num_sms > 0 ? plan_fq_tile(p.M, p.N, kb, w_bits == 4, num_sms) : 0;
-        // It repeats the quantization in every tile column and lost ground to the shorter pass and the channel-major GEMM.
-        // Those win wherever the layer fits single-CTA tiles (3000 x 640 x 640 W4 6.7 us against 8.7, 2048 x 320 x 320 5.1 and
-        // 6.2); on CTA pairs for int4 from four k-blocks (4096 x 640 x 640 8.1 and 9.1; 384 long 7.4 and 7.0), whose expansion
-        // the fused kernel repeats too, up to some 8000 rows (8192 x 320 x 640 9.6 and 9.1); for int8 not there (4096 x 640 x
-        // 640 8.1 and 7.5).  Layers left to the forms with tokens on the rows: int8 of four or five k-blocks up to 3072 rows
-        // (2048 x 640 x 640 6.4 and 6.9, 3000 7.1 and 7.3).
-        const ChanPlan chan = fq_bn > 0 ? plan_chan(p.M, p.N, kb, w_bits == 4, num_sms) : ChanPlan{};
-        const bool two = chan.tokens == 0 ? kb >= 4 && p.M <= 3072
-                                          : chan.cg == 1 || (w_bits == 4 && kb >= 4 && p.M < 8192);
-        if (fq_bn > 0 && !two)
-            return run_fq(p, packed, w_bits, fq_bn, stream);
-    }
+    LayerPlan plan;
+    int rc = plan_call(p, amode, true, w_bits, &plan);
+    if (rc != MIXDQ_OK) return rc;
+    if (plan.form == Form::FUSED) return run_fq(p, packed, w_bits, plan.channels, stream);
 
     // 1. quantize the activations once
     const bool conv = amode == A_CONV3;
@@ -1433,17 +1505,17 @@ int run_tma(const Params& p, int amode, const void* packed, int w_bits, void* sc
     const int row_len = conv ? p.Cin : p.K;
     const long long ldx = conv ? p.Cin : p.ldx;
     const long long tasks = in_rows * (row_len / 16);
-    int rc;
     if (pad)
         rc = launch_pdl(quant_pad_kernel, dim3(static_cast<unsigned>(ceil_div(tasks, 256))), dim3(256), 0, stream, 1,
                         p.X, p.batch, p.H, p.W, p.Cin, p.act_scale, p.act_zero, aq);
     else
         rc = launch_quant(p.X, ldx, in_rows, row_len, amode == A_BOS, p.act_scale, p.act_zero, aq, stream);
     if (rc != MIXDQ_OK) return rc;
-    return run_tma_gemm(p, amode, packed, w_bits, aq, stream);
+    return run_tma_gemm(p, amode, packed, w_bits, plan, aq, stream);
 }
 
-static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bits, int8_t* aq, cudaStream_t stream)
+static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bits, const LayerPlan& plan, const int8_t* aq,
+                        cudaStream_t stream)
 {
     const bool w4 = w_bits == 4;
     const int64_t pitch = row_pitch_bytes(p.K, w_bits, MIXDQ_LAYOUT_DEVICE);
@@ -1452,12 +1524,8 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
     int rc;
     const int num_sms = sm_count();
     if (num_sms <= 0) return MIXDQ_ERR_CUDA;
-    if (!p.addend && !p.test_drop_b_kblock) {
-        const int kb = static_cast<int>(conv ? 9 * ceil_div(p.Cin, BK) : ceil_div(p.K, BK));
-        const ChanPlan plan = plan_chan(p.M, p.N, kb, w4, num_sms, false, amode != A_BOS);
-        if (plan.many) return run_chan_many(p, amode, packed, aq, plan.tokens, num_sms, stream);
-        if (plan.tokens > 0) return run_chan(p, amode, packed, w_bits, aq, plan.cg, plan.tokens, stream);
-    }
+    if (plan.form == Form::CHAN_MANY) return run_chan_many(p, amode, packed, aq, plan.tokens, num_sms, stream);
+    if (plan.form == Form::CHAN) return run_chan(p, amode, packed, w_bits, aq, plan.channels / 128, plan.tokens, stream);
 
     // 2. tensor maps
     CUtensorMap ta, tw, ty{};
@@ -1513,11 +1581,8 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
         tp.k_blocks = static_cast<int>(ceil_div(p.K, BK));
     }
     if (rc != MIXDQ_OK) return rc;
-    // the pair form (two-CTA tiles of 256 x bn, i8_pair.cu) where its estimate beats the single-CTA kernels
-    int pair_splits = 1;
-    const int pair_bn = (!p.addend && amode != A_BOS && !p.test_drop_b_kblock)
-                            ? plan_pair_tile(p.M, p.N, tp.k_blocks, w4, num_sms, &pair_splits) : 0;
-    if (pair_bn > 0) {
+    if (plan.form == Form::PAIR) {  // two-CTA tiles of 256 x pair_bn, i8_pair.cu
+        const int pair_bn = plan.channels;
         if (w4)
             rc = encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, BK / 2, pair_bn / 2, false);
         else
@@ -1528,20 +1593,15 @@ static int run_tma_gemm(const Params& p, int amode, const void* packed, int w_bi
                                     static_cast<uint64_t>(p.ldy), 32, 32, true);
             if (rc != MIXDQ_OK) return rc;
         }
-        return launch_pair(ta, tw, ty, tp, w4, pair_bn, pair_splits, num_sms, stream);
+        return launch_pair(ta, tw, ty, tp, w4, pair_bn, plan.splits, num_sms, stream);
     }
-    // 256-wide tiles halve the A traffic per output but need enough tiles to cover the SMs
-    // (W4 runs on 128-wide tiles only: its packed ring needs the room, and it measured no slower)
-    const bool wide = !w4 && !p.addend && (p.N >= 1024 || p.N % 256 == 0) && ceil_div(p.M, BM) * ceil_div(p.N, 256) >= 100;
-    uint32_t bn = wide ? 256 : 128;
+    const bool wide = plan.channels == 256;
+    const uint32_t bn = static_cast<uint32_t>(plan.channels);
     // Tile-count quantization of the one-tile kernel: a layer whose 128-wide tiles number between half the SMs
     // and all of them (1024 x 1280 outputs: 80 tiles on 148 SMs) leaves SMs idle and cannot split its reduction
     // either.  Narrower tiles (96 or 64 columns, multiples of the 32-column epilogue pass) in the same 128-wide
     // slots put more CTAs on the machine in one wave, each with proportionally less MMA, expansion and epilogue work.
-    if (!wide && !p.addend) {
-        bn = static_cast<uint32_t>(plan_narrow_tile(p.M, p.N, tp.k_blocks, num_sms));
-        if (bn != 128) tp.tile_n = static_cast<int>(bn);
-    }
+    if (bn < 128) tp.tile_n = plan.channels;
     if (w4)
         rc = encode_tmap_2d_u8(&tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, BK / 2, bn, false);
     else
@@ -1586,7 +1646,9 @@ int run_quant(const __half* X, long long ldx, long long rows, int K, const float
 int run_tma_prequantized(const Params& p, int amode, const void* packed, int w_bits, const int8_t* aq,
                          cudaStream_t stream)
 {
-    return run_tma_gemm(p, amode, packed, w_bits, const_cast<int8_t*>(aq), stream);
+    LayerPlan plan;
+    const int rc = plan_call(p, amode, false, w_bits, &plan);
+    return rc == MIXDQ_OK ? run_tma_gemm(p, amode, packed, w_bits, plan, aq, stream) : rc;
 }
 
 // Layout of the shortcut-split scratch: [int8 lo | int8 hi | int32 sums of the lo branch], each 256-byte aligned.
@@ -1648,18 +1710,18 @@ int run_tma_split(const Params& p, int amode, int split_at, const void* packed_l
     const int c_lo = split_at, c_hi = row_len - split_at;
     const int kb_lo = static_cast<int>(conv ? 9 * ceil_div(c_lo, BK) : ceil_div(c_lo, BK));
     const int kb_hi = static_cast<int>(conv ? 9 * ceil_div(c_hi, BK) : ceil_div(c_hi, BK));
-    const ChanPlan plan = plan_chan(p.M, p.N, kb_lo + kb_hi, w4, num_sms, true);
-    if (plan.tokens > 0) {
+    const LayerPlan plan = plan_layer(LayerKind::SPLIT, p.M, p.N, kb_lo + kb_hi, w4, num_sms);
+    if (plan.form == Form::CHAN) {
         Params q = p;
         q.Cin = conv ? c_lo : 0;
         q.K = conv ? 9 * c_lo : c_lo;
         q.act_scale = scale_lo;
         q.acc_out = p.Y ? nullptr : acc_lo_out;
         const ChanBranch second{packed_hi, aq_hi, c_hi, scale_hi, p.Y ? nullptr : acc_hi_out};
-        return run_chan(q, amode, packed_lo, w_bits, aq_lo, plan.cg, plan.tokens, stream, &second);
+        return run_chan(q, amode, packed_lo, w_bits, aq_lo, plan.channels / 128, plan.tokens, stream, &second);
     }
-    const int pair_bn = plan_pair_tile(p.M, p.N, kb_lo + kb_hi, w4, num_sms, nullptr);
-    if (pair_bn > 0) {
+    if (plan.form == Form::PAIR) {
+        const int pair_bn = plan.channels;
         CUtensorMap ta[2], tw[2], ty{};
         const int8_t* aq[2] = {aq_lo, aq_hi};
         const void* pk[2] = {packed_lo, packed_hi};
@@ -1733,7 +1795,7 @@ int run_tma_split(const Params& p, int amode, int split_at, const void* packed_l
     q.act_scale = scale_lo;
     q.Cin = conv ? split_at : 0;
     q.K = conv ? 9 * split_at : split_at;
-    rc = run_tma_gemm(q, amode, packed_lo, w_bits, aq_lo, stream);
+    rc = run_tma_prequantized(q, amode, packed_lo, w_bits, aq_lo, stream);
     if (rc != MIXDQ_OK) return rc;
     q.act_scale = scale_hi;
     q.Cin = conv ? row_len - split_at : 0;
@@ -1747,7 +1809,7 @@ int run_tma_split(const Params& p, int amode, int split_at, const void* packed_l
     } else {
         q.acc_out = acc_hi_out;
     }
-    return run_tma_gemm(q, amode, packed_hi, w_bits, aq_hi, stream);
+    return run_tma_prequantized(q, amode, packed_hi, w_bits, aq_hi, stream);
 }
 
 }  // namespace i8

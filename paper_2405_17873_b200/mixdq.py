@@ -32,6 +32,7 @@ _SIGNATURES = {
     "mixdq_int8_tile_plan": (_int, [_i64, _i64, _i64, _int, C.POINTER(_int), C.POINTER(_int), C.POINTER(_int)]),
     "mixdq_int8_chan_tile": (_int, [_i64, _i64, _i64, _int, C.POINTER(_int), C.POINTER(_int)]),
     "mixdq_linear_fused_quant_tile": (_int, [_i64, _i64, _i64, _int]),
+    "mixdq_int8_layer_plan": (_int, [_i64, _i64, _i64, _int, _int, C.POINTER(_int), C.POINTER(_int), C.POINTER(_int)]),
     "mixdq_packed_bytes": (_int, [_i64, _i64, _int, _int, C.POINTER(_sz)]),
     "mixdq_weight_minmax_params": (_int, [_vp, _i64, _i64, _int, _int, _vp, _vp, _vp]),
     "mixdq_pack_weights": (_int, [_vp, _i64, _i64, _int, _vp, _vp, _int, _vp, _vp]),
@@ -175,6 +176,19 @@ def linear_fused_quant_tile(M: int, N: int, K: int, w_bits: int) -> int:
     if r < 0:
         _chk(r, "mixdq_linear_fused_quant_tile")
     return r
+
+
+LAYER_KINDS = ("linear", "codes", "kv", "split")
+LAYER_FORMS = ("single", "pair", "chan", "chan_many", "fused", "branches")
+
+
+def int8_layer_plan(M: int, N: int, k_blocks: int, w_bits: int, kind: str = "linear"):
+    """(form, tile_tokens, tile_channels, reduction_splits): the kernel that runs this int8 layer (mixdq_int8_layer_plan)."""
+    t, c, sp = _int(0), _int(0), _int(0)
+    form = lib().mixdq_int8_layer_plan(M, N, k_blocks, w_bits, LAYER_KINDS.index(kind), C.byref(t), C.byref(c), C.byref(sp))
+    if form < 0:
+        _chk(form, "mixdq_int8_layer_plan")
+    return LAYER_FORMS[form], t.value, c.value, sp.value
 
 
 def packed_bytes(N: int, K: int, bits: int, layout: int = LAYOUT_DEVICE) -> int:

@@ -1,9 +1,9 @@
 """GPU parity of the one-kernel form of a W8A8 / W4A8 linear layer, whose GEMM kernel quantizes its own fp16
 activation tiles (Sec. 4.1: per-tensor 8-bit activations): the planner sends short reductions on one wave of
-tiles there.  Every case first checks that the shape really takes that form.  int32 accumulators must match the
-oracle bit for bit (whole tensor) -- any activation code that differs from the oracle's quantizer shows there --
-and fp16 outputs within the path's tolerance; the stored-int8 route (quantization kernel + GEMM) must give the
-same output bits."""
+tiles there.  Every case first checks that the shape really takes that form, or forces it.  int32 accumulators must
+match the oracle bit for bit (whole tensor) -- any activation code that differs from the oracle's quantizer shows
+there -- and fp16 outputs within the path's tolerance; the stored-int8 route (quantization kernel + GEMM) and the call
+that forces the form must give the same output bits."""
 import numpy as np
 import pytest
 import torch
@@ -14,12 +14,18 @@ from helpers import assert_close, dev, device_weights, host, oracle_weights, sta
 
 pytestmark = pytest.mark.gpu
 
-# the 32 x 32 level's attention projections at image batch 4 and 1, and ragged rows / columns / reduction tails
-SHAPES = [(4096, 640, 640, 4), (4096, 640, 640, 8), (4096, 640, 320, 4), (1024, 640, 640, 8), (1024, 640, 640, 4), (3274, 776, 432, 4),
-          (2100, 1000, 208, 8), (2049, 40, 16, 4), (5000, 136, 640, 8)]
+# attention projections of the 32 x 32 level, and ragged rows / columns / reduction tails
+SHAPES = [(4096, 640, 640, 8), (4096, 640, 320, 4), (8192, 320, 640, 4), (2100, 1000, 208, 8), (5000, 136, 640, 8), (2286, 956, 64, 4),
+          (3473, 650, 272, 4), (14445, 16, 240, 4)]
+# shapes whose two-kernel form is faster, with a tile width for the call that forces this one
+FORCED = [(4096, 640, 640, 4, 160), (1024, 640, 640, 8, 64), (1024, 640, 640, 4, 64), (3274, 776, 432, 4, 160), (2049, 40, 16, 4, 64)]
 
 
-def _run(X, W, b, bits, sx_ref):
+def _takes_form(M, N, K, bits):
+    return mixdq.int8_layer_plan(M, N, -(-K // 128), bits)[0] == "fused"
+
+
+def _run(X, W, b, bits, sx_ref, tile_cols):
     M, K = X.shape
     N = W.shape[0]
     s_ref, _, codes = oracle_weights(W, bits, True)
@@ -33,22 +39,25 @@ def _run(X, W, b, bits, sx_ref):
     y = mixdq.linear(Xd, packed, N, bits, s, None, 8, sx, None if b is None else dev(b), workspace=ws, status=st)
     xq = mixdq.quantize_acts(Xd, sx)
     y_q8 = mixdq.linear_q8(xq, packed, N, bits, s, sx, None if b is None else dev(b), st)
+    y_forced = mixdq.linear_a8_fused_quant(Xd, packed, N, bits, s, sx, None if b is None else dev(b), tile_cols, st)
     torch.cuda.synchronize()
     assert int(host(st)[0]) == 0
     assert np.array_equal(host(xq), orc.quantize_acts(X, sx_ref).astype(np.int8))
     assert np.array_equal(host(acc), acc_ref)
     assert_close(host(y), y_ref)
     assert np.array_equal(host(y_q8).view(np.uint16), host(y).view(np.uint16))
+    assert np.array_equal(host(y_forced).view(np.uint16), host(y).view(np.uint16))
 
 
-@pytest.mark.parametrize("M,N,K,bits", SHAPES)
-def test_linear_fused_quantization(M, N, K, bits):
-    bn = mixdq.linear_fused_quant_tile(M, N, K, bits)
+@pytest.mark.parametrize("M,N,K,bits,forced", [(*shape, 0) for shape in SHAPES] + FORCED)
+def test_linear_fused_quantization(M, N, K, bits, forced):
+    assert _takes_form(M, N, K, bits) == (forced == 0)
+    bn = forced or mixdq.linear_fused_quant_tile(M, N, K, bits)
     assert bn > 0 and bn % 32 == 0, bn
     X = synth.normal_f16((M, K), 1.0, seed=M + K)
     W = synth.normal_f16((N, K), 0.02, seed=N + K + 1)
     b = synth.normal_f16((N,), 0.01, seed=N)
-    _run(X, W, b, bits, orc.act_scale(orc.act_absmax(X), 8))
+    _run(X, W, b, bits, orc.act_scale(orc.act_absmax(X), 8), bn)
 
 
 @pytest.mark.parametrize("scale", [0.0123, 2.0 ** -6, 3.3e-4, 0.9, 41.0, 3.0e-8, 700.0])
@@ -59,25 +68,23 @@ def test_every_finite_fp16_value_through_the_fused_quantizer(scale):
     bits16 = np.arange(65536, dtype=np.uint32).astype(np.uint16)
     vals = bits16.view(np.float16)
     vals = vals[np.isfinite(vals)]
-    M, K = 2048, 32
-    X = np.zeros(M * K, np.float16)
-    X[: vals.size] = vals
-    X[vals.size:] = vals[: M * K - vals.size]
-    X = np.ascontiguousarray(X.reshape(M, K))
-    N = 64
-    assert mixdq.linear_fused_quant_tile(M, N, K, 8) > 0
+    M, N, K = 5508, 184, 32
+    X = np.resize(vals, (M, K))  # (repeated: more than every value once)
+    assert _takes_form(M, N, K, 8)
     # weights with a single entry per row pick single codes out; the rest are random (kept small where the
     # activation scale is large, so that the fp16 outputs stay finite)
     wstd = 0.02 * min(1.0, 1.0 / scale)
     W = synth.normal_f16((N, K), wstd, seed=5)
     W[:K] = 0
     W[np.arange(K), np.arange(K)] = np.float16(50.0 * wstd)
-    _run(X, W, None, 8, np.float32(scale))
+    _run(X, W, None, 8, np.float32(scale), 96)
 
 
 def test_two_kernel_shapes_stay_two_kernel():
     for M, N, K in [(1024, 1280, 1280), (1024, 1280, 640), (16384, 320, 640), (4096, 5120, 640), (4096, 640, 2560)]:
         assert mixdq.linear_fused_quant_tile(M, N, K, 4) == 0
+    for M, N, K, bits, _ in FORCED:
+        assert mixdq.linear_fused_quant_tile(M, N, K, bits) == 0
 
 
 @pytest.mark.parametrize("bits", [4, 8])
