@@ -566,7 +566,7 @@ def sub_sweep_record(torch, UNetSweep, stream, peaks, batch, tokens, steps=10):
 def run_ours(args):
     import torch
     import torch.distributed as dist
-    from paper_2405_17873_b200 import build, mixdq, replicas
+    from paper_2405_17873_b200 import build, mixdq, replicas, synth
     from paper_2405_17873_b200.unet_sweep import UNetSweep
 
     rank = int(os.environ.get("RANK", "0"))
@@ -824,7 +824,6 @@ def run_ours(args):
                        not args.shortcut_split and not args.share_qkv_quant and not args.fuse_projections and
                        args.batch == 4 and not args.no_extras)
         if default_run:
-            from paper_2405_17873_b200 import synth
             out["peaks"] = {"measured": {"hbm_gbs": peaks["hbm_gbs"], "bf16_tflops_burst": peaks["bf16_tflops"],
                                          "bf16_tflops_sustained": peaks["bf16_tflops_sustained"],
                                          "int8_mma_loop_probe_tops": round(probe_int8, 1), "source": peaks["source"]},
