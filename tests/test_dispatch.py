@@ -5,6 +5,7 @@ import random
 
 import pytest
 
+import test_gpu_forms as forms
 from paper_2405_17873_b200 import mixdq
 from recorded import BUFFER, Recorded
 
@@ -66,3 +67,26 @@ def test_argument_errors(lib):
     assert plan(64, 64, 1, 8, 0, t, c, sp) >= 0
     assert plan(0, 64, 1, 8, 0, t, c, sp) == -1 and plan(64, 64, 1, 8, 4, t, c, sp) == -1 and plan(64, 64, 1, 8, 0, None, c, sp) == -1
     assert plan(64, 64, 1, 3, 0, t, c, sp) == -2
+
+
+def _launches(lib, kernel, case, call):
+    assert call(lib.so) == 0
+    names = [name for name, _ in lib.launches()]
+    assert kernel in names[-1], (case, names)
+
+
+def test_cases_of_the_rare_kernels_launch_them(lib):
+    """(of test_gpu_forms.py)"""
+    ws = lambda use: (BUFFER, BYTES) if use else (None, C.c_size_t(0))
+    for bits, sym, M, K, N, use, kernel in forms.LINEAR_A16:
+        _launches(lib, kernel, (bits, M, K, N), lambda so: so.mixdq_linear(
+            BUFFER, M, K, -(-K // 8) * 8, BUFFER, N, bits, BUFFER, None if sym else BUFFER, 16, None, BUFFER, BUFFER, *ws(use), None, None))
+    for bits, (B, H, W, Cin, Cout, stride), use, kernel in forms.CONV_A16:
+        _launches(lib, kernel, (bits, B, H, W, Cin, Cout, stride), lambda so: so.mixdq_conv3x3(
+            BUFFER, B, H, W, Cin, BUFFER, Cout, stride, bits, BUFFER, BUFFER, 16, None, BUFFER, BUFFER, *ws(use), None, None))
+    for bits, M, N, K, kernel in forms.LINEAR_Q8:
+        _launches(lib, kernel, (bits, M, N, K), lambda so: so.mixdq_linear_q8(
+            BUFFER, M, K, BUFFER, N, bits, BUFFER, BUFFER, None, BUFFER, None, None))
+    for bits, M, lo, hi, N, kernel in forms.SPLIT_A8:
+        _launches(lib, kernel, (bits, M, lo, hi, N), lambda so: so.mixdq_linear_a8_split(
+            BUFFER, M, lo + hi, lo + hi, lo, BUFFER, BUFFER, N, bits, BUFFER, BUFFER, BUFFER, None, BUFFER, BUFFER, BYTES, None, None))

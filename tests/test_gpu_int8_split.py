@@ -139,16 +139,14 @@ def _kb(c):
                                                        (5, 32, 32, 320, 320, 648, 1)])
 def test_split_conv_in_one_kernel(bits, B, H, W_, C_lo, C_hi, N, stride):
     Ho = (H - 1) // stride + 1
-    rows, cols = mixdq.int8_tile_plan(B * Ho * Ho, N, 9 * (_kb(C_lo) + _kb(C_hi)), bits)
-    assert rows == 256, (rows, cols)
+    assert mixdq.int8_layer_plan(B * Ho * Ho, N, 9 * (_kb(C_lo) + _kb(C_hi)), bits, "split")[0] == "pair"
     _run_conv(B, H, W_, C_lo, C_hi, N, bits, stride, seed=H + C_lo + N + 7)
 
 
 @pytest.mark.parametrize("bits", [8, 4])
 @pytest.mark.parametrize("M,C_lo,C_hi,N", [(5567, 400, 384, 776), (16384, 320, 320, 320), (4458, 1296, 656, 648)])
 def test_split_linear_in_one_kernel(bits, M, C_lo, C_hi, N):
-    rows, cols = mixdq.int8_tile_plan(M, N, _kb(C_lo) + _kb(C_hi), bits)
-    assert rows == 256, (rows, cols)
+    assert mixdq.int8_layer_plan(M, N, _kb(C_lo) + _kb(C_hi), bits, "split")[0] == "pair"
     _run_linear(M, C_lo, C_hi, N, bits, seed=M + C_lo + N + 7)
 
 
