@@ -353,6 +353,19 @@ int mixdq_selftest_abandoned_wait(const void* Xq, int64_t M, int64_t K, const vo
                                   const float* w_scale, const float* act_scale, void* Y, int drop_k_block,
                                   int32_t* status, void* stream);
 
+/*
+ * The same for the channel-major kernels, which run most layers, on the form that the layer takes: mixdq_linear_q8
+ * (act_bits 8, X int8 codes [M, K], w_zero NULL), a shortcut-split layer with one activation scale on its branches' codes (X,
+ * and X_hi [M, K_hi], with packed_W and packed_W_hi; X_hi NULL: no second branch), or the weight-only mixdq_linear without a
+ * workspace (act_bits 16, X fp16 [M, K], act_scale unused).  Weights never come, or not whole: where one wave of int8 tiles
+ * suffices from the first block of the last branch on, else from reduction block drop_k_block on (in the last of the tiles
+ * that a CTA pair walks).  MIXDQ_ERR_UNSUPPORTED where the layer takes another kernel.
+ */
+int mixdq_selftest_abandoned_chan_wait(const void* X, int64_t M, int64_t K, const void* packed_W, const void* X_hi,
+                                       int64_t K_hi, const void* packed_W_hi, int64_t N, int w_bits, const float* w_scale,
+                                       const int32_t* w_zero, int act_bits, const float* act_scale, void* Y,
+                                       int drop_k_block, int32_t* status, void* stream);
+
 /* Parity hook: int32 accumulators [M, N] of mixdq_linear_q8. */
 int mixdq_linear_q8_acc_i32(const void* Xq, int64_t M, int64_t K, const void* packed_W, int64_t N, int w_bits,
                             int32_t* acc_out, int32_t* status, void* stream);

@@ -368,7 +368,7 @@ namespace {
 
 int linear_q8_impl(const void* Xq, int64_t M, int64_t K, const void* packed_W, int64_t N, int w_bits,
                    const float* w_scale, const float* act_scale, const void* bias, void* Y, int32_t* acc_out,
-                   int32_t* status, void* stream, int test_drop_b_kblock = 0)
+                   int32_t* status, void* stream, int test_drop_b_kblock = 0, bool test_planned = false)
 {
     if (!Xq || !packed_W || (!Y && !acc_out)) return MIXDQ_ERR_INVALID_ARG;
     if (!fits_int(M) || !fits_int(K) || !fits_int(N)) return MIXDQ_ERR_INVALID_ARG;
@@ -389,6 +389,7 @@ int linear_q8_impl(const void* Xq, int64_t M, int64_t K, const void* packed_W, i
     p.acc_out = acc_out;
     p.status = status;
     p.test_drop_b_kblock = test_drop_b_kblock;
+    p.test_planned = test_planned;
     return i8::run_tma_prequantized(p, A_LINEAR, packed_W, w_bits, static_cast<const int8_t*>(Xq),
                                     static_cast<cudaStream_t>(stream));
 }
@@ -437,6 +438,58 @@ extern "C" int mixdq_selftest_abandoned_wait(const void* Xq, int64_t M, int64_t 
     if (drop_k_block < 1 || drop_k_block > (K + 127) / 128) return MIXDQ_ERR_INVALID_ARG;
     return linear_q8_impl(Xq, M, K, packed_W, N, w_bits, w_scale, act_scale, nullptr, Y, nullptr, status, stream,
                           drop_k_block);
+}
+
+extern "C" int mixdq_selftest_abandoned_chan_wait(const void* X, int64_t M, int64_t K, const void* packed_W,
+                                                  const void* X_hi, int64_t K_hi, const void* packed_W_hi, int64_t N,
+                                                  int w_bits, const float* w_scale, const int32_t* w_zero, int act_bits,
+                                                  const float* act_scale, void* Y, int drop_k_block, int32_t* status,
+                                                  void* stream)
+{
+    if (!X || !packed_W || !w_scale || !Y || !status) return MIXDQ_ERR_INVALID_ARG;
+    if (!fits_int(M) || !fits_int(K) || !fits_int(N)) return MIXDQ_ERR_INVALID_ARG;
+    if (X_hi && (!packed_W_hi || !fits_int(K_hi) || act_bits != 8 || !act_scale)) return MIXDQ_ERR_INVALID_ARG;
+    if (drop_k_block < 1 || drop_k_block > (K + 127) / 128) return MIXDQ_ERR_INVALID_ARG;
+    const int rc = check_widths(w_bits, act_bits, w_zero);
+    if (rc != MIXDQ_OK) return rc;
+    if (act_bits == 8 && !X_hi)
+        return linear_q8_impl(X, M, K, packed_W, N, w_bits, w_scale, act_scale, nullptr, Y, nullptr, status, stream,
+                              drop_k_block, true);
+    if (X_hi) {
+        if (K % 16 != 0 || K_hi % 16 != 0) return MIXDQ_ERR_UNSUPPORTED;
+        if (!aligned16(X) || !aligned16(packed_W) || !aligned16(X_hi) || !aligned16(packed_W_hi)) return MIXDQ_ERR_ALIGNMENT;
+        const int sms = sm_count();
+        if (sms <= 0) return MIXDQ_ERR_CUDA;
+        const i8::LayerPlan plan = i8::plan_layer(i8::LayerKind::SPLIT, static_cast<int>(M), static_cast<int>(N),
+                                                  static_cast<int>(ceil_div(K, 128) + ceil_div(K_hi, 128)), w_bits == 4, sms);
+        if (plan.form != i8::Form::CHAN) return MIXDQ_ERR_UNSUPPORTED;
+        i8::Params p;
+        p.M = static_cast<int>(M);
+        p.N = static_cast<int>(N);
+        p.K = static_cast<int>(K);
+        p.act_scale = act_scale;
+        p.w_scale = w_scale;
+        p.Y = static_cast<__half*>(Y);
+        p.ldy = N;
+        p.status = status;
+        p.test_drop_b_kblock = drop_k_block;
+        const i8::ChanBranch second{packed_W_hi, static_cast<const int8_t*>(X_hi), static_cast<int>(K_hi), act_scale, nullptr};
+        return i8::run_chan(p, A_LINEAR, packed_W, w_bits, static_cast<const int8_t*>(X), plan.channels / 128, plan.tokens,
+                            static_cast<cudaStream_t>(stream), &second);
+    }
+    wo::Params p;
+    p.X = static_cast<const __half*>(X);
+    p.ldx = K;
+    p.M = static_cast<int>(M);
+    p.N = static_cast<int>(N);
+    p.K = static_cast<int>(K);
+    p.w_scale = w_scale;
+    p.w_zero = w_zero;
+    p.Y = static_cast<__half*>(Y);
+    p.ldy = N;
+    p.status = status;
+    p.test_drop_b_kblock = drop_k_block;
+    return wo::run(p, A_LINEAR, packed_W, w_bits, static_cast<cudaStream_t>(stream));
 }
 
 extern "C" int mixdq_linear_q8_acc_i32(const void* Xq, int64_t M, int64_t K, const void* packed_W, int64_t N,

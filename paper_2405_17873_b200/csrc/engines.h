@@ -43,9 +43,10 @@ struct Params {
     // activation scale; the epilogue adds addend * (*addend_scale) * w_scale[n]
     const int32_t* addend = nullptr;
     const float* addend_scale = nullptr;
-    // self-test of the bounded waits (mixdq_selftest_abandoned_wait): > 0 = the weight tile of that k-block
-    // (1-based) is announced to its barrier but never requested, so the waits on it run out
+    // self-test of the bounded waits: > 0 = the weight tile of that k-block (1-based) is never requested, so the waits on
+    // it run out; on the single-CTA kernels, or (test_planned) on the channel-major form that the layer takes
     int test_drop_b_kblock = 0;
+    bool test_planned = false;
 };
 
 // Scratch of the fused kernel's split reduction (tickets + int32 partial sums).
@@ -148,6 +149,7 @@ struct Params {
     // optional scratch for the layer's weights expanded to fp16 (many-token path); no initial content needed
     void* workspace = nullptr;
     size_t ws_bytes = 0;
+    int test_drop_b_kblock = 0;  // self-test, channel-major form only (see i8::Params)
 };
 
 int run(Params p, int amode, const void* packed, int w_bits, cudaStream_t stream);

@@ -444,15 +444,15 @@ int launch(const CUtensorMap* maps, const TmaParams& tp, const ChanArgs& g, int 
 }  // namespace
 
 // Tensor maps of one branch: its weights [N, taps * cin] and its activations, int8 [M, cin] or the NHWC image of cin channels
-// (with its border when pad is set).
+// (with its border when pad is set).  w_rows: channels of a weight tile that arrive, CH but for the self-test.
 int encode_chan_branch(CUtensorMap* tw, CUtensorMap* tx, const Params& p, bool conv, int pad, int cin, const void* packed, bool w4, bool wide,
-                  const int8_t* codes, int rows)
+                       const int8_t* codes, int rows, int w_rows)
 {
     const int64_t K = (conv ? 9ll : 1ll) * cin;
     const int64_t pitch = row_pitch_bytes(K, w4 ? 4 : 8, MIXDQ_LAYOUT_DEVICE);
-    const int rc = w4 ? encode_tmap_2d_u8(tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, wide ? BK : BK / 2, CH,
+    const int rc = w4 ? encode_tmap_2d_u8(tw, packed, static_cast<uint64_t>(pitch), p.N, pitch, wide ? BK : BK / 2, w_rows,
                                           wide ? SWIZZLE_128 : SWIZZLE_64)
-                      : encode_tmap_2d_u8(tw, packed, static_cast<uint64_t>(K), p.N, pitch, BK, CH, SWIZZLE_128);
+                      : encode_tmap_2d_u8(tw, packed, static_cast<uint64_t>(K), p.N, pitch, BK, w_rows, SWIZZLE_128);
     if (rc != MIXDQ_OK) return rc;
     if (conv) return encode_tmap_im2col3x3(tx, codes, false, p.batch, p.H + 2 * pad, p.W + 2 * pad, cin, pad, p.stride, BK, rows);
     return encode_tmap_2d_u8(tx, codes, static_cast<uint64_t>(cin), static_cast<uint64_t>(p.M), static_cast<uint64_t>(cin), BK,
@@ -504,10 +504,15 @@ int run_chan(const Params& p, int amode, const void* packed, int w_bits, const i
         tp.Wo = p.Wo;
     }
     CUtensorMap maps[4]{};  // weights, activations; the second branch's
-    int rc = encode_chan_branch(&maps[0], &maps[1], p, conv, pad, cin, packed, w4, g.wide, codes, rows);
+    // self-test of the bounded waits: half of every weight tile of the last branch never comes, so that the waits on the first
+    // of them run out.  (A producer that left tiles out would do for any of them, but a test of it in the kernel, even a bound
+    // passed in, cost the 4096 x 640 x 640 W8 layer 0.13 to 0.2 us.)
+    const int last_rows = p.test_drop_b_kblock ? CH / 2 : CH;
+    int rc = encode_chan_branch(&maps[0], &maps[1], p, conv, pad, cin, packed, w4, g.wide, codes, rows, second ? CH : last_rows);
     if (rc != MIXDQ_OK) return rc;
     if (!second) return launch<false>(maps, tp, g, cg, w4, stream);
-    rc = encode_chan_branch(&maps[2], &maps[3], p, conv, pad, second->cin, second->packed, w4, g.wide, second->codes, rows);
+    rc = encode_chan_branch(&maps[2], &maps[3], p, conv, pad, second->cin, second->packed, w4, g.wide, second->codes, rows,
+                            last_rows);
     if (rc != MIXDQ_OK) return rc;
     g.kb_lo = tp.k_blocks;
     g.cblocks2 = static_cast<int>(ceil_div(second->cin, BK));

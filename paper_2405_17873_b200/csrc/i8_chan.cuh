@@ -219,7 +219,7 @@ __device__ __forceinline__ void store_tokens(uint32_t acc, uint32_t acc2, int c0
 }
 
 int encode_chan_branch(CUtensorMap* tw, CUtensorMap* tx, const Params& p, bool conv, int pad, int cin, const void* packed, bool w4,
-                       bool wide, const int8_t* codes, int rows);
+                       bool wide, const int8_t* codes, int rows, int w_rows = CH);
 
 }  // namespace i8
 }  // namespace mixdq

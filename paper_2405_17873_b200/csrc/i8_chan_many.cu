@@ -174,8 +174,9 @@ chan_many_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
             const int tile = pair0 + t * npairs;
             const int n0 = (tile % g.c_tiles) * (2 * CH) + static_cast<int>(rank) * CH;
             const int first = (which + t * pairs) & 1;
+            const int end = p.test_drop_b_kblock && t == my_tiles - 1 ? (p.test_drop_b_kblock - 1) >> 1 : pairs;
             KPos at(2 * first, p.cblocks);
-            for (int j = first; j < pairs; j += 2) {
+            for (int j = first; j < end; j += 2) {
                 ok = mbar_wait(bar0 + 8 * (EMPTY_P + s), par, abort_flag);
                 if (!__all_sync(0xffffffffu, ok)) {
                     ok = false;
@@ -406,6 +407,7 @@ int run_chan_many(const Params& p, int amode, const void* packed, const int8_t* 
     tp.ldy = p.ldy;
     tp.acc_out = p.acc_out;
     tp.status = p.status;
+    tp.test_drop_b_kblock = p.test_drop_b_kblock;
     tp.cblocks = static_cast<int>(ceil_div(cin, BK));
     tp.k_blocks = (conv ? 9 : 1) * tp.cblocks;
     if (!chan_many_tile_ok(tokens, tp.k_blocks) || amode == A_BOS || p.addend) return MIXDQ_ERR_INVALID_ARG;

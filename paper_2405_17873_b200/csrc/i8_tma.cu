@@ -1470,14 +1470,14 @@ int run_fq(const Params& p, const void* packed, int w_bits, int bn, cudaStream_t
     return launch_fq(tx, tw, ty, tp, w4, bn, stream);
 }
 
-// The plan of a call; the self-test of the bounded waits runs on the single-CTA kernels.
+// The plan of a call.
 static int plan_call(const Params& p, int amode, bool fp16_rows, int w_bits, LayerPlan* plan)
 {
     const int num_sms = sm_count();
     if (num_sms <= 0) return MIXDQ_ERR_CUDA;
     const bool w4 = w_bits == 4;
     const int k_blocks = static_cast<int>(amode == A_CONV3 ? 9 * ceil_div(p.Cin, BK) : ceil_div(p.K, BK));
-    if (p.test_drop_b_kblock) {
+    if (p.test_drop_b_kblock && !p.test_planned) {
         *plan = LayerPlan{};
         plan->tokens = BM;
         plan->channels = plan_single_tile(p.M, p.N, k_blocks, w4, num_sms);
@@ -1487,6 +1487,7 @@ static int plan_call(const Params& p, int amode, bool fp16_rows, int w_bits, Lay
                                     : (amode == A_BOS ? LayerKind::BOS
                                                       : (fp16_rows && amode == A_LINEAR && !p.act_zero ? LayerKind::ROWS : LayerKind::CODES));
     *plan = plan_layer(kind, p.M, p.N, k_blocks, w4, num_sms);
+    if (p.test_drop_b_kblock && plan->form != Form::CHAN && plan->form != Form::CHAN_MANY) return MIXDQ_ERR_UNSUPPORTED;
     return MIXDQ_OK;
 }
 

@@ -230,7 +230,9 @@ wo_chan_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
             mbar_arrive_expect_tx(full, P_BYTES);
             tma_load_2d(p0 + s * P_BYTES, &tmap_w, u * 16 * BITS, n0, full);
         };
-        produce<false>(warp == 1 ? 0 : 1, lane, PS, pr, 1 << 30, 1, bar0 + 8 * EMPTY_P, PS, abort_flag, request);
+        Pairs<false> requested = pr;
+        if (p.test_drop_b_kblock) requested.n = min(pr.n, p.test_drop_b_kblock - 1);
+        produce<false>(warp == 1 ? 0 : 1, lane, PS, requested, 1 << 30, 1, bar0 + 8 * EMPTY_P, PS, abort_flag, request);
     } else if (warp == 2 || warp == HELP0 + 1) {
         // ------------------------------------------------------------ fp16 token rows by TMA
         const int m0 = tok0 + static_cast<int>(rank) * rows;
@@ -457,6 +459,7 @@ int run_chan(const Params& p, int amode, const void* packed, int w_bits, int cg,
     tp.Y = p.Y;
     tp.ldy = p.ldy;
     tp.status = p.status;
+    tp.test_drop_b_kblock = p.test_drop_b_kblock;
     tp.cblocks = static_cast<int>(ceil_div(conv ? p.Cin : p.K, BKE));
     tp.k_blocks = (conv ? 9 : 1) * tp.cblocks;
     const int rows = tokens / cg;

@@ -539,6 +539,7 @@ int run(Params p, int amode, const void* packed, int w_bits, cudaStream_t stream
         const int tokens = plan_chan(p, amode, w_bits, pair, num_sms, &cg);
         if (tokens > 0) return run_chan(p, amode, packed, w_bits, cg, tokens, stream);
     }
+    if (p.test_drop_b_kblock) return MIXDQ_ERR_UNSUPPORTED;
     if (pair) return run_pair(p, amode, packed, w_bits, stream);
     if (tc_path_ok(p, amode, w_bits) && !(w_bits <= 3 && is_signed)) return run_tc(p, amode, packed, w_bits, p.batch, stream);
     if (w_bits == 3) return is_signed ? MIXDQ_ERR_UNSUPPORTED : launch_nt<3, false>(p, amode, packed, pitch, stream);

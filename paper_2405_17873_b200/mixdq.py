@@ -57,6 +57,7 @@ _SIGNATURES = {
     "mixdq_conv3x3_q8": (_int, [_vp, _i64, _i64, _i64, _i64, _vp, _i64, _int, _int, _vp, _vp, _vp, _vp, _vp, _vp]),
     "mixdq_linear_a8_fused_quant": (_int, [_vp, _i64, _i64, _i64, _vp, _i64, _int, _vp, _vp, _vp, _vp, _i64, _int, _vp, _vp]),
     "mixdq_selftest_abandoned_wait": (_int, [_vp, _i64, _i64, _vp, _i64, _int, _vp, _vp, _vp, _int, _vp, _vp]),
+    "mixdq_selftest_abandoned_chan_wait": (_int, [_vp, _i64, _i64, _vp, _vp, _i64, _vp, _i64, _int, _vp, _vp, _int, _vp, _vp, _int, _vp, _vp]),
     "mixdq_linear_q8_acc_i32": (_int, [_vp, _i64, _i64, _vp, _i64, _int, _vp, _vp, _vp]),
     "mixdq_split_workspace_bytes": (_int, [_i64, _i64, _i64, _i64, _i64, C.POINTER(_sz)]),
     "mixdq_linear_a8_split": (_int, [_vp, _i64, _i64, _i64, _i64, _vp, _vp, _i64, _int, _vp, _vp, _vp, _vp, _vp, _vp,
@@ -273,6 +274,18 @@ def selftest_abandoned_wait(Xq, packed_W, N: int, w_bits: int, w_scale, act_scal
     _chk(lib().mixdq_selftest_abandoned_wait(_ptr(Xq), M, K, _ptr(packed_W), N, w_bits, _ptr(w_scale), _ptr(act_scale),
                                              _ptr(Y), drop_k_block, _ptr(status), _stream()),
          "mixdq_selftest_abandoned_wait")
+    return Y
+
+
+def selftest_abandoned_chan_wait(X, packed_W, N: int, w_bits: int, w_scale, w_zero, act_bits: int, act_scale, drop_k_block: int,
+                                 status, X_hi=None, packed_W_hi=None):
+    """The same on the channel-major kernel that runs the layer (act_bits 8: X int8 codes, X_hi a second branch's; 16: X fp16)."""
+    M, K = X.shape
+    K_hi = 0 if X_hi is None else X_hi.shape[1]
+    Y = torch.empty((M, N), dtype=torch.float16, device=X.device)
+    _chk(lib().mixdq_selftest_abandoned_chan_wait(_ptr(X), M, K, _ptr(packed_W), _ptr(X_hi), K_hi, _ptr(packed_W_hi), N, w_bits,
+                                                  _ptr(w_scale), _ptr(w_zero), act_bits, _ptr(act_scale), _ptr(Y), drop_k_block,
+                                                  _ptr(status), _stream()), "mixdq_selftest_abandoned_chan_wait")
     return Y
 
 
