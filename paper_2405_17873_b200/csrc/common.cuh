@@ -293,6 +293,17 @@ __device__ __forceinline__ bool mbar_wait(uint32_t bar, uint32_t parity, volatil
     return mbar_wait_poll(bar, parity, abort_flag);
 }
 
+// What every thread does before a kernel's last barrier: where a wait has run out, gives copies that may still be in flight
+// time to land before shared memory goes away, and reports.  Whoever sees the flag reports: thread 0 may have come through
+// here before another thread gave up.
+__device__ __forceinline__ void report_abandoned_wait(const volatile int* abort_flag, int32_t* status)
+{
+    if (*abort_flag) {
+        for (int i = 0; i < 64; ++i) __nanosleep(1000);
+        if (status) atomicExch(status, MIXDQ_ERR_TIMEOUT);
+    }
+}
+
 // One lane of a converged warp.
 __device__ __forceinline__ bool elect_one()
 {

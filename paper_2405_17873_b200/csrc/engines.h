@@ -44,7 +44,8 @@ struct Params {
     const int32_t* addend = nullptr;
     const float* addend_scale = nullptr;
     // self-test of the bounded waits: > 0 = the weight tile of that k-block (1-based) is never requested, so the waits on
-    // it run out; on the single-CTA kernels, or (test_planned) on the channel-major form that the layer takes
+    // it run out; on the single-CTA kernels, or (test_planned) on the channel-major form that the layer takes (there of all
+    // k-blocks from it on, or, see run_chan, of the last branch)
     int test_drop_b_kblock = 0;
     bool test_planned = false;
 };

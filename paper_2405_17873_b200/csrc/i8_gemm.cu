@@ -422,11 +422,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const Params p)
         }
     }
 
-    if (*s_abort) {
-        // give copies that may still be in flight time to land before shared memory goes away
-        for (int i = 0; i < 64; ++i) __nanosleep(1000);
-        if (tid == 0 && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
-    }
+    report_abandoned_wait(s_abort, p.status);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, BN);

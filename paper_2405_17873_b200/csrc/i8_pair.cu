@@ -782,10 +782,7 @@ pair_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_consta
         }
     }
 
-    if (*s_abort) {
-        for (int i = 0; i < 64; ++i) __nanosleep(1000);
-        if (tid == 0 && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
-    }
+    report_abandoned_wait(s_abort, p.status);
     // neither CTA leaves (or frees tensor memory) while its peer may still read its shared memory, signal its
     // barriers or run instructions that write its tensor memory
     tc_fence_before_sync();

@@ -850,10 +850,7 @@ tma_gemm_kernel(const __grid_constant__ CUtensorMap tmap_a, const __grid_constan
             }
         }
     }
-    if (*s_abort) {
-        for (int i = 0; i < 64; ++i) __nanosleep(1000);
-        if (tid == 0 && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
-    }
+    report_abandoned_wait(s_abort, p.status);
     tc_fence_before_sync();
     __syncthreads();
     if (splits > 1) cluster_sync();  // peers may still be reading this CTA's shared memory
@@ -1116,10 +1113,7 @@ tma_gemm_persistent_kernel(const __grid_constant__ CUtensorMap tmap_a, const __g
         pdl_wait();
     }
 
-    if (*s_abort) {
-        for (int i = 0; i < 64; ++i) __nanosleep(1000);
-        if (tid == 0 && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
-    }
+    report_abandoned_wait(s_abort, p.status);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, 2 * L::ACC_COLS);

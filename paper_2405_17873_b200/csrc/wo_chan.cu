@@ -352,10 +352,7 @@ wo_chan_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_constant
         }
     }
 
-    if (*abort_flag) {
-        for (int i = 0; i < 64; ++i) __nanosleep(1000);
-        if (tid == 0 && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
-    }
+    report_abandoned_wait(abort_flag, p.status);
     tc_fence_before_sync();
     __syncthreads();
     if (CG == 2) cluster_sync();  // neither CTA leaves while its peer may still signal its barriers or use its memory

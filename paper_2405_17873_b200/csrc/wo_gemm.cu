@@ -409,7 +409,7 @@ wo_small_kernel(const uint8_t* __restrict__ packed, long long pitch, const Param
     }
     __syncthreads();
     const bool x_ok = mbar_wait(smem_u32(&x_bar), 0, &x_abort);
-    if (!x_ok && tid == 0 && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
+    if (!x_ok && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
 
     for (; grp < groups; grp += gridDim.x) {
         const __half2 zlo_a = __float2half2_rn(1024.f + z_a), zhi_a = __float2half2_rn(-(64.f + z_a));

@@ -387,10 +387,7 @@ wo_tc_kernel(const __grid_constant__ CUtensorMap tmap_x, const TcParams p, int n
         }
     }
 
-    if (*s_abort) {
-        for (int i = 0; i < 64; ++i) __nanosleep(1000);
-        if (tid == 0 && p.status) atomicExch(p.status, MIXDQ_ERR_TIMEOUT);
-    }
+    report_abandoned_wait(s_abort, p.status);
     tc_fence_before_sync();
     __syncthreads();
     if (warp == 1) tmem_dealloc(tmem_base, 2 * BN);

@@ -59,12 +59,13 @@ def _gives_up(call, status):
     assert int(host(status)[0]) == MIXDQ_ERR_TIMEOUT
 
 
-# one- and two-CTA tiles, tiles that a CTA pair walks one after another; the first weight tile and one in the middle (int8 layers
-# of one wave: always the first)
+# one- and two-CTA tiles, tiles that a CTA pair walks one after another; the first weight tile, one in the middle, the last
+# (int8 layers of one wave: always the first)
 @pytest.mark.parametrize("bits,act_bits,M,N,K,drop,form", [
     (8, 8, 100, 320, 640, 1, "chan"), (4, 8, 256, 1280, 1296, 1, "chan"), (4, 8, 1024, 1280, 2560, 1, "chan"),
-    (8, 8, 1024, 1280, 2560, 1, "chan"), (4, 8, 4096, 5120, 640, 3, "chan_many"), (4, 8, 1024, 10240, 1280, 1, "chan_many"),
-    (3, 16, 64, 320, 1288, 1, None), (4, 16, 1024, 1280, 2560, 11, None), (8, 16, 300, 1280, 648, 5, None)])
+    (8, 8, 1024, 1280, 2560, 1, "chan"), (4, 8, 1024, 10240, 1536, 11, "chan_many"), (4, 8, 4096, 5120, 640, 3, "chan_many"), (4, 8, 1024, 10240, 1280, 1, "chan_many"),
+    (3, 16, 64, 320, 1288, 1, None), (4, 16, 1024, 1280, 2560, 11, None), (8, 16, 300, 1280, 648, 5, None),
+    (8, 16, 300, 1280, 1024, 8, None)])
 def test_abandoned_wait_in_the_channel_major_kernels(bits, act_bits, M, N, K, drop, form):
     if form:
         assert mixdq.int8_layer_plan(M, N, -(-K // 128), bits, "codes")[0] == form
@@ -89,7 +90,9 @@ def test_abandoned_wait_in_the_channel_major_kernels(bits, act_bits, M, N, K, dr
     assert_close(host(y), y_ref)
 
 
-@pytest.mark.parametrize("bits,M,N,lo,hi", [(8, 100, 320, 640, 640), (4, 1024, 1280, 1280, 1280), (4, 100, 320, 512, 384)])
+@pytest.mark.parametrize("bits,M,N,lo,hi", [(8, 100, 320, 640, 640), (4, 1024, 1280, 1280, 1280), (4, 100, 320, 512, 384),
+                                               # the last pair of k-blocks alone, which is not the first issuer's: that one has long finished
+                                               (8, 100, 320, 640, 128), (4, 1024, 1280, 640, 128)])
 def test_abandoned_wait_in_the_second_branch(bits, M, N, lo, hi):
     assert mixdq.int8_layer_plan(M, N, -(-lo // 128) - (-hi // 128), bits, "split")[0] == "chan"
     X, W = synth.normal_f16((M, lo + hi), 1.0, seed=61), synth.normal_f16((N, lo + hi), 0.02, seed=62)
