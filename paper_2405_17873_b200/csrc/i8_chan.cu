@@ -294,9 +294,9 @@ chan_gemm_kernel(const __grid_constant__ CUtensorMap tmap_w, const __grid_consta
     } else if (expander) {
         // ------------------------------------------------------------ packed int4 -> int8 (x16) in tensor memory
         // A thread owns a channel: its 64 packed bytes of a k-block become 32 columns of its lane.  Groups of four warps
-        // take alternate pairs and fetch the next packed rows into registers before they wait for its slots.  (One k-block at a time, a turn took its group 1200 cycles, half of them for the waits and
-        // arrivals.)  The swizzle of the rows (128 bytes, or 64 where a pair is not contiguous) makes the reads
-        // conflict-free.
+        // take alternate pairs and fetch the next packed rows into registers before they wait for its slots.  (One k-block at
+        // a time, a turn took its group 1200 cycles, half of them for the waits and arrivals.)  The swizzle of the rows (128
+        // bytes, or 64 where a pair is not contiguous) makes the reads conflict-free.
         const int group = (warp - WORK0) >> 2, row = (warp & 3) * 32 + lane;
         constexpr uint32_t PS = L::PS > 0 ? L::PS : 1;
         const uint32_t a_lane = tmem_base + (static_cast<uint32_t>((warp & 3) * 32) << 16) + g.a_col;

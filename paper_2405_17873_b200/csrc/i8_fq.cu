@@ -11,10 +11,10 @@
 // Measured on B200, this form is bound by the converter warps' turn (waits, some 3.3 instructions per element,
 // proxy fence, arrival: 1500 cycles per k-block and more against 420 to 580 for the two-kernel path's main loop),
 // so it pays only where the reduction is short and the quantization pass large: at most five k-blocks and one wave of
-// tiles.  There the planner takes it (fq_tile, two_kernels_win in i8_tma.cu): over 56 layers that it takes, of 1024 to
-// 16384 rows and 64 to 1000 channels, the two-kernel form took 1.24 times the time on average, from 1.0 (16384 x 320 x 320)
-// over 1.09 (4096 x 640 x 640 W8, 7.4 us against 8.0) to 1.6 (15781 x 192 x 400 W8, 7.6 against 12.5).  Everything else, and
-// asymmetric activations, convolutions and the BOS-aware projection, stay on the two-kernel path.
+// tiles.  There the planner takes it (fq_tile, two_kernels_win in i8_tma.cu): over 54 layers that it takes, of 1024 to
+// 16384 rows and 64 to 1000 channels in eights, the two-kernel form took 1.25 times the time on average, from 1.03 (4096 x
+// 640 x 320 W4, 7.0 us against 7.2) over 1.09 (4096 x 640 x 640 W8, 7.4 and 8.0) to 1.67 (8645 x 368 x 128 W4, 5.2 and 8.7).
+// Everything else, and asymmetric activations, convolutions and the BOS-aware projection, stay on the two-kernel path.
 #include "common.cuh"
 #include "engines.h"
 #include "i8_tiles.cuh"

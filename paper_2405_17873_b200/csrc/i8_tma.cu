@@ -1199,6 +1199,10 @@ TokenPlan token_plan(int M, int N, int k_blocks, bool w4, int num_sms, bool allo
             }
         }
     }
+    // (What the pair form gives where it is taken beside the channel-major ones: int4 layers of 130 to 560 channels on 5000 to
+    // 16000 rows, in which a third column of 256 channels would be mostly empty or one wave just too small, 1.09 times the
+    // speed of the next best form over 14 layers, 0.95 to 1.23; split reductions, int4 from 130 k-blocks 1.15 times over 14,
+    // 0.96 to 1.34, int8 from 90 k-blocks 1.42 times over 26, 1.0 to 1.88.)
     // single-CTA kernels: 128 x 128 tiles (128 x 256 for wide int8 layers), persistent once the tiles cover the
     // SMs, else one tile per CTA with the reduction split over a cluster
     const double c = w4 ? 580.0 : 420.0;
@@ -1337,6 +1341,11 @@ int fq_tile(int M, int N, int k_blocks, int num_sms)
 // repeats too, up to some 8000 rows (8192 x 320 x 640 9.6 and 9.1); for int8 not there (4096 x 640 x 640 8.1 and 7.5).
 // Layers left to the forms with tokens on the rows: int8 of four or five k-blocks up to 3072 rows (2048 x 640 x 640 6.4 and
 // 6.9, 3000 7.1 and 7.3).
+// How far the rule carries, on 112 other layers (1024 to 16384 rows, 64 to 1000 channels in eights, 64 to 640 long): where it
+// says two kernels, they took 0.94 of the fused kernel's time (0.70 to 1.20; the worst below 140 channels on 4500 rows and
+// more), where it says the fused one, 1.21 of it (0.97 to 1.61).  It does not look at rows of Y that are no multiple of 16
+// bytes (N % 8 != 0), where the fused kernel cannot store by TMA and takes 2 to 2.6 times the channel-major forms' time (5040 x
+// 388 x 96 W8 15.8 us and 6.7).
 bool two_kernels_win(const ChanPlan& chan, int M, int k_blocks, bool w4)
 {
     if (chan.tokens == 0) return k_blocks >= 4 && M <= 3072;

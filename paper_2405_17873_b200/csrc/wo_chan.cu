@@ -10,10 +10,10 @@
 //     results do not change from run to run;
 //   * there is no quantization pass: the activations are the layer's input as it is.
 //
-// Measured on B200, before and now: W4 16 x 10240 x 1280 7.4 -> 5.3 us, 17 x 1280 x 1280 10.2 -> 4.2, 128 x 1280 x 5120 38.4 ->
-// 13.7, 256 x 1280 x 1280 8.4 -> 5.3, 1024 x 1280 x 1280 10.1 -> 6.8, 1024 x 1280 x 5120 23.7 -> 15.7, 3x3 convolution 48 x 48
-// x 640 -> 640 28.9 -> 17.6; W3 the first two 7.5 -> 5.6, 10.4 -> 4.3; W8
-// 16 x 10240 x 1280 7.4 -> 5.0, 17 x 1280 x 1280 10.2 -> 4.1, 1024 x 1280 x 1280 10.9 -> 6.6, 1024 x 1280 x 5120 25.0 -> 15.9.  A long reduction takes 300 cycles per k-block of 64:
+// Measured on B200, before and now: W4 16 x 10240 x 1280 7.4 -> 5.0 us, 17 x 1280 x 1280 10.2 -> 4.2, 128 x 1280 x 5120 38.4 ->
+// 13.5, 256 x 1280 x 1280 8.4 -> 5.2, 1024 x 1280 x 1280 10.1 -> 6.3, 1024 x 1280 x 5120 23.7 -> 15.2, 3x3 convolution 48 x 48
+// x 640 -> 640 28.9 -> 17.6; W3 the first two 7.5 -> 5.2, 10.4 -> 4.3; W8 16 x 10240 x 1280 7.4 -> 5.0, 17 x 1280 x 1280 10.2
+// -> 4.1, 1024 x 1280 x 1280 10.9 -> 6.4, 1024 x 1280 x 5120 25.0 -> 15.  A long reduction takes 300 cycles per k-block of 64:
 // the expansion (three groups of four warps, some 1700 cycles for a pair of k-blocks; 3 bits more) and the rings' latency.
 #include <algorithm>
 
@@ -406,7 +406,7 @@ bool chan_path_ok(const Params& p, int amode, const void* packed, int w_bits)
 // fitted to the same layers:
 //   * up to 16 rows, a linear layer: the kernels of wo_gemm.cu, which split the reduction inside a CTA and win wherever it is
 //     long or the rows are eight at most and the weights few (16 x 1280 x 5120 W4 5.6 us against 13.0), and lose by up to half
-//     on many channels (16 x 10240 x 1280 7.4 and 5.3);
+//     on many channels (16 x 10240 x 1280 7.4 and 5.0);
 //   * 17 to 255 rows: nothing comes near (17 x 1280 x 1280 W4 10.2 us and 4.2, 128 x 1280 x 5120 38 and 13.7), so tiles of
 //     more than one wave are taken too;
 //   * from 256 rows, with a workspace: the pair form, whose split reductions win on the longest.
