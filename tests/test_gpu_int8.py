@@ -307,3 +307,29 @@ def test_pack_then_capture_on_one_stream():
     _, y_ref = orc.linear_a8(X, codes, s_ref, orc.act_scale(orc.act_absmax(X), 8), None)
     assert_close(host(captured), y_ref)
     assert np.array_equal(host(captured).view(np.uint16), host(eager).view(np.uint16))
+
+
+def test_pack_and_layer_in_one_graph():
+    """Both captured, replayed on weights that change from replay to replay."""
+    M, K, N = 256, 1280, 640
+    X = synth.normal_f16((M, K), 1.0, seed=77)
+    Ws = [synth.normal_f16((N, K), 0.02 * (1 + r), seed=790 + r) for r in range(3)]
+    Xd, Wd = dev(X), dev(Ws[0])
+    sx, st, ws = mixdq.act_scale(Xd), status_word(), workspace_for(M, N, K, 4)
+    s = torch.zeros(N, dtype=torch.float32, device="cuda")
+    packed = torch.zeros(mixdq.packed_bytes(N, K, 4), dtype=torch.uint8, device="cuda")
+    y = torch.zeros((M, N), dtype=torch.float16, device="cuda")
+    torch.cuda.synchronize()
+    stream, graph = torch.cuda.Stream(), torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph, stream=stream):
+        mixdq.weight_minmax_params(Wd, 4, True, scale_out=s)
+        mixdq.pack_weights(Wd, 4, s, out=packed)
+        mixdq.linear(Xd, packed, N, 4, s, None, 8, sx, None, workspace=ws, status=st, out=y)
+    for W in Ws:
+        Wd.copy_(dev(W))
+        graph.replay()
+        torch.cuda.synchronize()
+        s_ref, _, codes = oracle_weights(W, 4, True)
+        _, y_ref = orc.linear_a8(X, codes, s_ref, orc.act_scale(orc.act_absmax(X), 8), None)
+        assert_close(host(y), y_ref)
+    assert int(host(st)[0]) == 0
